@@ -32,7 +32,6 @@ using namespace sm100;
 constexpr int BLOCK_M = 128;
 constexpr int kRowBytes = 128;         // one swizzle row of K per stage: 64 halves or 128 int8
 constexpr int kUmmaBytes = 32;         // K bytes one tcgen05.mma contracts (16 halves / 32 int8)
-constexpr int kStages = 4;
 constexpr int kThreads = 320;          // producer, MMA issuer, 2 x 4 epilogue warps
 
 template <int BLOCK_N>
@@ -40,6 +39,9 @@ struct SmemLayout {
   static constexpr int kABytes = BLOCK_M * kRowBytes;
   static constexpr int kBBytes = BLOCK_N * kRowBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
+  // What fits: 4, 6 or 8 stages of 48, 32 or 24 KB.  The narrow blocks run where a CTA has one or
+  // two items, and then nearly all of an item's operands are in flight at once.
+  static constexpr int kStages = 196608 / kStageBytes;
   static constexpr int kBarrierOffset = kStages * kStageBytes;
   static constexpr int kTotal = kBarrierOffset + 256 + 1024;     // barriers + alignment slack
 };
@@ -57,9 +59,10 @@ template <int BLOCK_N, bool I8, bool PROF = false>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmU,
                     float* __restrict__ Mo, int nfreq, int pc, int pc_pad, int C, int K,
-                    int* __restrict__ status, const uint8_t* __restrict__ Vdrop, int f_major, int keep_pct,
+                    int* __restrict__ status, const uint8_t* __restrict__ Vdrop, int f_major, int spread, int keep_pct,
                     unsigned long long* __restrict__ prof) {
   using L = SmemLayout<BLOCK_N>;
+  constexpr int kStages = L::kStages;
   constexpr int BLOCK_K = I8 ? kRowBytes : kRowBytes / 2;   // elements of K per stage
   constexpr uint32_t kTmemCols = 2 * BLOCK_N;       // two accumulators; 128, 256 or 512
   extern __shared__ uint8_t smem_raw[];
@@ -82,15 +85,23 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
   // transform reads first.  With f_major the frequency is outermost instead (see the launcher).
   // Pair i of this CTA is pair blockIdx.x + i * gridDim.x; the CTA runs
   // the pair's filter blocks one after the other (items), so that it is the only reader of the
-  // pair's rows of V and knows when they have been read for the last time.
-  const long long num_pairs = (long long)nfreq * num_pb;
-  const uint32_t pairs_local = num_pairs > blockIdx.x ? (uint32_t)((num_pairs - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0u;
-  const uint32_t n_local = pairs_local * (uint32_t)num_kb;
+  // pair's rows of V and knows when they have been read for the last time.  With `spread` the
+  // filter blocks of a pair are dealt out to different CTAs instead (see the launcher).
+  const long long num_units = (long long)nfreq * num_pb * (spread ? num_kb : 1);
+  const uint32_t units_local = num_units > blockIdx.x ? (uint32_t)((num_units - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0u;
+  const uint32_t n_local = spread ? units_local : units_local * (uint32_t)num_kb;
   auto item_of = [&](uint32_t local, int& pb, int& f, int& kb) {
-    const unsigned pair = blockIdx.x + (local / (unsigned)num_kb) * gridDim.x;
+    unsigned pair;
+    if (spread) {
+      const unsigned unit = blockIdx.x + local * gridDim.x;
+      pair = unit / (unsigned)num_kb;
+      kb = (int)(unit % (unsigned)num_kb);
+    } else {
+      pair = blockIdx.x + (local / (unsigned)num_kb) * gridDim.x;
+      kb = (int)(local % (unsigned)num_kb);
+    }
     if (f_major) { f = (int)(pair / (unsigned)num_pb); pb = num_pb - 1 - (int)(pair % (unsigned)num_pb); }
     else { pb = num_pb - 1 - (int)(pair / (unsigned)nfreq); f = (int)(pair % (unsigned)nfreq); }
-    kb = (int)(local % (unsigned)num_kb);
   };
 
   if (threadIdx.x == 0) {
@@ -113,11 +124,23 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
   bool timed_out = false;
   // everything above touched no global memory: it may overlap the tail of the preceding kernel
   pdl_launch_dependents();
-  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer
     WaitClock<PROF> w_empty, total;
+    // The first stages' pieces of U do not wait for the input transform, which lets this kernel
+    // start only once everything before the transform itself has completed (it releases its
+    // dependents after its own wait): U is final by then.
+    const int early = n_local > 0 ? (num_ks < kStages ? num_ks : kStages) : 0;
+    if (lane == 0 && early > 0) {
+      int pb, f, kb;
+      item_of(0, pb, f, kb);
+      for (int ks = 0; ks < early; ++ks) {
+        mbar_expect_tx(&full_bar[ks], L::kStageBytes);
+        tma_load_3d(smem + ks * L::kStageBytes + L::kABytes, &tmU, &full_bar[ks], ks * BLOCK_K, kb * BLOCK_N, f);
+      }
+    }
+    pdl_wait();
     total.start();
     uint32_t stage = 0, phase = 0;
     for (uint32_t local = 0; local < n_local && !timed_out; ++local) {
@@ -130,9 +153,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
         if (lane == 0) {
           uint8_t* sa = smem + stage * L::kStageBytes;
           uint8_t* sb = sa + L::kABytes;
-          mbar_expect_tx(&full_bar[stage], L::kStageBytes);
+          if (local > 0 || ks >= early) {
+            mbar_expect_tx(&full_bar[stage], L::kStageBytes);
+            tma_load_3d(sb, &tmU, &full_bar[stage], ks * BLOCK_K, kb * BLOCK_N, f);
+          }
           tma_load_3d(sa, &tmV, &full_bar[stage], ks * BLOCK_K, pb * BLOCK_M, f);
-          tma_load_3d(sb, &tmU, &full_bar[stage], ks * BLOCK_K, kb * BLOCK_N, f);
         }
         __syncwarp();
         if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -146,6 +171,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     // ---------------- MMA issuer
     constexpr uint32_t idesc = I8 ? umma_idesc_i8(BLOCK_M, BLOCK_N) : umma_idesc_f16(BLOCK_M, BLOCK_N);
     WaitClock<PROF> w_acc, w_ops, total;
+    pdl_wait();
     total.start();
     uint32_t stage = 0, phase = 0;
     for (uint32_t local = 0; local < n_local && !timed_out; ++local) {
@@ -203,13 +229,16 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     }
   } else {
     // ---------------- epilogue (warps 2..9); a warp may only read TMEM lanes 32*(warp%4)..+31.
-    // Rows >= pc of the last row block are zeros (the TMA loads of V fill them) and land in the
-    // padding rows pc..pc_pad-1 of M.
+    // Rows >= pc of the last row block are zeros (the TMA loads of V fill them); the output
+    // transform reads whole groups of 8 rows, so those up to the next multiple of 8 are stored and
+    // the rest of the block is not.
     const int quad = warp & 3;
     const int half = (warp - 2) >> 2;                    // which half of the BLOCK_N columns
     constexpr int HALF_N = BLOCK_N / 2;
     const int k4 = K >> 2;
+    const int live_rows = (pc + 7) & ~7;
     WaitClock<PROF> w_full, total;
+    pdl_wait();
     total.start();
     for (uint32_t local = 0; local < n_local && !timed_out; ++local) {
       int pb, f, kb;
@@ -228,11 +257,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
       else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
       const int row = pb * BLOCK_M + quad * 32 + lane;
       const int col_base = kb * BLOCK_N + half * HALF_N;
-      const int k_left = K - col_base;
+      const int k_left = row < live_rows ? K - col_base : 0;
+      const int warp_k_left = row - lane < live_rows ? K - col_base : 0;       // the same for all lanes
       float* dst = Mo + (((size_t)f * k4 + (size_t)(col_base >> 2)) * pc_pad + row) * 4;
       const size_t q_stride = (size_t)pc_pad * 4;        // floats between consecutive filter quads
 #pragma unroll 1
-      for (int cb = 0; cb < HALF_N && cb < k_left; cb += 32) {
+      for (int cb = 0; cb < HALF_N && cb < warp_k_left; cb += 32) {
         uint32_t r[32];
         tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + acc * BLOCK_N + half * HALF_N + cb, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -280,6 +310,30 @@ bool make_map_3d(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+long long item_rounds(long long items, int sms) { return (items + sms - 1) / sms; }
+
+// Width of the filter blocks.  A narrow block loads V more often, so a problem with many rounds of
+// items per SM takes 256; one with few pairs (frequency, row block) needs the narrow ones, and the
+// blocks of a pair on different CTAs, to reach all SMs.  The estimate is rounds x bytes per stage
+// (rows of V that exist + columns of U), plus a term for what an item costs by itself.
+// Measured, whole layer, always-256-and-whole against this rule: one image 14 x 14, 512 -> 512,
+// F(4,3) (36 pairs) 17.9 -> 11.6 us; 28 x 28 18.4 -> 12.3 us; 32 images of 14 x 14, F(6,3) (192 pairs)
+// 41.9 -> 32.1 us; 45 x 61, 7 images, 200 -> 328 channels 45.6 -> 40.5 us; layers of ten rounds and more
+// keep 256 (56 x 56, 32 images, 256 -> 256: 120 us either way).
+int pick_block_n(long long pairs, int pc, int K, int sms) {
+  const int rows = pc < BLOCK_M ? pc : BLOCK_M;
+  int best = 64;
+  long long best_cost = -1;
+  for (int bn = 64; bn <= 256; bn *= 2) {
+    if (bn > 64 && bn / 2 >= K) break;
+    const long long num_kb = (K + bn - 1) / bn;
+    const long long whole = item_rounds(pairs, sms) * num_kb, dealt = item_rounds(pairs * num_kb, sms);
+    const long long cost = (whole < dealt ? whole : dealt) * (rows + bn + 32);
+    if (best_cost < 0 || cost <= best_cost) { best = bn; best_cost = cost; }
+  }
+  return best;
+}
+
 template <int BLOCK_N, bool I8>
 int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int nfreq, int pc, int pc_pad, int C, int K,
              int* status, cudaStream_t stream, unsigned long long* prof = nullptr) {
@@ -293,7 +347,10 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
       !make_map_3d(&tmU, dt, esize, U, C, K, (long long)K * C, nfreq, BLOCK_K, BLOCK_N))
     return (int)cudaErrorUnknown;
   const long long pairs = (long long)nfreq * ((pc + BLOCK_M - 1) / BLOCK_M);
-  const int grid = (int)(pairs < sms ? pairs : sms);
+  const int num_kb = (K + BLOCK_N - 1) / BLOCK_N;
+  const bool spread = item_rounds(pairs * num_kb, sms) < item_rounds(pairs, sms) * num_kb;
+  const long long units = spread ? pairs * num_kb : pairs;
+  const int grid = (int)(units < sms ? units : sms);
   // Work order.  Row-block-major re-streams all of U once per row block; that is free while U
   // stays in the L2 (8 MB at C = K = 256) and costs device-memory reads once it does not (52 MB at
   // C = K = 512 with 100 frequencies: 164 MB read per launch).  Frequency-major lets the CTAs that
@@ -308,7 +365,8 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
   int keep_pct = f_major ? 100 : (int)(100.0 * (2.0 / 3.0) * l2_bytes / m_bytes);
   if (keep_pct > 100) keep_pct = 100;
   // V may be dropped from the L2 after its last read when the pieces read are whole 128-byte lines
-  const bool drop = ((size_t)C * esize) % kRowBytes == 0 && (reinterpret_cast<uintptr_t>(V) % kRowBytes) == 0;
+  // by the CTA that reads them last, which is known only where a pair stays with one CTA
+  const bool drop = !spread && ((size_t)C * esize) % kRowBytes == 0 && (reinterpret_cast<uintptr_t>(V) % kRowBytes) == 0;
   const uint8_t* vdrop = drop ? (const uint8_t*)V : (const uint8_t*)nullptr;
   // the wait-profiling variant exists for the half product with 256-wide filter blocks only
   if constexpr (BLOCK_N == 256 && !I8) {
@@ -317,11 +375,11 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
       // CTAs beyond this launch's grid must read as "did not run"
       if (cudaError_t e = cudaMemsetAsync(prof, 0, sizeof(unsigned long long) * 8 * sms, stream); e != cudaSuccess) return (int)e;
       return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8, true>, grid, kThreads, L::kTotal, stream, tmV, tmU, M,
-                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, keep_pct, prof);
+                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, prof);
     }
   }
   return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8>, grid, kThreads, L::kTotal, stream, tmV, tmU, M, nfreq,
-                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, keep_pct, (unsigned long long*)nullptr);
+                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, (unsigned long long*)nullptr);
 }
 
 }  // namespace
@@ -330,8 +388,9 @@ int launch_gemm_tcgen05(const nova_plan* plan, const void* V, const void* U, flo
                         int pc_pad, int C, int K, int* status_dev, void* stream, unsigned long long* prof) {
   cudaStream_t s = (cudaStream_t)stream;
   const int sms = plan->sm_count;
-  if (K > 128) return launch_n<256, false>(sms, plan->l2_bytes, V, U, M, nfreq, pc, pc_pad, C, K, status_dev, s, prof);
-  if (K > 64) return launch_n<128, false>(sms, plan->l2_bytes, V, U, M, nfreq, pc, pc_pad, C, K, status_dev, s);
+  const int bn = prof ? 256 : pick_block_n((long long)nfreq * ((pc + BLOCK_M - 1) / BLOCK_M), pc, K, sms);
+  if (bn == 256) return launch_n<256, false>(sms, plan->l2_bytes, V, U, M, nfreq, pc, pc_pad, C, K, status_dev, s, prof);
+  if (bn == 128) return launch_n<128, false>(sms, plan->l2_bytes, V, U, M, nfreq, pc, pc_pad, C, K, status_dev, s);
   return launch_n<64, false>(sms, plan->l2_bytes, V, U, M, nfreq, pc, pc_pad, C, K, status_dev, s);
 }
 
@@ -342,8 +401,9 @@ int launch_gemm_tcgen05_i8(const nova_plan* plan, const void* V, const void* U, 
   cudaStream_t s = (cudaStream_t)stream;
   const int sms = plan->sm_count;
   float* Mf = reinterpret_cast<float*>(M);            // the epilogue moves 32-bit words
-  if (K > 128) return launch_n<256, true>(sms, plan->l2_bytes, V, U, Mf, nfreq, pc, pc_pad, C, K, status_dev, s);
-  if (K > 64) return launch_n<128, true>(sms, plan->l2_bytes, V, U, Mf, nfreq, pc, pc_pad, C, K, status_dev, s);
+  const int bn = pick_block_n((long long)nfreq * ((pc + BLOCK_M - 1) / BLOCK_M), pc, K, sms);
+  if (bn == 256) return launch_n<256, true>(sms, plan->l2_bytes, V, U, Mf, nfreq, pc, pc_pad, C, K, status_dev, s);
+  if (bn == 128) return launch_n<128, true>(sms, plan->l2_bytes, V, U, Mf, nfreq, pc, pc_pad, C, K, status_dev, s);
   return launch_n<64, true>(sms, plan->l2_bytes, V, U, Mf, nfreq, pc, pc_pad, C, K, status_dev, s);
 }
 

@@ -157,8 +157,10 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     for (int b = 0; b < 2 * Cfg::KA; ++b)
       tma_load_2d(kron + (size_t)b * Cfg::NFP * 128, &tmKron, kron_bar, 0, b * Cfg::NFP);
   }
-  pdl_launch_dependents();
+  // The product kernel may be scheduled from here on; it relies on everything before this kernel
+  // having completed by then (it fetches U before its own wait), hence after the wait.
   pdl_wait();
+  pdl_launch_dependents();
 
   if (warp < kProdWarps) {
     // ---------------- TMA producers

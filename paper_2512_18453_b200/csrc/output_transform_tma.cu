@@ -64,7 +64,10 @@ output_transform_tma_kernel(const __grid_constant__ CUtensorMap tmM, const __gri
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int KG = (K + kUnitK - 1) / kUnitK;           // filter groups of 16 * VEC
-  const int TG = pc_pad >> 3;                         // tile groups of 8 (pc_pad is a multiple of 128)
+  // Tile groups of 8 that hold a tile, not all of pc_pad: the last chunk of a layer that needs two
+  // (224 x 224, 64 -> 64, 32 images, F(6,3)) holds 2 560 tiles of a stride of 43 648, and its padding cost
+  // this kernel 110 of 261 us.
+  const int TG = (pc + 7) >> 3;
   // Unit i of this CTA is unit blockIdx.x + i * gridDim.x: ascending tiles chip-wide, i.e. the
   // rows of M the product kernel wrote last (still in L2) first.
   const unsigned num_units = (unsigned)TG * (unsigned)KG;
@@ -162,7 +165,7 @@ int launch_one(const nova_plan* plan, const Geom& g, const CUtensorMap& tmM, con
                int pc_pad, int relu, const float* scale_U, const float* scale_V, cudaStream_t stream) {
   using Cfg = OtCfg<M, VEC, R>;
   if (cudaError_t e = allow_dynamic_smem(output_transform_tma_kernel<M, T, SYM, VEC, QUANT, R>, Cfg::kTotal); e != cudaSuccess) return (int)e;
-  const long long units = (long long)(pc_pad / 8) * ((g.K + 16 * VEC - 1) / (16 * VEC));
+  const long long units = (long long)((pc + 7) / 8) * ((g.K + 16 * VEC - 1) / (16 * VEC));
   const int grid = (int)(units < plan->sm_count ? units : plan->sm_count);
   return (int)launch_overlapped(output_transform_tma_kernel<M, T, SYM, VEC, QUANT, R>, grid, kOtThreads, Cfg::kTotal,
                                 stream, tmM, plan->kcoefs, (T*)y, g.H, g.W, g.K, g.Th, g.Tw, p0, pc, pc_pad, relu,

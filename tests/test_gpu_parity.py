@@ -326,6 +326,25 @@ def test_ragged_last_row_block_after_full_blocks():
         assert d.max() <= 4 * 2.0 ** -10 * np.abs(yb.astype(np.float32)).max()
 
 
+@pytest.mark.parametrize("kind,m,shape", [
+    ("nova", 4, (1, 14, 14, 64, 512)),      # 16 tiles, 36 pairs: 128-wide filter blocks dealt out to different CTAs
+    ("nova", 4, (1, 9, 9, 64, 64)),         # 9 live rows of 128: stores stop at row 16
+    ("std", 2, (1, 17, 15, 72, 520)),       # 72 tiles, 16 pairs: 64-wide blocks, the last one 8 filters wide
+    ("nova", 6, (3, 56, 56, 64, 264)),      # 300 tiles: ragged third row block, 264 = 256 + 8 filters
+    ("nova", 8, (2, 65, 33, 128, 136)),     # 90 tiles, 100 pairs
+    ("std", 2, (1, 64, 64, 64, 200))])      # 1024 tiles, 8 full row blocks
+def test_product_work_splits_match_the_cuda_core_product(kind, m, shape):
+    # every way the product kernel deals out its filter blocks, against the CUDA-core product on the same V:
+    # the same operands summed in another order, so the bound of test_tcgen05_and_simt_products_agree
+    N, H, W, C, K = shape
+    x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=480 + m)
+    pts = point_set(kind, m)
+    ya, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, nv.GEMM_TCGEN05)
+    yb, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, nv.GEMM_SIMT)
+    assert np.isfinite(ya.astype(np.float32)).all()
+    assert conv.rel_l2(ya, yb) < 0.05 * conv.rel_l2(yb, conv.direct_conv_fp64(x, g)) + 2.0 ** -13
+
+
 def test_gpu_is_close_to_emulation_elementwise():
     x, g = make_conv_inputs(2, 24, 24, 64, 64, "fp16", True, True, seed=410)
     pts = point_set("nova", 4)
