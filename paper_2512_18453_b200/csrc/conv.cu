@@ -69,6 +69,10 @@ bool use_fused_small_c(const nova_plan* p, const Geom& g, int flags) {
   return (flags & forcing) == 0 && fused_small_c_applies(p, g);
 }
 
+bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
+  return fused_fp32_applies(p) || use_fused_small_c(p, g, flags);
+}
+
 bool use_tcgen05(const nova_plan* p, int flags) {
   if (p->mode == NOVA_FP32) return false;
   return (flags & NOVA_GEMM_SIMT) == 0;
@@ -119,7 +123,7 @@ extern "C" int nova_conv2d_launch_count(const nova_plan* p, int N, int H, int W,
   Geom g = make_geom(p, N, H, W, C, K);
   Chunking c;
   if (!choose_chunking(p, g, workspace_bytes, &c)) return NOVA_ERR_WORKSPACE;
-  if (use_fused_small_c(p, g, flags)) return 1;
+  if (one_kernel(p, g, flags)) return 1;
   return 3 * c.chunks;
 }
 
@@ -143,10 +147,15 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
   Geom g = make_geom(p, N, H, W, C, K);
   Chunking c;
   if (!choose_chunking(p, g, ws_bytes, &c)) return NOVA_ERR_WORKSPACE;
-  if (use_fused_small_c(p, g, flags)) {
+  if (one_kernel(p, g, flags)) {
     // steps 2-4 in one kernel, V and M kept on the SM: the workspace is not touched
     if (ev) cudaEventRecord(ev[0], (cudaStream_t)stream);
-    if (launch_fused_small_c(p, g, x, U, y, (flags & NOVA_RELU) ? 1 : 0, stream)) return NOVA_ERR_CUDA;
+    const int relu = (flags & NOVA_RELU) ? 1 : 0;
+    if (int e = p->mode == NOVA_FP32 ? launch_fused_fp32(p, g, x, U, y, relu, stream)
+                                     : launch_fused_small_c(p, g, x, U, y, relu, stream)) {
+      g_last_cuda_error = e;
+      return NOVA_ERR_CUDA;
+    }
     if (ev) cudaEventRecord(ev[1], (cudaStream_t)stream);
     return NOVA_OK;
   }

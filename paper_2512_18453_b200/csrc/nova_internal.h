@@ -19,6 +19,11 @@ struct Coefs {
   float AT[kMaxM][kMaxN];
   float G[kMaxN][kMaxR];
 };
+// B^T and A^T once more for kernels that carry their sums in double: the same rounded values.
+struct CoefsD {
+  double BT[kMaxN][kMaxN];
+  double AT[kMaxM][kMaxN];
+};
 
 }  // namespace nova
 
@@ -41,6 +46,7 @@ struct nova_plan {
   // paths rely on (checked entry by entry), and symmetric = 1; otherwise the
   // order is the caller's and the kernels evaluate dense products.
   nova::Coefs kcoefs;
+  nova::CoefsD kcoefs_d;                  // B^T and A^T of kcoefs
   int perm[nova::kMaxN];
   int symmetric;
   void* kron_dev;                         // device table of the tensor-core input transform (may be null)
@@ -110,6 +116,9 @@ int launch_gemm_tcgen05(const nova_plan* plan, const void* V, const void* U, flo
 bool fused_small_c_applies(const nova_plan* plan, const Geom& g);
 int launch_fused_small_c(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu,
                          void* stream);
+// The same for the fp32 mode (tiles of up to 8 points)
+bool fused_fp32_applies(const nova_plan* plan);
+int launch_fused_fp32(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, void* stream);
 int launch_maxpool2x2(const void* x, void* y, int N, int H, int W, int C, int mode, void* stream);
 
 }  // namespace nova

@@ -391,6 +391,10 @@ int create_impl(int m, int r, const nova_rat* points, int n, const nova_rat* sca
       for (int kk = 0; kk < r; ++kk) k.G[p][kk] = pl->coefs.G[pl->perm[p]][kk];
       for (int j = 0; j < n; ++j) k.BT[p][j] = pl->coefs.BT[pl->perm[p]][j];
     }
+    for (int p = 0; p < n; ++p)
+      for (int j = 0; j < n; ++j) pl->kcoefs_d.BT[p][j] = (double)k.BT[p][j];
+    for (int i = 0; i < m; ++i)
+      for (int p = 0; p < n; ++p) pl->kcoefs_d.AT[i][p] = (double)k.AT[i][p];
     // The SYM kernel paths skip the structural zeros and share even/odd partial sums of a
     // +-pair; they are used only if the rounded tables have exactly that structure.
     if (sym && cnt == n) {

@@ -40,6 +40,16 @@ __device__ __forceinline__ float vadd(float a, float b) { return a + b; }
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float vsub(float a, float b) { return a - b; }
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+// The same for double sums: one value, or two filters' values side by side.
+struct Dbl2 { double x, y; };
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ Dbl2 vmul(double a, Dbl2 b) { return {a * b.x, a * b.y}; }
+__device__ __forceinline__ Dbl2 vfma(double a, Dbl2 b, Dbl2 c) { return {fma(a, b.x, c.x), fma(a, b.y, c.y)}; }
+__device__ __forceinline__ Dbl2 vadd(Dbl2 a, Dbl2 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ Dbl2 vsub(Dbl2 a, Dbl2 b) { return {a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ float vrelu(float v) { return v < 0.f ? 0.f : v; }
 __device__ __forceinline__ float2 vrelu(float2 v) { return make_float2(v.x < 0.f ? 0.f : v.x, v.y < 0.f ? 0.f : v.y); }
 __device__ __forceinline__ void vstore(__half* p, float v) { *p = __float2half_rn(v); }
@@ -59,48 +69,48 @@ __device__ __forceinline__ void vstore(float* p, float2 v) { st2(p, v); }
 // a +-pair shared; SYM = false is the dense product.
 
 // Two rows of B^T applied to one n-vector.  Group g = 0 gives rows (0, n-1); g >= 1 gives the
-// pair (2g-1, 2g).
-template <int N, bool SYM, int G>
-__device__ __forceinline__ void bt_two_rows(const Coefs& cf, const float2 (&in)[N], float2& oa, float2& ob) {
+// pair (2g-1, 2g).  V: float2, or a double type with the tables in double (CF).
+template <int N, bool SYM, int G, typename CF, typename V>
+__device__ __forceinline__ void bt_two_rows(const CF& cf, const V (&in)[N], V& oa, V& ob) {
   constexpr int RA = (G == 0) ? 0 : 2 * G - 1;
   constexpr int RB = (G == 0) ? N - 1 : 2 * G;
   if constexpr (!SYM) {
-    float2 a = mul2(cf.BT[RA][0], in[0]), b = mul2(cf.BT[RB][0], in[0]);
+    V a = vmul(cf.BT[RA][0], in[0]), b = vmul(cf.BT[RB][0], in[0]);
 #pragma unroll
     for (int j = 1; j < N; ++j) {
-      a = fma2(cf.BT[RA][j], in[j], a);
-      b = fma2(cf.BT[RB][j], in[j], b);
+      a = vfma(cf.BT[RA][j], in[j], a);
+      b = vfma(cf.BT[RB][j], in[j], b);
     }
     oa = a; ob = b;
   } else if constexpr (G == 0) {
-    float2 e = mul2(cf.BT[0][0], in[0]);
+    V e = vmul(cf.BT[0][0], in[0]);
 #pragma unroll
-    for (int j = 2; j < N; j += 2) e = fma2(cf.BT[0][j], in[j], e);
-    float2 o = mul2(cf.BT[N - 1][1], in[1]);
+    for (int j = 2; j < N; j += 2) e = vfma(cf.BT[0][j], in[j], e);
+    V o = vmul(cf.BT[N - 1][1], in[1]);
 #pragma unroll
-    for (int j = 3; j < N; j += 2) o = fma2(cf.BT[N - 1][j], in[j], o);
+    for (int j = 3; j < N; j += 2) o = vfma(cf.BT[N - 1][j], in[j], o);
     oa = e; ob = o;
   } else {
-    float2 e = mul2(cf.BT[RA][0], in[0]);
+    V e = vmul(cf.BT[RA][0], in[0]);
 #pragma unroll
-    for (int j = 2; j < N; j += 2) e = fma2(cf.BT[RA][j], in[j], e);
-    float2 o = mul2(cf.BT[RA][1], in[1]);
+    for (int j = 2; j < N; j += 2) e = vfma(cf.BT[RA][j], in[j], e);
+    V o = vmul(cf.BT[RA][1], in[1]);
 #pragma unroll
-    for (int j = 3; j < N - 1; j += 2) o = fma2(cf.BT[RA][j], in[j], o);
-    oa = make_float2(e.x + o.x, e.y + o.y);
-    ob = make_float2(e.x - o.x, e.y - o.y);
+    for (int j = 3; j < N - 1; j += 2) o = vfma(cf.BT[RA][j], in[j], o);
+    oa = vadd(e, o);
+    ob = vsub(e, o);
   }
 }
 
 // All n rows of B^T applied to one n-vector.
-template <int N, bool SYM>
-__device__ __forceinline__ void bt_all_rows(const Coefs& cf, const float2 (&in)[N], float2 (&out)[N]) {
+template <int N, bool SYM, typename CF, typename V>
+__device__ __forceinline__ void bt_all_rows(const CF& cf, const V (&in)[N], V (&out)[N]) {
   if constexpr (!SYM) {
 #pragma unroll
     for (int p = 0; p < N; ++p) {
-      float2 s = mul2(cf.BT[p][0], in[0]);
+      V s = vmul(cf.BT[p][0], in[0]);
 #pragma unroll
-      for (int j = 1; j < N; ++j) s = fma2(cf.BT[p][j], in[j], s);
+      for (int j = 1; j < N; ++j) s = vfma(cf.BT[p][j], in[j], s);
       out[p] = s;
     }
   } else {
@@ -113,8 +123,8 @@ __device__ __forceinline__ void bt_all_rows(const Coefs& cf, const float2 (&in)[
 }
 
 // z[i] = sum_p A^T[i][p] * in[p], i < M.  N = M + r - 1 points: 0, (N - 2) / 2 pairs +-a, infinity.
-template <int M, bool SYM, typename V, int N = M + 2>
-__device__ __forceinline__ void at_apply(const Coefs& cf, const V (&in)[N], V (&z)[M]) {
+template <int M, bool SYM, typename V, int N = M + 2, typename CF = Coefs>
+__device__ __forceinline__ void at_apply(const CF& cf, const V (&in)[N], V (&z)[M]) {
   constexpr int NP = (N - 2) / 2;
   if constexpr (!SYM) {
 #pragma unroll

@@ -112,6 +112,32 @@ def test_fp32_mode_matches_direct(kind, m, shape):
     np.testing.assert_allclose(y, y1, rtol=0, atol=tol * scale)
 
 
+@pytest.mark.parametrize("m,key,r,shape", [
+    (2, ("std", 2), 3, (1, 5, 7, 8, 520)),       # one block of tiles, ragged last filter block
+    (4, ("nova", 4), 3, (1, 14, 14, 256, 24)),   # few blocks, many channels: the channels of a block split over a cluster
+    (4, ("asym", 4), 3, (3, 33, 18, 40, 40)),    # 135 tiles, a chunk of 16 channels half outside the tensor
+    (6, ("half", 6), 3, (2, 50, 50, 64, 72)),    # several blocks per CTA
+    (6, ("asym", 6), 3, (1, 12, 12, 136, 16)),   # dense transforms, split
+    (4, ("half", 6), 5, (2, 23, 19, 24, 64)),
+    (2, ("nova", 4), 5, (1, 40, 41, 16, 136))])
+def test_fp32_one_kernel_blocks_match_direct(m, key, r, shape):
+    # edges of the tile, filter and channel blocks of the one-kernel fp32 path; its sums are carried in double and
+    # only V and y are rounded, so the bounds of test_fp32_mode_matches_direct hold with room
+    N, H, W, C, K = shape
+    pts = point_set(*key)
+    x, g = make_conv_inputs(N, H, W, C, K, "fp32", True, True, seed=130 + m, r=r)
+    plan = nv.Plan(m, pts, nv.FP32, r=r)
+    assert plan.launch_count(N, H, W, C, K, plan.workspace_bytes(N, H, W, C, K)) == 1
+    xd, gd = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda()
+    y = torch.full((N, H, W, K), float("nan"), dtype=torch.float32, device="cuda")
+    plan.conv2d(xd, plan.filter_transform(gd), y=y, flags=nv.RELU)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0
+    y1 = np.maximum(conv.direct_conv_fp64(x, g), 0.0)
+    e_emu = conv.rel_l2(conv.winograd_conv_emulated(x, g, m, pts, "fp32", apply_relu=True), y1)
+    assert conv.rel_l2(y.cpu().numpy(), y1) <= 1.5 * e_emu + 1e-7
+
+
 def test_cfg1_fp32_standard_f2():
     c = CONFIGS["cfg1"]
     x, g = make_conv_inputs(c.N, c.H, c.W, c.C, c.K, c.dtype, c.relu_inputs, c.he_weights, c.seed)
