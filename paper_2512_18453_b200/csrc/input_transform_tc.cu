@@ -87,15 +87,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
       : "memory");
 }
 
-// QMODE 0: V rounded to half.  QMODE 1: nothing is stored; the largest |V| is reduced into *qslot
-// (as float bits; first pass of the int8 pipeline's data-derived scale).  QMODE 2: V / *qslot
-// rounded to nearest even and saturated to signed 8 bit (the quantiser of the INT8 set-up,
-// Section 5.1), as one float multiplication by the reciprocal scale per value.
+// QMODE 0: V rounded to half.  QMODE 1: nothing is stored but the CTA's largest |V|, in
+// qparts[CTA] (first pass of the int8 pipeline's data-derived scale).  QMODE 2: V / s rounded to
+// nearest even and saturated to signed 8 bit (the quantiser of the INT8 set-up, Section 5.1), as one
+// float multiplication by the reciprocal scale per value; s = qgiven, or the largest of the first
+// pass's qparts / 127 where qgiven is 0, and is left in *qslot for the output transform.  (A cleared
+// word, atomics and a kernel that made the scale of it were two more launches per call, and neither
+// could overlap its neighbours.)
 template <int M, int QMODE, int R = 3>
 __global__ void __launch_bounds__(kTcThreads, 1)
 input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmKron,
                           void* __restrict__ Vout, int C, int Th, int Tw, long long p0, int pc, int pc_pad,
-                          int* __restrict__ status, float* __restrict__ qslot) {
+                          int* __restrict__ status, float* __restrict__ qslot, float* __restrict__ qparts, float qgiven) {
   using Cfg = TcCfg<M, R>;
   static_assert(TcCfgCheck<M, R>::ok, "");
   constexpr int kStages = Cfg::kStages;
@@ -112,6 +115,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
   uint64_t* kron_bar = tmem_empty + kNumAcc;
   uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(kron_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_slot + 1);
+  unsigned* cta_max = reinterpret_cast<unsigned*>(tmem_base_slot + 2);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -131,6 +135,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     for (int a = 0; a < kNumAcc; ++a) { mbar_init(&tmem_full[a], 1); mbar_init(&tmem_empty[a], 4); }
     mbar_init(kron_bar, 1);
     *abort_flag = 0;
+    *cta_max = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kProdWarps) tmem_alloc(tmem_base_slot, 512);
@@ -219,7 +224,14 @@ const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
     const size_t f_stride = (size_t)pc_pad * C;
     float qs = 1.f, amax = 0.f;
     if constexpr (QMODE == 2) {
-      qs = *qslot;
+      qs = qgiven;
+      if (!(qs > 0.f)) {
+        float mx = 0.f;
+        for (unsigned i = lane; i < gridDim.x; i += 32) mx = fmaxf(mx, qparts[i]);   // the passes have the same grid
+        mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+        qs = __fdiv_rn(mx, 127.f);
+      }
+      if (blockIdx.x == 0 && quad == 0 && group == 0 && lane == 0) *qslot = qs;
       if (qs == 0.f) qs = 1.f;
       qs = __fdiv_rn(1.f, qs);                    // the quantiser multiplies by the reciprocal scale
     }
@@ -289,7 +301,7 @@ const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
     }
     if constexpr (QMODE == 1) {                   // non-negative floats order like their bit patterns
       const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
-      if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(qslot), mx);
+      if (lane == 0) atomicMax(cta_max, mx);
     }
   }
 
@@ -299,6 +311,7 @@ const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
   }
   tc_fence_before();
   __syncthreads();
+  if (QMODE == 1 && threadIdx.x == 0) qparts[blockIdx.x] = __uint_as_float(*cta_max);
   if (warp == kProdWarps) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
@@ -307,7 +320,7 @@ const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
 
 template <int M, int QMODE, int R = 3>
 int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0, int pc, int pc_pad,
-             float* qslot, cudaStream_t stream) {
+             float* qslot, float* qparts, float qgiven, cudaStream_t stream) {
   using Cfg = TcCfg<M, R>;
   if (cudaError_t e = allow_dynamic_smem(input_transform_tc_kernel<M, QMODE, R>, Cfg::kTotal); e != cudaSuccess) return (int)e;
   EncodeTiledFn enc = tensor_map_encoder();
@@ -337,7 +350,7 @@ int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long 
   const long long units = ((long long)pc * ((g.C + 63) / 64) + 1) / 2;   // two (tile, 64-channel block) pairs each
   const int grid = (int)(units < sms ? units : sms);
   return (int)launch_overlapped(input_transform_tc_kernel<M, QMODE, R>, grid, kTcThreads, Cfg::kTotal, stream, tmX, tmK,
-                                V, g.C, g.Th, g.Tw, p0, pc, pc_pad, plan->status_dev, qslot);
+                                V, g.C, g.Th, g.Tw, p0, pc, pc_pad, plan->status_dev, qslot, qparts, qgiven);
 }
 
 }  // namespace
@@ -372,33 +385,34 @@ int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* 
   cudaStream_t s = (cudaStream_t)stream;
   if (plan->r == 5) {                                 // 5 x 5 filters: n = m + 4 points, halo of 2
     switch (plan->m) {
-      case 2: return launch_m<2, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
-      case 4: return launch_m<4, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
-      case 6: return launch_m<6, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
+      case 2: return launch_m<2, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
+      case 4: return launch_m<4, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
+      case 6: return launch_m<6, 0, 5>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
     }
     return (int)cudaErrorInvalidValue;
   }
   switch (plan->m) {
-    case 2: return launch_m<2, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
-    case 4: return launch_m<4, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
-    case 6: return launch_m<6, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
-    case 8: return launch_m<8, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, s);
+    case 2: return launch_m<2, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
+    case 4: return launch_m<4, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
+    case 6: return launch_m<6, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
+    case 8: return launch_m<8, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
   }
   return (int)cudaErrorInvalidValue;
 }
 
-// int8 pipeline: pass 0 reduces max|V| into *slot (zeroed by the caller), pass 1 quantises with
-// the scale at *slot into Vq [n*n][pc_pad][C] signed bytes.
+// int8 pipeline: pass 0 writes the CTAs' max|V| to parts[0 .. sm_count - 1], pass 1 quantises into Vq
+// [n*n][pc_pad][C] signed bytes with the scale `given` or, if that is 0, the one of pass 0's parts, and
+// leaves the scale in *slot.
 int launch_input_transform_tc_int8(const nova_plan* plan, const Geom& g, const void* x, void* Vq, float* slot,
-                                   int pass, long long p0, int pc, int pc_pad, void* stream) {
+                                   float* parts, float given, int pass, long long p0, int pc, int pc_pad, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
 #define NOVA_TC8(MM) \
-  return pass == 0 ? launch_m<MM, 1>(plan, g, x, Vq, p0, pc, pc_pad, slot, s) \
-                   : launch_m<MM, 2>(plan, g, x, Vq, p0, pc, pc_pad, slot, s)
+  return pass == 0 ? launch_m<MM, 1>(plan, g, x, Vq, p0, pc, pc_pad, slot, parts, given, s) \
+                   : launch_m<MM, 2>(plan, g, x, Vq, p0, pc, pc_pad, slot, parts, given, s)
   if (plan->r == 5) {
 #define NOVA_TC8R5(MM) \
-  return pass == 0 ? launch_m<MM, 1, 5>(plan, g, x, Vq, p0, pc, pc_pad, slot, s) \
-                   : launch_m<MM, 2, 5>(plan, g, x, Vq, p0, pc, pc_pad, slot, s)
+  return pass == 0 ? launch_m<MM, 1, 5>(plan, g, x, Vq, p0, pc, pc_pad, slot, parts, given, s) \
+                   : launch_m<MM, 2, 5>(plan, g, x, Vq, p0, pc, pc_pad, slot, parts, given, s)
     switch (plan->m) {
       case 2: NOVA_TC8R5(2);
       case 4: NOVA_TC8R5(4);
