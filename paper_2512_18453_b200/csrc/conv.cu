@@ -73,6 +73,15 @@ bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
   return fused_fp32_applies(p) || use_fused_small_c(p, g, flags);
 }
 
+// Input transform on the tensor cores or on CUDA cores.  The tensor-core kernel computes 64 channels
+// at a time, zero fill included, and is the faster one for narrow layers too where a tile has enough
+// points: 2 x 14 x 14, 16 -> 64, whole call: F(4,3) 9.7 -> 7.5 us, F(6,3) 15.2 -> 8.9, F(8,3) 17.1 -> 10.1; 32 x 56 x 56,
+// 24 -> 64: 38.7 -> 37.3, 49.8 -> 35.2, 65.4 -> 34.1.  With 4 points its units are too small to pay below 64
+// channels once a layer has many tiles: 98 tiles 8.0 -> 6.7 us, 1568 tiles 11.8 -> 12.1, 12544 tiles 24.3 -> 35.5.
+bool tensor_core_input(const nova_plan* p, const Geom& g, int flags) {
+  return p->kron_dev && !(flags & NOVA_TRANSFORM_SIMT) && (p->n > 4 || g.C >= 64 || g.P <= 1024);
+}
+
 bool use_tcgen05(const nova_plan* p, int flags) {
   if (p->mode == NOVA_FP32) return false;
   return (flags & NOVA_GEMM_SIMT) == 0;
@@ -170,7 +179,7 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
     const int pc = (int)((g.P - p0) < c.pc ? (g.P - p0) : c.pc);
     if (ev) cudaEventRecord(ev[4 * ci + 0], s);
     const bool f32 = p->mode == NOVA_FP32;
-    const bool tc_in = tc && p->kron_dev && C >= 64 && !(flags & NOVA_TRANSFORM_SIMT);
+    const bool tc_in = tc && tensor_core_input(p, g, flags);
     if (f32     ? launch_input_transform_f32(p, g, x, Vb, p0, pc, c.pc_pad, stream)
         : tc_in ? launch_input_transform_tc(p, g, x, Vb, p0, pc, c.pc_pad, stream)
                 : launch_input_transform(p, g, x, Vb, p0, pc, c.pc_pad, stream))
@@ -390,7 +399,7 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
   int e = 0;
   // The tensor-core transform needs the exact hi + lo table of half-rounded coefficients; plans
   // with float32 coefficients (and narrow layers) use the CUDA-core transform.
-  const bool tc_in = p->kron_dev && C >= 64 && !(flags & NOVA_TRANSFORM_SIMT);
+  const bool tc_in = tensor_core_input(p, g, flags);
   if (ev) cudaEventRecord(ev[0], s);
   // s_V is given, or max|V| / 127 over the batch, which costs one more pass of the input transform
   if (tc_in) {

@@ -41,9 +41,8 @@ struct SmemLayout {
   static constexpr int kStageBytes = kABytes + kBBytes;
   // What fits: 4, 6 or 8 stages of 48, 32 or 24 KB.  The narrow blocks run where a CTA has one or
   // two items, and then nearly all of an item's operands are in flight at once.
-  static constexpr int kStages = 196608 / kStageBytes;
-  static constexpr int kBarrierOffset = kStages * kStageBytes;
-  static constexpr int kTotal = kBarrierOffset + 256 + 1024;     // barriers + alignment slack
+  static constexpr int kMaxStages = 196608 / kStageBytes;
+  static constexpr int total(int stages) { return stages * kStageBytes + 256 + 1024; }   // + barriers, alignment slack
 };
 
 // Measurement aid: sums of clock64() spent in (or around) the waits of one warp.  With ON = false
@@ -60,14 +59,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmU,
                     float* __restrict__ Mo, int nfreq, int pc, int pc_pad, int C, int K,
                     int* __restrict__ status, const uint8_t* __restrict__ Vdrop, int f_major, int spread, int keep_pct,
-                    unsigned long long* __restrict__ prof) {
+                    int kStages, unsigned long long* __restrict__ prof) {
   using L = SmemLayout<BLOCK_N>;
-  constexpr int kStages = L::kStages;
   constexpr int BLOCK_K = I8 ? kRowBytes : kRowBytes / 2;   // elements of K per stage
   constexpr uint32_t kTmemCols = 2 * BLOCK_N;       // two accumulators; 128, 256 or 512
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + L::kBarrierOffset);
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kStages * L::kStageBytes);
   uint64_t* empty_bar = full_bar + kStages;
   uint64_t* tmem_full = empty_bar + kStages;        // [2]
   uint64_t* tmem_empty = tmem_full + 2;             // [2]
@@ -338,7 +336,12 @@ template <int BLOCK_N, bool I8>
 int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int nfreq, int pc, int pc_pad, int C, int K,
              int* status, cudaStream_t stream, unsigned long long* prof = nullptr) {
   using L = SmemLayout<BLOCK_N>;
-  if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8>, L::kTotal); e != cudaSuccess) return (int)e;
+  // With 16 frequencies the neighbouring transforms are small enough for their CTAs to run beside this kernel's, if
+  // it leaves them room (F(2,3), 8 x 56 x 56, 64 -> 64: 24.7 us with 8 stages, 18.8 us with 4).  Otherwise as many
+  // stages as fit (F(4,3), 224 x 224, 64 -> 64: 22.9 us with 4, 19.2 us with 8).
+  const int stages = nfreq <= 16 ? 4 : L::kMaxStages;
+  const size_t smem = (size_t)L::total(stages);
+  if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8>, (int)smem); e != cudaSuccess) return (int)e;
   CUtensorMap tmV, tmU;
   const CUtensorMapDataType dt = I8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   constexpr int esize = I8 ? 1 : 2;
@@ -371,15 +374,15 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
   // the wait-profiling variant exists for the half product with 256-wide filter blocks only
   if constexpr (BLOCK_N == 256 && !I8) {
     if (prof) {
-      if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8, true>, L::kTotal); e != cudaSuccess) return (int)e;
+      if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8, true>, (int)smem); e != cudaSuccess) return (int)e;
       // CTAs beyond this launch's grid must read as "did not run"
       if (cudaError_t e = cudaMemsetAsync(prof, 0, sizeof(unsigned long long) * 8 * sms, stream); e != cudaSuccess) return (int)e;
-      return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8, true>, grid, kThreads, L::kTotal, stream, tmV, tmU, M,
-                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, prof);
+      return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8, true>, grid, kThreads, smem, stream, tmV, tmU, M,
+                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, prof);
     }
   }
-  return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8>, grid, kThreads, L::kTotal, stream, tmV, tmU, M, nfreq,
-                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, (unsigned long long*)nullptr);
+  return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8>, grid, kThreads, smem, stream, tmV, tmU, M, nfreq,
+                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, (unsigned long long*)nullptr);
 }
 
 }  // namespace
