@@ -128,6 +128,31 @@ def lib():
     return L
 
 
+_fastcall = None
+
+
+def _fast():
+    """The CPython extension that makes the hot calls (csrc/fastcall.c), bound to libnova's functions; False
+    where the build had no Python headers, and the calls go through ctypes then."""
+    global _fastcall
+    if _fastcall is None:
+        L = lib()
+        try:
+            from . import _fastcall as ext
+        except ImportError:
+            _fastcall = False
+            return False
+        import torch
+        torch.cuda.current_stream()                  # initialises CUDA
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get is None or dev is None:
+            get, dev = (lambda d: torch.cuda.current_stream().cuda_stream), (lambda: 0)
+        addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+        ext.bind(addr(L.nova_conv2d_fwd), addr(L.nova_filter_transform), addr(L.nova_conv2d_fwd_int8), dev, get)
+        _fastcall = ext
+    return _fastcall
+
+
 def status_string(status):
     return lib().nova_status_string(int(status)).decode()
 
@@ -318,8 +343,13 @@ class Plan:
         assert g.is_cuda and g.is_contiguous() and g.dtype == _torch_dtype(self.mode)
         K, _, _, C = g.shape
         U = torch.empty(self.n * self.n, K, C, dtype=g.dtype, device=g.device)
-        _check(lib().nova_filter_transform(self._h, g.data_ptr(), K, C, U.data_ptr(), _stream()),
-               "nova_filter_transform")
+        ext = _fastcall or _fast()
+        if ext:
+            h = self._h
+            st = ext.filter_transform(h.value if h else 0, g, K, C, U)
+        else:
+            st = lib().nova_filter_transform(self._h, g.data_ptr(), K, C, U.data_ptr(), _stream())
+        _check(st, "nova_filter_transform")
         return U
 
     def workspace_bytes(self, N, H, W, C, K):
@@ -333,6 +363,13 @@ class Plan:
 
     def conv2d(self, x, U, y=None, workspace=None, flags=0):
         """x [N,H,W,C], U from filter_transform -> y [N,H,W,K]."""
+        ext = _fastcall or _fast()
+        if ext and y is not None and workspace is not None:
+            h = self._h
+            st = ext.conv2d(h.value if h else 0, _torch_dtype(self.mode), x, U, y, workspace, flags)
+            if st:
+                raise NovaError(st, "nova_conv2d_fwd")
+            return y
         assert x.is_cuda and x.is_contiguous() and x.dtype == _torch_dtype(self.mode)
         N, H, W, C = x.shape
         K = U.shape[1]
@@ -409,6 +446,12 @@ class Plan:
             y = torch.empty((N, H // 2, W // 2, K) if flags & POOL2X2 else (N, H, W, K), dtype=torch.float16, device=x.device)
         if workspace is None:
             workspace = torch.empty(self.int8_workspace_bytes(N, H, W, C, K), dtype=torch.uint8, device=x.device)
+        ext = _fastcall or _fast()
+        if ext and not timed:
+            h = self._h
+            _check(ext.conv2d_int8(h.value if h else 0, x, Uq, scale_U, scale_V, y, workspace, N, H, W, C, K, flags),
+                   "nova_conv2d_fwd_int8")
+            return y
         args = (self._h, x.data_ptr(), Uq.data_ptr(), scale_U.data_ptr(), float(scale_V), y.data_ptr(),
                 N, H, W, C, K, workspace.data_ptr(), workspace.numel(), flags, _stream())
         if timed:

@@ -2,11 +2,13 @@
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnova.so")
+EXT = os.path.join(HERE, "_fastcall.so")
 SOURCES = ["plan.cpp", "transforms.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "conv.cu"]
 
 
@@ -21,12 +23,25 @@ def needs_build():
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "nova.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "fastcall.c"] + [os.path.join(ROOT, "include", "nova.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_ext():
+    """The CPython extension of the binding's hot calls; without Python headers the binding uses ctypes."""
+    src, inc = os.path.join(CSRC, "fastcall.c"), sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(inc, "Python.h")):
+        sys.stderr.write("no Python headers in %s: calls go through ctypes\n" % inc)
+        return
+    newest = max(os.path.getmtime(f) for f in (src, os.path.join(ROOT, "include", "nova.h")))
+    if not os.path.exists(EXT) or os.path.getmtime(EXT) < newest:
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                               "-I", inc, src, "-o", EXT])
 
 
 def build(force=False, verbose=False):
     """Compile every source for sm_100a and link the shared library."""
+    build_ext()
     if not force and not needs_build():
         return LIB
     objdir = os.path.join(HERE, "_build")
