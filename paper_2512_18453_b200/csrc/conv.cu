@@ -77,7 +77,8 @@ bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
 // at a time, zero fill included, and is the faster one for narrow layers too where a tile has enough
 // points: 2 x 14 x 14, 16 -> 64, whole call: F(4,3) 9.7 -> 7.5 us, F(6,3) 15.2 -> 8.9, F(8,3) 17.1 -> 10.1; 32 x 56 x 56,
 // 24 -> 64: 38.7 -> 37.3, 49.8 -> 35.2, 65.4 -> 34.1.  With 4 points its units are too small to pay below 64
-// channels once a layer has many tiles: 98 tiles 8.0 -> 6.7 us, 1568 tiles 11.8 -> 12.1, 12544 tiles 24.3 -> 35.5.
+// channels once a layer has many tiles (98 tiles 8.0 -> 6.7 us, 1568 tiles 11.8 -> 12.1, 12544 tiles 24.3 -> 35.5); the
+// half pipeline has a kernel of its own for them, so that the line matters to the INT8 pipeline alone.
 bool tensor_core_input(const nova_plan* p, const Geom& g, int flags) {
   return p->kron_dev && !(flags & NOVA_TRANSFORM_SIMT) && (p->n > 4 || g.C >= 64 || g.P <= 1024);
 }
@@ -179,8 +180,10 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
     const int pc = (int)((g.P - p0) < c.pc ? (g.P - p0) : c.pc);
     if (ev) cudaEventRecord(ev[4 * ci + 0], s);
     const bool f32 = p->mode == NOVA_FP32;
+    const bool n4_in = tc && p->n == 4 && !(flags & NOVA_TRANSFORM_SIMT);
     const bool tc_in = tc && tensor_core_input(p, g, flags);
     if (f32     ? launch_input_transform_f32(p, g, x, Vb, p0, pc, c.pc_pad, stream)
+        : n4_in ? launch_input_transform_n4(p, g, x, Vb, p0, pc, c.pc_pad, stream)
         : tc_in ? launch_input_transform_tc(p, g, x, Vb, p0, pc, c.pc_pad, stream)
                 : launch_input_transform(p, g, x, Vb, p0, pc, c.pc_pad, stream))
       return NOVA_ERR_CUDA;

@@ -336,11 +336,14 @@ template <int BLOCK_N, bool I8>
 int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int nfreq, int pc, int pc_pad, int C, int K,
              int* status, cudaStream_t stream, unsigned long long* prof = nullptr) {
   using L = SmemLayout<BLOCK_N>;
-  // With 16 frequencies the neighbouring transforms are small enough for their CTAs to run beside this kernel's, if
-  // it leaves them room (F(2,3), 8 x 56 x 56, 64 -> 64: 24.7 us with 8 stages, 18.8 us with 4).  Otherwise as many
-  // stages as fit (F(4,3), 224 x 224, 64 -> 64: 22.9 us with 4, 19.2 us with 8).
-  const int stages = nfreq <= 16 ? 4 : L::kMaxStages;
-  const size_t smem = (size_t)L::total(stages);
+  // With 16 frequencies the output transform is small enough for its CTAs to run beside this kernel's, if it leaves
+  // them room (F(2,3), 8 x 56 x 56, 64 -> 64: 24.7 us with 8 stages, 18.8 us with 4); the padding keeps two of this
+  // kernel's own CTAs from sharing an SM while another SM has none (22.1 us without).  Otherwise as many stages as fit
+  // (F(4,3), 224 x 224, 64 -> 64: 22.9 us with 4, 19.2 us with 8).
+  const bool lean = nfreq <= 16 && BLOCK_N < 256;
+  const int stages = lean ? (BLOCK_N == 64 ? 4 : 3) : L::kMaxStages;
+  size_t smem = (size_t)L::total(stages);
+  if (lean && smem < 118 * 1024) smem = 118 * 1024;
   if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8>, (int)smem); e != cudaSuccess) return (int)e;
   CUtensorMap tmV, tmU;
   const CUtensorMapDataType dt = I8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;

@@ -392,7 +392,6 @@ int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* 
     return (int)cudaErrorInvalidValue;
   }
   switch (plan->m) {
-    case 2: return launch_m<2, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
     case 4: return launch_m<4, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
     case 6: return launch_m<6, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);
     case 8: return launch_m<8, 0>(plan, g, x, V, p0, pc, pc_pad, nullptr, nullptr, 0.f, s);

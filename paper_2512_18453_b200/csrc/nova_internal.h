@@ -79,6 +79,9 @@ inline Geom make_geom(const nova_plan* p, int N, int H, int W, int C, int K) {
 int launch_filter_transform(const nova_plan* plan, const void* g, int K, int C, void* U, void* stream);
 int launch_input_transform(const nova_plan* plan, const Geom& g, const void* x, void* V,
                            long long p0, int pc, int pc_pad, void* stream);
+// half mode, 4 points, any channel count
+int launch_input_transform_n4(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0, int pc,
+                              int pc_pad, void* stream);
 int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* x, void* V,
                               long long p0, int pc, int pc_pad, void* stream);
 size_t kron_table_halves(int n);   // n points

@@ -339,6 +339,30 @@ def test_many_units_per_cta_in_every_ring(kind, m, shape):
     check_fp16(ya, x, g, m, pts)
 
 
+@pytest.mark.parametrize("kind", ["std", "asym"])
+@pytest.mark.parametrize("shape", [(1, 1, 1, 8, 8), (2, 3, 5, 8, 16), (1, 31, 2, 24, 24), (3, 17, 18, 200, 16), (1, 64, 66, 512, 8)])
+def test_four_point_input_transform_agrees_with_the_plain_kernel(kind, shape):
+    # F(2,3): a thread owns four channels of a tile; the plain kernel sums the same terms.
+    # Images smaller than a tile, odd sizes, channel counts that end inside a warp
+    N, H, W, C, K = shape
+    x, g = make_conv_inputs(N, H, W, C, K, "fp16", False, True, seed=495)
+    pts = point_set(kind, 2)
+    ya, _, _ = gpu_conv(x, g, 2, pts, nv.FP16_F32ACC, nv.GEMM_TCGEN05)
+    plan = nv.Plan(2, pts)
+    xd = torch.from_numpy(x).cuda()
+    U = plan.filter_transform(torch.from_numpy(g).cuda())
+    yb = plan.conv2d(xd, U, flags=nv.GEMM_TCGEN05 | nv.TRANSFORM_SIMT).cpu().numpy()
+    # Both evaluate V in float and round once to half, so y differs by flips of the last bit of V and of y: below
+    # 2^-11 in norm and 4 * 2^-10 of the largest output element by element (as the two products above).  The per-tile
+    # bound of check_fp16 does not apply: a tile has 4 * K = 32 outputs here, and one flipped last bit among them
+    # (2^-11 / sqrt(32)) is of the order of the tile's whole emulation error (5e-4 / sqrt(32) and less).
+    assert conv.rel_l2(ya, yb) <= 2.0 ** -11
+    d = np.abs(ya.astype(np.float32) - yb.astype(np.float32))
+    assert d.max() <= 4 * 2.0 ** -10 * np.abs(yb.astype(np.float32)).max()
+    y1 = conv.direct_conv_fp64(x, g)
+    assert conv.rel_l2(ya, y1) <= 2.0 * conv.rel_l2(conv.winograd_conv_emulated(x, g, 2, pts, "fp16"), y1)
+
+
 def test_ragged_last_row_block_after_full_blocks():
     """532 tiles = 4 full 128-row blocks + 20 rows, 36 x 5 work items on 148 SMs: a CTA
     that handles a full block and then the ragged one must not reuse an epilogue
