@@ -339,10 +339,9 @@ class Plan:
 
     def filter_transform(self, g):
         """g [K,3,3,C] on the GPU in the plan's storage dtype -> opaque U tensor."""
-        import torch
         assert g.is_cuda and g.is_contiguous() and g.dtype == _torch_dtype(self.mode)
         K, _, _, C = g.shape
-        U = torch.empty(self.n * self.n, K, C, dtype=g.dtype, device=g.device)
+        U = g.new_empty((self.n * self.n, K, C))
         ext = _fastcall or _fast()
         if ext:
             h = self._h

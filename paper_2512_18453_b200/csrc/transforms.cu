@@ -80,8 +80,8 @@ __global__ void scales_from_absmax_kernel(float* slots, int count, int per_chann
 }
 __global__ void set_scale_kernel(float* slot, float value) { *slot = value; }
 
-// ---------------------------------------------------------------- U = G g G^T
-// One thread per (filter k, channel pair).  g [K,3,3,C] -> U [n*n][K][C].
+// ---------------------------------------------------------------- U = G g G^T for the int8 pipeline
+// (the half pipeline's is filter_transform.cu).  One thread per (filter k, channel pair).  g [K,3,3,C] -> U [n*n][K][C].
 template <int M, typename T, typename Sink, int R = 3>
 __global__ void __launch_bounds__(256)
 filter_transform_kernel(const __grid_constant__ Coefs cf, const T* __restrict__ g, Sink sink,
@@ -343,21 +343,6 @@ inline unsigned blocks_for(long long work, int threads) {
   return (unsigned)((work + threads - 1) / threads);
 }
 
-template <int M, typename T>
-int filter_launch(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
-  const long long work = (long long)K * (C / 2);
-  if (plan->r == 5) {
-    if constexpr (M <= 6)
-      filter_transform_kernel<M, T, StoreSink<T>, 5><<<blocks_for(work, 256), 256, 0, s>>>(
-          plan->kcoefs, (const T*)g, StoreSink<T>{(T*)U}, K, C);
-    else
-      return (int)cudaErrorInvalidValue;
-    return (int)cudaGetLastError();
-  }
-  filter_transform_kernel<M, T, StoreSink<T>><<<blocks_for(work, 256), 256, 0, s>>>(
-      plan->kcoefs, (const T*)g, StoreSink<T>{(T*)U}, K, C);
-  return (int)cudaGetLastError();
-}
 // int8 filter transform: absmax pass (unless the scales are given), scales, quantising pass.
 template <int M, typename T>
 int filter_launch_int8(const nova_plan* plan, const void* g, int K, int C, void* Uq, float* scales, int quant,
@@ -499,9 +484,6 @@ int output_launch(const nova_plan* plan, const Geom& g, const void* Mb, void* y,
     return (int)cudaErrorInvalidValue;                                               \
   } while (0)
 
-int launch_filter_transform(const nova_plan* plan, const void* g, int K, int C, void* U, void* stream) {
-  NOVA_DISPATCH_M_T(filter_launch, plan, g, K, C, U, (cudaStream_t)stream);
-}
 int launch_input_transform(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0,
                            int pc, int pc_pad, void* stream) {
   NOVA_DISPATCH_M_T(input_launch, plan, g, x, V, p0, pc, pc_pad, (cudaStream_t)stream);
