@@ -23,7 +23,7 @@ using namespace xf;
 constexpr int kFtThreads = 256;
 
 template <int N, int R>
-constexpr int rows_per_thread() { return R == 3 ? 2 : N / 2; }
+constexpr int kRowsPerThread = R == 3 ? 2 : N / 2;
 
 template <int N, int R>
 __global__ void __launch_bounds__(kFtThreads)
@@ -47,8 +47,8 @@ filter_transform_half_kernel(const __grid_constant__ Coefs cf, const __half* __r
   const size_t f_stride = (size_t)K * C;
   __half* dst = U + (size_t)k * C + c;
 #pragma unroll
-  for (int e = 0; e < rows_per_thread<N, R>(); ++e) {
-    const int p = rows_per_thread<N, R>() * (int)blockIdx.y + e;
+  for (int e = 0; e < kRowsPerThread<N, R>; ++e) {
+    const int p = kRowsPerThread<N, R> * (int)blockIdx.y + e;
     float2 t[2][R];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -78,7 +78,7 @@ template <int N, int R>
 int go(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
   const long long work = (long long)K * (C / 4);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / rows_per_thread<N, R>());
+  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / kRowsPerThread<N, R>);
   cfg.blockDim = dim3(kFtThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
