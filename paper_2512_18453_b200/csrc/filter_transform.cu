@@ -2,10 +2,10 @@
 // evaluated in float and rounded once to half.  g [K,R,R,C] -> U [n*n][K][C].
 //
 // What bounds it: the stores of U, n*n / (R*R) times the bytes of g.  A thread owns one filter, four consecutive
-// channels (eight-byte accesses, a warp's store 256 contiguous bytes) and some rows of the n x n frequencies, so that
-// a small layer still spreads over the SMs; the threads that share a filter's taps find them in the L1 or L2.  Two rows
-// with 9 taps; half of the rows with 25, whose loads weigh more.  Launched as a programmatic dependent: a plain launch
-// costs the host up to twice as much and nothing of it overlaps.
+// channels (eight-byte accesses, a warp's store 256 contiguous bytes) and two rows of the n x n frequencies, so that
+// a small layer still spreads over the SMs; the threads that share a filter's taps find them in the L1 or L2 (F(4,5),
+// 512 x 512: 12.6 us with two rows, 13.6 with half of the rows per thread).  Launched as a programmatic dependent: a
+// plain launch costs the host up to twice as much and nothing of it overlaps.
 // Against one thread per channel pair and whole filter, launched plainly: F(6,3) 512 x 512 (38 MB) 7.5 -> 7.2 us back to
 // back, 64 x 64 3.4 -> 2.1; F(8,3) 512 x 512 (57 MB) 10.9 -> 9.9; per call 11.2 -> 6.0 us wherever the host is the bound.
 #include <cuda_fp16.h>
@@ -21,9 +21,6 @@ namespace {
 using namespace xf;
 
 constexpr int kFtThreads = 256;
-
-template <int N, int R>
-constexpr int kRowsPerThread = R == 3 ? 2 : N / 2;
 
 template <int N, int R>
 __global__ void __launch_bounds__(kFtThreads)
@@ -47,8 +44,8 @@ filter_transform_half_kernel(const __grid_constant__ Coefs cf, const __half* __r
   const size_t f_stride = (size_t)K * C;
   __half* dst = U + (size_t)k * C + c;
 #pragma unroll
-  for (int e = 0; e < kRowsPerThread<N, R>; ++e) {
-    const int p = kRowsPerThread<N, R> * (int)blockIdx.y + e;
+  for (int e = 0; e < 2; ++e) {
+    const int p = 2 * (int)blockIdx.y + e;
     float2 t[2][R];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -78,7 +75,7 @@ template <int N, int R>
 int go(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
   const long long work = (long long)K * (C / 4);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / kRowsPerThread<N, R>);
+  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / 2);
   cfg.blockDim = dim3(kFtThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
