@@ -667,6 +667,8 @@ def run_int8(args):
     else:
         achieved, peak, runit = work / dur / 1e9, peaks["hbm_gbs"], "GB/s"
     roof_s = max(actual / (i8_peak * 1e12), min_bytes / (peaks["hbm_gbs"] * 1e9))
+    # input transform once or twice, product, output transform; the CUDA-core input transform has a scale kernel besides
+    launches = (4 if scale_V == 0 else 3) + (1 if args.int8_coef == "fp32" else 0)
     out = {
         "metric": METRIC.replace("fp16", "int8"), "value": whole_job_value(world, direct, ms_per_step), "unit": UNIT,
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
@@ -690,7 +692,7 @@ def run_int8(args):
                      "frac": achieved / peak, "traffic": None, "peak_source": peaks["source"], "launch_us": dur * 1e6},
         "e2e": {"value": world * direct / (e2e_ms * 1e-3) / 1e12, "unit": UNIT, "ms_per_step": e2e_ms,
                 "h2d_bytes_per_step": int(x_np.nbytes), "d2h_bytes_per_step": int(yh.numel() * 2)},
-        "gpu_launches": (3 + 2 * passes) * args.steps if scale_V == 0 else 4 * args.steps,
+        "gpu_launches": launches * args.steps,
         "device_status": status, "kappa2_V": plan.kappa(), "clocks": clocks,
     }
     if world == 1 and (args.accuracy or not args.no_cpu_baseline):

@@ -64,10 +64,13 @@ bool on_plan_device(const nova_plan* p) {
 
 // The one-kernel path for 8 input channels runs unless a flag asks for a particular kernel of the
 // three-kernel path.
+constexpr int kThreeKernelFlags = NOVA_GEMM_SIMT | NOVA_GEMM_TCGEN05 | NOVA_TRANSFORM_SIMT | NOVA_PROFILE_WAITS;
 bool use_fused_small_c(const nova_plan* p, const Geom& g, int flags) {
-  const int forcing = NOVA_GEMM_SIMT | NOVA_GEMM_TCGEN05 | NOVA_TRANSFORM_SIMT | NOVA_PROFILE_WAITS | NOVA_POOL2X2;
-  return (flags & forcing) == 0 && fused_small_c_applies(p, g);
+  return (flags & (kThreeKernelFlags | NOVA_POOL2X2)) == 0 && fused_small_c_applies(p, g);
 }
+
+// Bits of the output stage's `relu` argument: 0 = ReLU, 1 = pooled store
+int store_flags(int flags) { return ((flags & NOVA_RELU) ? 1 : 0) | ((flags & NOVA_POOL2X2) ? 2 : 0); }
 
 bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
   return fused_fp32_applies(p) || use_fused_small_c(p, g, flags);
@@ -81,6 +84,24 @@ bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
 // half pipeline has a kernel of its own for them, so that the line matters to the INT8 pipeline alone.
 bool tensor_core_input(const nova_plan* p, const Geom& g, int flags) {
   return p->kron_dev && !(flags & NOVA_TRANSFORM_SIMT) && (p->n > 4 || g.C >= 64 || g.P <= 1024);
+}
+
+// Product and output transform in one kernel, for callers with the recommended workspace (a smaller one asks for the
+// chunked three kernels); only V is in it then, in as many chunks as it takes.
+bool two_kernels(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags, Chunking* c) {
+  if ((flags & kThreeKernelFlags) || !use_product_output(p, g, false)) return false;
+  if (ws_bytes < nova_conv2d_workspace_bytes(p, g.N, g.H, g.W, g.C, g.K)) return false;
+  const size_t v_tile = (size_t)g.n * g.n * g.C * elt_bytes(p->mode);
+  long long pc = (long long)(ws_bytes / v_tile) / 128 * 128;
+  const long long p_pad = round_up_ll(g.P, 128);
+  if (pc > p_pad) pc = p_pad;
+  if (pc < 128) return false;
+  c->pc = (int)(pc < g.P ? pc : g.P);
+  c->pc_pad = (int)pc;
+  c->chunks = (int)((g.P + pc - 1) / pc);
+  c->v_bytes = (size_t)pc * v_tile;
+  c->m_bytes = 0;
+  return true;
 }
 
 bool use_tcgen05(const nova_plan* p, int flags) {
@@ -134,6 +155,7 @@ extern "C" int nova_conv2d_launch_count(const nova_plan* p, int N, int H, int W,
   Chunking c;
   if (!choose_chunking(p, g, workspace_bytes, &c)) return NOVA_ERR_WORKSPACE;
   if (one_kernel(p, g, flags)) return 1;
+  if (two_kernels(p, g, workspace_bytes, flags, &c)) return 2 * c.chunks;
   return 3 * c.chunks;
 }
 
@@ -171,6 +193,7 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
   }
   const bool tc = use_tcgen05(p, flags);
   if (tc && !p->status_dev) return NOVA_ERR_CUDA;
+  const bool two = two_kernels(p, g, ws_bytes, flags, &c);
   char* Vb = static_cast<char*>(ws);
   float* Mb = reinterpret_cast<float*>(Vb + c.v_bytes);
   const int nfreq = g.n * g.n;
@@ -188,12 +211,20 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
                 : launch_input_transform(p, g, x, Vb, p0, pc, c.pc_pad, stream))
       return NOVA_ERR_CUDA;
     if (ev) cudaEventRecord(ev[4 * ci + 1], s);
+    if (two) {
+      if (int e = launch_product_output(p, g, Vb, U, y, p0, pc, c.pc_pad, store_flags(flags), stream)) {
+        g_last_cuda_error = e;
+        return NOVA_ERR_CUDA;
+      }
+      if (ev) { cudaEventRecord(ev[4 * ci + 2], s); cudaEventRecord(ev[4 * ci + 3], s); }
+      continue;
+    }
     const int e = tc ? launch_gemm_tcgen05(p, Vb, U, Mb, nfreq, pc, c.pc_pad, C, K, p->status_dev, stream,
                                            (flags & NOVA_PROFILE_WAITS) ? p->prof_dev : nullptr)
                      : launch_gemm_simt(p, Vb, U, Mb, nfreq, pc, c.pc_pad, C, K, stream);
     if (e) return NOVA_ERR_CUDA;
     if (ev) cudaEventRecord(ev[4 * ci + 2], s);
-    const int relu = ((flags & NOVA_RELU) ? 1 : 0) | ((flags & NOVA_POOL2X2) ? 2 : 0);   // bit 1: pooled store
+    const int relu = store_flags(flags);
     if (f32 ? launch_output_transform_f32(p, g, Mb, y, p0, pc, c.pc_pad, relu, stream)
         : (p->status_dev && !(flags & NOVA_TRANSFORM_SIMT))
             ? launch_output_transform_tma(p, g, Mb, y, p0, pc, c.pc_pad, relu, stream)
@@ -229,7 +260,8 @@ extern "C" int nova_conv2d_fwd_timed(const nova_plan* p, const void* x, const vo
     cudaEventDestroy(e2[1]);
     return st1;
   }
-  const int chunks = launches / 3;
+  Chunking two;                      // two kernels per chunk: the second one's time is reported as the product's
+  const int chunks = two_kernels(p, make_geom(p, N, H, W, C, K), ws_bytes, flags, &two) ? two.chunks : launches / 3;
   cudaEvent_t* ev = new cudaEvent_t[4 * chunks];
   for (int i = 0; i < 4 * chunks; ++i) cudaEventCreate(&ev[i]);
   int st = conv2d_fwd_impl(p, x, U, y, N, H, W, C, K, ws, ws_bytes, flags, stream, ev);
@@ -436,13 +468,19 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
     if (!e) e = launch_input_transform_int8(p, g, x, Vq, slot, 1, 0, pc, l.pad, stream);
   }
   if (ev) cudaEventRecord(ev[1], s);
+  if (!e && use_product_output(p, g, true) && !(flags & kThreeKernelFlags)) {
+    e = launch_product_output(p, g, Vq, Uq, y, 0, pc, l.pad, store_flags(flags), stream, scale_U, slot);
+    if (ev) { cudaEventRecord(ev[2], s); cudaEventRecord(ev[3], s); }
+    if (e) g_last_cuda_error = e;
+    return e ? NOVA_ERR_CUDA : NOVA_OK;
+  }
   if (!e)
     e = (flags & NOVA_GEMM_SIMT) ? launch_gemm_simt_i8(Vq, Uq, Mb, nfreq, pc, l.pad, C, K, stream)
                                  : launch_gemm_tcgen05_i8(p, Vq, Uq, Mb, nfreq, pc, l.pad, C, K, p->status_dev, stream);
   if (ev) cudaEventRecord(ev[2], s);
   if (!e)
     e = launch_output_transform_tma(p, g, Mb, y, 0, pc, l.pad,
-                                    ((flags & NOVA_RELU) ? 1 : 0) | ((flags & NOVA_POOL2X2) ? 2 : 0), stream, scale_U, slot);
+                                    store_flags(flags), stream, scale_U, slot);
   if (ev) cudaEventRecord(ev[3], s);
   if (e) g_last_cuda_error = e;
   return e ? NOVA_ERR_CUDA : NOVA_OK;

@@ -122,6 +122,11 @@ int launch_fused_small_c(const nova_plan* plan, const Geom& g, const void* x, co
 // The same for the fp32 mode (tiles of up to 8 points)
 bool fused_fp32_applies(const nova_plan* plan);
 int launch_fused_fp32(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, void* stream);
+// Product and output transform in one kernel (tiles of 4, 6 or 8 points), tiles p0 .. p0+pc-1; scale_U / scale_V
+// non-null: the int8 pipeline.  relu: bit 0 = ReLU, bit 1 = pooled store
+bool use_product_output(const nova_plan* plan, const Geom& g, bool int8);
+int launch_product_output(const nova_plan* plan, const Geom& g, const void* V, const void* U, void* y, long long p0, int pc,
+                          int pc_pad, int relu, void* stream, const float* scale_U = nullptr, const float* scale_V = nullptr);
 int launch_maxpool2x2(const void* x, void* y, int N, int H, int W, int C, int mode, void* stream);
 
 }  // namespace nova

@@ -1124,6 +1124,42 @@ def test_vgg_stack_with_fused_pooling_gives_the_same_bits():
     assert a.shape == b.shape and np.array_equal(a.view(np.int16), b.view(np.int16))
 
 
+# ---------------------------------------------------------------- product and output transform in one kernel
+@pytest.mark.parametrize("op,m,key,r,shape", [
+    ("conv", 2, ("std", 2), 3, (4, 64, 66, 24, 72)),        # 33 blocks of 128 tiles, filter blocks of 64 + 8
+    ("conv", 2, ("asym", 2), 3, (1, 20, 20, 136, 2056)),    # 100 tiles: boxes of fewer than 128 rows; 33 filter blocks
+    ("conv", 4, ("nova", 4), 3, (2, 104, 106, 16, 520)),    # 1404 tiles, last block 124, filter blocks of 32, the last of 8
+    ("conv", 4, ("asym", 4), 3, (3, 102, 98, 72, 952)),     # two rows of channels, ragged tiles
+    ("conv", 6, ("half", 6), 3, (6, 116, 118, 64, 520)),    # 8-CTA clusters
+    ("conv", 6, ("asym", 6), 3, (6, 116, 118, 104, 520)),
+    ("conv", 2, ("nova", 4), 5, (2, 84, 82, 16, 128)),
+    ("conv", 4, ("half", 6), 5, (2, 62, 66, 40, 160)),
+    ("int8", 4, ("dyadic", 4), 3, (2, 104, 106, 112, 528)), ("int8", 2, ("std", 2), 3, (4, 64, 66, 272, 80))])
+def test_product_and_output_in_one_kernel_give_the_bits_of_two(op, m, key, r, shape):
+    # The same sums in the same order, M kept on the chip: bit for bit the output of the separate kernels (which a flag
+    # names), plain and pooled.
+    N, H, W, C, K = shape
+    plan = nv.Plan(m, point_set(*key), r=r)
+    gen = torch.Generator(device="cuda").manual_seed(77 + m)
+    x = torch.randn(N, H, W, C, generator=gen, device="cuda").relu_().half()
+    g = (torch.randn(K, r, r, C, generator=gen, device="cuda") * (2.0 / (r * r * C)) ** 0.5).half()
+    if op == "conv":
+        U = plan.filter_transform(g)
+        ws = plan.workspace_bytes(N, H, W, C, K)
+        assert plan.launch_count(N, H, W, C, K, ws, nv.RELU) == 2
+        assert plan.launch_count(N, H, W, C, K, ws, nv.GEMM_TCGEN05) == 3
+        run = lambda flags: plan.conv2d(x, U, flags=flags)
+    else:
+        U, sU = plan.filter_transform_int8(g, nv.QUANT_PER_CHANNEL)
+        run = lambda flags: plan.conv2d_int8(x, U, sU, flags=flags)
+    for flags in (0, nv.RELU | nv.POOL2X2):
+        got, want = run(flags), run(flags | nv.GEMM_TCGEN05)
+        torch.cuda.synchronize()
+        assert plan.device_status() == 0
+        assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+        assert torch.isfinite(got.float()).all()
+
+
 def test_pooled_output_through_the_int8_and_host_entry_points():
     m, N, H, W, C, K = 4, 3, 20, 24, 64, 80
     x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=421)
