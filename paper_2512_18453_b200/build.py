@@ -9,7 +9,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnova.so")
 EXT = os.path.join(HERE, "_fastcall.so")
-SOURCES = ["plan.cpp", "transforms.cu", "filter_transform.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "input_transform_n4.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "conv.cu"]
+SOURCES = ["plan.cpp", "transforms.cu", "filter_transform.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "input_transform_n4.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "product_output.cu", "conv.cu"]
 
 
 def _nvcc():
