@@ -1,10 +1,10 @@
 // Section 2.1 steps 2-4 in ONE kernel for layers with 8 input channels (half mode, 3-tap filters):
-// V = B^T d B, M[f] = V[f] U[f]^T and Y = A^T M A for a group of 8 tiles at a time, with V and M
+// V = B^T d B, M[f] = V[f] U[f]^T and Y = A^T M A for a group of 8 to 64 tiles at a time, with V and M
 // never leaving the SM.  The first layer of an image network is of this kind (3 colour channels
 // padded to 8).  There the three-kernel path is bound by its intermediate tensors alone - the
 // n*n*K floats of M per tile are 160 times the bytes of the tile's input patch - while the product
 // itself is tiny (8 channels), so it fits the register-level tensor-core instruction: one
-// mma.sync m16n8k8 per frequency gives M[f] for 8 tiles x 8 filters, the two results a thread
+// mma.sync m16n8k8 per frequency gives M[f] for 16 tiles x 8 filters, two results that a thread
 // holds are the same tile's two adjacent filters, i.e. one packed-fp32 operand of the output
 // transform, whose n*n inputs per (tile, filter) are consumed row by row and never all alive.
 // (The TMEM-accumulator route of the large-C product kernel cannot do this: n*n frequencies x 8
@@ -12,7 +12,7 @@
 //
 // One CTA per SM, 12 warps in two roles with their own register budgets (setmaxnreg); the CTA
 // keeps the transformed filters of its 64-filter block in shared memory for its whole life and
-// walks groups of 8 consecutive tiles:
+// walks groups of consecutive tiles:
 //   helper warps (4)   TMA: one n x n x 8-channel box per tile straight from x (out-of-range pixels
 //                      read as 0: halo and ragged tiles), issued for the next group as soon as
 //                      pass 1 has read this one's;
@@ -24,7 +24,7 @@
 //   product warps (8)  warp w owns filters 8w..8w+7: per row xi of frequencies n mma.sync, then
 //                      A^T along nu and the accumulation of Y = sum_xi A^T[.][xi] z_xi, all in
 //                      registers (packed fp32); Y rounded to half (and ReLU) into a shared-memory
-//                      image of the 8 tiles x 64 filters
+//                      image of the group's tiles x 64 filters
 // The roles meet at mbarriers (V full / free, image full / free), every wait bounded.
 // Rounding points are those of the three-kernel path: tables as the plan holds them, V evaluated
 // in float and rounded once to half, products of halves summed in float, Y evaluated in float and
@@ -44,9 +44,7 @@ using namespace xf;
 
 constexpr int kProductWarps = 8;   // two warpgroups
 constexpr int kHelperWarps = 4;    // one warpgroup
-constexpr int kStoreLanes = 16;    // lanes per helper warp that issue the copies of y: 64 threads, one per (tile, output row)
 constexpr int kThreads = (kProductWarps + kHelperWarps) * 32;
-constexpr int kGroupTiles = 8;     // rows 0..7 of the m16n8k8 product (rows 8..15 are fed zeros)
 constexpr int kFilterBlock = 64;   // 8 product warps x 8 filters
 // Registers per thread after the role split.  The CTA is alone on its SM (shared memory), so the
 // register file holds 256 x 216 + 128 x 72 = 64 512 <= 65 536 whatever the kernel was launched with.
@@ -56,9 +54,18 @@ constexpr int kHelperRegs = 72;
 // barrier of the helper warps only
 __device__ __forceinline__ void helper_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kHelperWarps * 32) : "memory"); }
 
-template <int M>
+// Tiles of a large group.  A group costs some 3000 cycles of hand-overs between the roles whatever it holds, so it is
+// as large as shared memory (and, for the copies of y, 128 helper threads) allow: 64, 32, 16, 8.  The product takes 16 of
+// them at a time, the rows of one m16n8k8; with 8 outputs per row only 8 (a thread can hold the Y of two (tile, filter)
+// pairs there, not four) and rows 8..15 are fed zeros.
+constexpr int large_group(int M) { return M == 2 ? 64 : M == 4 ? 32 : M == 6 ? 16 : 8; }
+
+template <int M, int GT>
 struct SmallCLayout {
   static constexpr int N = M + 2;
+  static constexpr int kGroupTiles = GT;
+  static constexpr int kStoreLanes = kGroupTiles * M / kHelperWarps;    // lanes per helper warp that copy y, one output row each
+  static_assert(kStoreLanes <= 32, "");
   static constexpr int kPatchBytes = N * N * 16;                        // one tile: [a][b][8 halves]
   static constexpr int kPatchStride = (kPatchBytes + 127) & ~127;       // TMA destinations: 128-byte aligned
   static constexpr int kUBytes = N * kFilterBlock * 4 * N * 4;          // [xi][filter][channel pair][nu] half2
@@ -93,47 +100,61 @@ __device__ __forceinline__ uint2 lds_v2(uint32_t saddr) {
   return v;
 }
 #pragma nv_diag_suppress 550
-// D[0..7][0..7] = A[0..7][0..7] * B[0..7][0..7] (halves, float sums) on the warp's tensor-core
-// path; rows 8..15 of A are zero and their results are dropped.  A thread (g = lane / 4, t = lane
-// % 4) passes A[g][2t, 2t+1] and B[2t, 2t+1][g] and receives D[g][2t, 2t+1].
-__device__ __forceinline__ float2 mma_8x8x8(uint32_t a, uint32_t b) {
-  float d0, d1, d2, d3;                 // d2, d3: rows 8..15, unused
+// D[0..15][0..7] = A[0..15][0..7] * B[0..7][0..7] (halves, float sums) on the warp's tensor-core path.  A thread (g =
+// lane / 4, t = lane % 4) passes A[g][2t, 2t+1], A[g + 8][2t, 2t+1] and B[2t, 2t+1][g] and receives D[g][2t, 2t+1]
+// and D[g + 8][2t, 2t+1].
+struct TilePair { float2 lo, hi; };      // the same filter pair of two tiles
+__device__ __forceinline__ TilePair mma_16x8x8(uint32_t a0, uint32_t a1, uint32_t b) {
+  TilePair d;
   asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%7, %7, %7, %7};"
-               : "=f"(d0), "=f"(d1), "=f"(d2), "=f"(d3)
-               : "r"(a), "r"(0u), "r"(b), "f"(0.f));
-  return make_float2(d0, d1);
+               : "=f"(d.lo.x), "=f"(d.lo.y), "=f"(d.hi.x), "=f"(d.hi.y)
+               : "r"(a0), "r"(a1), "r"(b), "f"(0.f));
+  return d;
 }
+// 8 rows only: rows 8..15 of A are zero and their results are dropped
+__device__ __forceinline__ float2 mma_8x8x8(uint32_t a, uint32_t b) { return mma_16x8x8(a, 0u, b).lo; }
 #pragma nv_diag_default 550
 
+__device__ __forceinline__ TilePair vmul(float a, TilePair b) { return {xf::vmul(a, b.lo), xf::vmul(a, b.hi)}; }
+__device__ __forceinline__ TilePair vfma(float a, TilePair b, TilePair c) { return {xf::vfma(a, b.lo, c.lo), xf::vfma(a, b.hi, c.hi)}; }
+__device__ __forceinline__ TilePair vadd(TilePair a, TilePair b) { return {xf::vadd(a.lo, b.lo), xf::vadd(a.hi, b.hi)}; }
+__device__ __forceinline__ TilePair vsub(TilePair a, TilePair b) { return {xf::vsub(a.lo, b.lo), xf::vsub(a.hi, b.hi)}; }
+
 // z_xi[j] = sum_nu A^T[j][nu] * M[xi][nu] with M[xi][nu] made on the spot from the thread's
-// operands of V and U in shared memory.
-template <int M, bool SYM>
+// operands of V and U in shared memory; V is float2 (one tile) or TilePair (tiles 8 apart).
+template <int M, int GT, bool SYM, typename V>
 struct ProductRows {
   static constexpr int N = M + 2;
-  using L = SmallCLayout<M>;
+  using L = SmallCLayout<M, GT>;
   const Coefs& cf;
   uint32_t va, ub;          // shared addresses of this thread's words of V and U at xi = 0, nu = 0
   template <int XI>
-  __device__ __forceinline__ void row(float2 (&z)[M]) const {
-    float2 in[N];
+  __device__ __forceinline__ void row(V (&z)[M]) const {
+    V in[N];
 #pragma unroll
     for (int h = 0; h < N / 2; ++h) {
       const uint2 a = lds_v2<XI * (L::kVBytes / N) + 0>(va + h * 8);
       const uint2 b = lds_v2<XI * (L::kUBytes / N) + 0>(ub + h * 8);
-      in[2 * h] = mma_8x8x8(a.x, b.x);
-      in[2 * h + 1] = mma_8x8x8(a.y, b.y);
+      if constexpr (sizeof(V) == sizeof(TilePair)) {
+        const uint2 a8 = lds_v2<XI * (L::kVBytes / N) + 8 * 4 * N * 4>(va + h * 8);
+        in[2 * h] = mma_16x8x8(a.x, a8.x, b.x);
+        in[2 * h + 1] = mma_16x8x8(a.y, a8.y, b.y);
+      } else {
+        in[2 * h] = mma_8x8x8(a.x, b.x);
+        in[2 * h + 1] = mma_8x8x8(a.y, b.y);
+      }
     }
-    at_apply<M, SYM, float2, N>(cf, in, z);
+    at_apply<M, SYM, V, N>(cf, in, z);
   }
 };
 
-template <int M, bool SYM>
+template <int M, int GT, bool SYM>
 __global__ void __launch_bounds__(kThreads, 1)
 fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ CUtensorMap tmX,
                      const uint32_t* __restrict__ U, __half* __restrict__ y, int H, int W, int K, int Th, int Tw,
                      long long P, int num_kb, int relu, int* __restrict__ status) {
-  using L = SmallCLayout<M>;
-  constexpr int N = L::N;
+  using L = SmallCLayout<M, GT>;
+  constexpr int N = L::N, kGroupTiles = L::kGroupTiles, kStoreLanes = L::kStoreLanes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
   uint32_t* Us = reinterpret_cast<uint32_t*>(smem + L::kOffU);
@@ -198,20 +219,44 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
     uint32_t it = 0;
     for (long long grp = cta; grp < groups; grp += ctas, ++it) {
       if (!mbar_poll(v_full, it & 1, abort_flag)) { *abort_flag = 1; break; }
-      float2 Y[M][M];
-      const ProductRows<M, SYM> rows{cf, va0, ub0};
-      accumulate_rows<M, SYM, float2, N>(cf, rows, Y);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(v_free);
-      // the copies of the previous group must have read the image before it is overwritten
-      if (!mbar_wait(y_free, (it & 1) ^ 1, abort_flag)) { *abort_flag = 1; break; }
       // rounded to half, then the ReLU (NaN and +inf pass)
-      uint8_t* dst = Ys + g * L::kYTile + warp * 16 + t * 4;
+      auto put = [&](uint8_t* dst, const float2& v, int i, int j) {
+        *reinterpret_cast<__half2*>(dst + (i * M + j) * 128) = __hmax2_nan(__floats2half2_rn(v.x, v.y), lo2);
+      };
+      bool ok = true;
+      if constexpr (kGroupTiles == 8) {
+        float2 Y[M][M];
+        accumulate_rows<M, SYM, float2, N>(cf, ProductRows<M, GT, SYM, float2>{cf, va0, ub0}, Y);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(v_free);
+        // the copies of the previous group must have read the image before it is overwritten
+        ok = mbar_wait(y_free, (it & 1) ^ 1, abort_flag);
+        uint8_t* dst = Ys + g * L::kYTile + warp * 16 + t * 4;
 #pragma unroll
-      for (int i = 0; i < M; ++i)
+        for (int i = 0; i < M; ++i)
 #pragma unroll
-        for (int j = 0; j < M; ++j)
-          *reinterpret_cast<__half2*>(dst + (i * M + j) * 128) = __hmax2_nan(__floats2half2_rn(Y[i][j].x, Y[i][j].y), lo2);
+          for (int j = 0; j < M; ++j) put(dst, Y[i][j], i, j);
+      } else {
+#pragma unroll 1
+        for (int s = 0; s < kGroupTiles / 16; ++s) {
+          TilePair Y[M][M];
+          accumulate_rows<M, SYM, TilePair, N>(cf, ProductRows<M, GT, SYM, TilePair>{cf, va0 + (uint32_t)(s * 16 * 4 * N * 4), ub0}, Y);
+          if (s == kGroupTiles / 16 - 1) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(v_free);
+          }
+          if (s == 0) ok = mbar_wait(y_free, (it & 1) ^ 1, abort_flag);
+          uint8_t* dst = Ys + (s * 16 + g) * L::kYTile + warp * 16 + t * 4;
+#pragma unroll
+          for (int i = 0; i < M; ++i)
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+              put(dst, Y[i][j].lo, i, j);
+              put(dst + 8 * L::kYTile, Y[i][j].hi, i, j);
+            }
+        }
+      }
+      if (!ok) { *abort_flag = 1; break; }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the bulk copies read these writes
       __syncwarp();
       if (lane == 0) mbar_arrive(y_full);
@@ -221,7 +266,7 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs));
     const int ht = tid - kProductWarps * 32;                 // 0 .. 127
     const int k_here = min(kFilterBlock, K - kb * kFilterBlock);      // filters of this block that exist
-    // Lanes 0 and 1 of every helper warp, one tile each (tile 2 hw + lane of the group): the tile's box
+    // The first lanes of every helper warp, one tile each (two with 8 tiles: tile 2 hw + lane): the tile's box
     // into the patch buffer and its output record into record set `set`.  Tiles past the end are not
     // fetched and get an empty record.  (Eight lanes of one warp took 1 500 cycles over it, on the
     // critical path of that warp.)
@@ -301,7 +346,7 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
       if (!mbar_poll(v_free, (it & 1) ^ 1, abort_flag)) *abort_flag = 1;   // on the critical path
       // ---- pass 2: V[xi][nu] = sum_b T[xi][b] B^T[nu][b], rounded to half
       for (int item = ht; item < kGroupTiles * N * 4; item += kHelperWarps * 32) {
-        const int cp = item & 3, tl = (item >> 2) & (kGroupTiles - 1), xi = item >> 5;
+        const int cp = item & 3, tl = (item >> 2) & (kGroupTiles - 1), xi = item / (4 * kGroupTiles);
         const float2* src = reinterpret_cast<const float2*>(Ts + tl * L::kTTile) + xi * N * 4 + cp;
         float2 d[N], o[N];
 #pragma unroll
@@ -329,9 +374,9 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
   if (*abort_flag && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
 }
 
-template <int M, bool SYM>
+template <int M, int GT, bool SYM>
 int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, cudaStream_t stream) {
-  using L = SmallCLayout<M>;
+  using L = SmallCLayout<M, GT>;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return (int)cudaErrorUnknown;
   CUtensorMap tmX;
@@ -343,13 +388,13 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return (int)cudaErrorUnknown;
-  if (cudaError_t e = allow_dynamic_smem(fused_small_c_kernel<M, SYM>, L::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem(fused_small_c_kernel<M, GT, SYM>, L::kTotal); e != cudaSuccess) return (int)e;
   const int num_kb = (g.K + kFilterBlock - 1) / kFilterBlock;
-  const long long groups = (g.P + kGroupTiles - 1) / kGroupTiles;
+  const long long groups = (g.P + L::kGroupTiles - 1) / L::kGroupTiles;
   long long per_kb = plan->sm_count / num_kb;
   if (per_kb < 1) per_kb = 1;
   if (per_kb > groups) per_kb = groups;
-  return (int)launch_overlapped(fused_small_c_kernel<M, SYM>, (int)(per_kb * num_kb), kThreads, L::kTotal, stream,
+  return (int)launch_overlapped(fused_small_c_kernel<M, GT, SYM>, (int)(per_kb * num_kb), kThreads, L::kTotal, stream,
                                 plan->kcoefs, tmX, (const uint32_t*)U, (__half*)y, g.H, g.W, g.K, g.Th, g.Tw, g.P, num_kb,
                                 relu, plan->status_dev);
 }
@@ -360,14 +405,25 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
 // Tile indices are 32-bit in the kernel: larger problems stay on the three-kernel path.
 bool fused_small_c_applies(const nova_plan* plan, const Geom& g) {
   return plan->mode == NOVA_FP16_F32ACC && plan->r == 3 && g.C == 8 && plan->status_dev != nullptr &&
-         g.P < ((long long)1 << 31) - kGroupTiles;
+         g.P < ((long long)1 << 31) - 64;
 }
 
 int launch_fused_small_c(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu,
                          void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-#define NOVA_SMALLC(MV)                                                       \
-  return plan->symmetric ? go<MV, true>(plan, g, x, U, y, relu, s) : go<MV, false>(plan, g, x, U, y, relu, s)
+  // Large or small groups by rounds of groups x time per group (a large one takes 3.1, 2.8, 1.75 times a small one's
+  // 3100, 3800, 5400 cycles at m = 2, 4, 6; below four rounds what counts is the time through one group: 224 x 224, 8 -> 64,
+  // F(4,3) 8.2 us large, 7.4 small).  Small groups against this rule: F(2,3) 32 x 224 x 224, 8 -> 64: 548 -> 213 us,
+  // 8 x 56 x 56, 8 -> 136: 37.6 -> 13.3; F(4,3) 171 -> 121, 16.2 -> 10.9; F(6,3) 110 -> 99 (8 x 56 x 56: 16 us, 19 with large).
+  const long long ctas = plan->sm_count / ((g.K + kFilterBlock - 1) / kFilterBlock);
+  auto rounds = [&](long long tiles) { const long long n = (g.P + tiles - 1) / tiles; return ctas > 0 ? (n + ctas - 1) / ctas : n; };
+  const long long weight = plan->m == 2 ? 310 : plan->m == 4 ? 280 : 175;
+  const bool large = rounds(8) >= 4 && rounds(large_group(plan->m)) * weight < rounds(8) * 100;
+#define NOVA_SMALLC(MV)                                                                                                \
+  if (large)                                                                                                           \
+    return plan->symmetric ? go<MV, large_group(MV), true>(plan, g, x, U, y, relu, s)                                  \
+                           : go<MV, large_group(MV), false>(plan, g, x, U, y, relu, s);                                \
+  return plan->symmetric ? go<MV, 8, true>(plan, g, x, U, y, relu, s) : go<MV, 8, false>(plan, g, x, U, y, relu, s)
   switch (plan->m) {
     case 2: NOVA_SMALLC(2);
     case 4: NOVA_SMALLC(4);

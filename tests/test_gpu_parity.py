@@ -1048,6 +1048,25 @@ def test_eight_channel_layers_run_in_one_kernel_and_match_the_emulation(kind, m,
     assert whole <= EMU_CLOSE and tile <= EMU_CLOSE_TILE, (whole, tile)
 
 
+@pytest.mark.parametrize("kind,m,N", [("std", 2, 1), ("asym", 2, 1), ("nova", 4, 1), ("asym", 4, 1), ("half", 6, 4),
+                                      ("asym", 6, 4)])
+def test_one_kernel_path_in_large_groups_matches_the_three_kernels(kind, m, N):
+    # Nine filter blocks leave 16 CTAs each, so that groups of 64, 32 and 16 tiles are taken (m = 2, 4, 6); the last group
+    # and the last filter block are ragged, and so are the tiles.  Judged against the three kernels, the same roundings
+    # with sums in another order.  Per tile the bound is twice EMU_CLOSE_TILE: either side may be that far from the
+    # emulation (triangle inequality), and a flipped rounding of one V reaches every output of its tile.
+    H, W, C, K = 81, 85, 8, 520
+    x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=305 + m)
+    pts = point_set(kind, m)
+    y, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, flags=nv.RELU)
+    y3, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, flags=nv.RELU | nv.GEMM_TCGEN05)
+    xd, gd = torch.from_numpy(x).cuda().double().permute(0, 3, 1, 2), torch.from_numpy(g).cuda().double().permute(0, 3, 1, 2)
+    y1 = torch.nn.functional.conv2d(xd, gd, padding=1).relu().permute(0, 2, 3, 1).cpu().numpy()
+    assert np.isfinite(y.astype(np.float32)).all()
+    whole, tile = closeness(y, y3, y1, m)
+    assert whole <= EMU_CLOSE and tile <= 2 * EMU_CLOSE_TILE, (whole, tile)
+
+
 def test_one_kernel_path_passes_nan_and_inf_through_relu_like_the_three_kernel_path():
     m, N, H, W, C, K = 4, 1, 12, 12, 8, 64
     x, g = make_conv_inputs(N, H, W, C, K, "fp16", False, True, seed=311)
