@@ -192,6 +192,7 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
   const int my_chunks = (args.chunks - (int)rank + split - 1) / split;
   const int f_run = 8 * args.nb * Cfg::NH;
 
+  if (threadIdx.x == 32) { tma_prefetch(&tmX); tma_prefetch(&tmU); }
   if (threadIdx.x == 0) {
     for (int i = 0; i < ST; ++i) { mbar_init(&u_full[i], 1); mbar_init(&u_free[i], Cfg::kProductWarps); }
     mbar_init(x_full, 1);

@@ -177,6 +177,7 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
   const int cta = blockIdx.x / num_kb, ctas = gridDim.x / num_kb;
   const long long groups = (P + kGroupTiles - 1) / kGroupTiles;
 
+  if (tid == 32) tma_prefetch(&tmX);
   if (tid == 0) {
     mbar_init(patch_full, 1);
     mbar_init(v_full, kHelperWarps);

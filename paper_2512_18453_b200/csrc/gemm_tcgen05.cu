@@ -6,7 +6,7 @@
 // Persistent, warp-specialised kernel.  One CTA per SM walks a list of work
 // items (f, 128-row block of tiles p, BLOCK_N-wide block of filters k; the filter blocks of a (f, p) pair one after the other):
 //   warp 0    TMA producer: 128B-swizzled [rows][64 channels] boxes of V and U
-//             into a 4-stage shared-memory ring, completion on mbarriers;
+//             into a shared-memory ring of 3 to 8 stages, completion on mbarriers;
 //   warp 1    issues tcgen05.mma (kind::f16, M=128, N=BLOCK_N, K=16) from
 //             shared-memory descriptors into one of two TMEM accumulators;
 //   warps 2-9 epilogue, warps 2-5 for the first half of the columns and warps
@@ -16,6 +16,13 @@
 //             MMAs on the other accumulator.  M is laid out
 //             [f][K/4][pc_pad][4]: each 16-byte store instruction of a warp
 //             then covers 512 contiguous bytes (32 tiles x 4 filters).
+// A layer of few tiles is bound by the chain from the end of the input transform to the first
+// product, so everything that does not need V happens before the wait for it: the tensor maps, the
+// first item's indices, the barriers' byte counts and the first stages' pieces of U; and the first
+// pieces of V, which one thread would issue one after the other (some 300 cycles each), are issued
+// by one epilogue warp each, in boxes no higher than the tiles there are.  Whole call, before / with
+// all of this: 14 x 14, 512 -> 512, F(4,3) 11.75 / 11.2 us; 28 x 28, 256 -> 512 10.6 / 10.0; 8 images
+// 8 x 8, 32 -> 16 7.35 / 6.67; 2 of 20 x 20, 256 -> 256, F(8,3) 13.7 / 13.0; large layers unchanged.
 // Every wait is bounded; on expiry the kernel records a status and drains.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -59,7 +66,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmU,
                     float* __restrict__ Mo, int nfreq, int pc, int pc_pad, int C, int K,
                     int* __restrict__ status, const uint8_t* __restrict__ Vdrop, int f_major, int spread, int keep_pct,
-                    int kStages, unsigned long long* __restrict__ prof) {
+                    int kStages, int box_rows, unsigned long long* __restrict__ prof) {
   using L = SmemLayout<BLOCK_N>;
   constexpr int BLOCK_K = I8 ? kRowBytes : kRowBytes / 2;   // elements of K per stage
   constexpr uint32_t kTmemCols = 2 * BLOCK_N;       // two accumulators; 128, 256 or 512
@@ -102,11 +109,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     else { pb = num_pb - 1 - (int)(pair / (unsigned)nfreq); f = (int)(pair % (unsigned)nfreq); }
   };
 
+  // The first item's first stages are armed here, before any warp can load into them: warp 0 fetches
+  // their pieces of U before the wait for the input transform, one epilogue warp each their pieces of V after it.
+  const uint32_t stage_tx = (uint32_t)(box_rows * kRowBytes + L::kBBytes);
+  const int early = n_local > 0 ? (num_ks < kStages ? num_ks : kStages) : 0;
+  if (threadIdx.x == 64) { tma_prefetch(&tmU); tma_prefetch(&tmV); }
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(&tmem_full[a], 1); mbar_init(&tmem_empty[a], 8); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int ks = 0; ks < early; ++ks) mbar_expect_tx(&full_bar[ks], stage_tx);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -129,35 +142,33 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     // The first stages' pieces of U do not wait for the input transform, which lets this kernel
     // start only once everything before the transform itself has completed (it releases its
     // dependents after its own wait): U is final by then.
-    const int early = n_local > 0 ? (num_ks < kStages ? num_ks : kStages) : 0;
+    int pb = 0, f = 0, kb = 0;
+    if (early > 0) item_of(0, pb, f, kb);
     if (lane == 0 && early > 0) {
-      int pb, f, kb;
-      item_of(0, pb, f, kb);
-      for (int ks = 0; ks < early; ++ks) {
-        mbar_expect_tx(&full_bar[ks], L::kStageBytes);
+      for (int ks = 0; ks < early; ++ks)
         tma_load_3d(smem + ks * L::kStageBytes + L::kABytes, &tmU, &full_bar[ks], ks * BLOCK_K, kb * BLOCK_N, f);
-      }
     }
     pdl_wait();
     total.start();
     uint32_t stage = 0, phase = 0;
     for (uint32_t local = 0; local < n_local && !timed_out; ++local) {
-      int pb, f, kb;
-      item_of(local, pb, f, kb);
+      if (local > 0) item_of(local, pb, f, kb);
       for (int ks = 0; ks < num_ks; ++ks) {
-        w_empty.start();
-        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag)) { timed_out = true; break; }
-        w_empty.stop();
-        if (lane == 0) {
-          uint8_t* sa = smem + stage * L::kStageBytes;
-          uint8_t* sb = sa + L::kABytes;
-          if (local > 0 || ks >= early) {
-            mbar_expect_tx(&full_bar[stage], L::kStageBytes);
+        // The early stages have been loaded without this warp.  It must not ask whether they were
+        // free: they may have been consumed by now, and the parity would name a later phase.
+        if (local > 0 || ks >= early) {
+          w_empty.start();
+          if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag)) { timed_out = true; break; }
+          w_empty.stop();
+          if (lane == 0) {
+            uint8_t* sa = smem + stage * L::kStageBytes;
+            uint8_t* sb = sa + L::kABytes;
+            mbar_expect_tx(&full_bar[stage], stage_tx);
             tma_load_3d(sb, &tmU, &full_bar[stage], ks * BLOCK_K, kb * BLOCK_N, f);
+            tma_load_3d(sa, &tmV, &full_bar[stage], ks * BLOCK_K, pb * BLOCK_M, f);
           }
-          tma_load_3d(sa, &tmV, &full_bar[stage], ks * BLOCK_K, pb * BLOCK_M, f);
+          __syncwarp();
         }
-        __syncwarp();
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
     }
@@ -236,7 +247,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
     const int k4 = K >> 2;
     const int live_rows = (pc + 7) & ~7;
     WaitClock<PROF> w_full, total;
+    int pb0 = 0, f0 = 0, kb0 = 0;
+    if (warp - 2 < early) item_of(0, pb0, f0, kb0);
     pdl_wait();
+    if (warp - 2 < early && lane == 0) {
+      const int ks = warp - 2;
+      tma_load_3d(smem + ks * L::kStageBytes, &tmV, &full_bar[ks], ks * BLOCK_K, pb0 * BLOCK_M, f0);
+    }
+    __syncwarp();
     total.start();
     for (uint32_t local = 0; local < n_local && !timed_out; ++local) {
       int pb, f, kb;
@@ -349,7 +367,8 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
   const CUtensorMapDataType dt = I8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   constexpr int esize = I8 ? 1 : 2;
   constexpr int BLOCK_K = kRowBytes / esize;
-  if (!make_map_3d(&tmV, dt, esize, V, C, pc, (long long)pc_pad * C, nfreq, BLOCK_K, BLOCK_M) ||
+  const int box_rows = pc < BLOCK_M ? (pc + 7) / 8 * 8 : BLOCK_M;
+  if (!make_map_3d(&tmV, dt, esize, V, C, pc, (long long)pc_pad * C, nfreq, BLOCK_K, box_rows) ||
       !make_map_3d(&tmU, dt, esize, U, C, K, (long long)K * C, nfreq, BLOCK_K, BLOCK_N))
     return (int)cudaErrorUnknown;
   const long long pairs = (long long)nfreq * ((pc + BLOCK_M - 1) / BLOCK_M);
@@ -381,11 +400,11 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
       // CTAs beyond this launch's grid must read as "did not run"
       if (cudaError_t e = cudaMemsetAsync(prof, 0, sizeof(unsigned long long) * 8 * sms, stream); e != cudaSuccess) return (int)e;
       return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8, true>, grid, kThreads, smem, stream, tmV, tmU, M,
-                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, prof);
+                                    nfreq, pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, box_rows, prof);
     }
   }
   return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8>, grid, kThreads, smem, stream, tmV, tmU, M, nfreq,
-                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, (unsigned long long*)nullptr);
+                                pc, pc_pad, C, K, status, vdrop, f_major ? 1 : 0, spread ? 1 : 0, keep_pct, stages, box_rows, (unsigned long long*)nullptr);
 }
 
 }  // namespace

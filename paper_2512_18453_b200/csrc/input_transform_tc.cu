@@ -130,6 +130,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
   const unsigned num_units = (num_sub + 1) / 2;
   const uint32_t n_local = num_units > blockIdx.x ? (num_units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
 
+  if (threadIdx.x == 32) { tma_prefetch(&tmKron); tma_prefetch(&tmX); }
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < kNumAcc; ++a) { mbar_init(&tmem_full[a], 1); mbar_init(&tmem_empty[a], 4); }
@@ -162,6 +163,22 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     for (int b = 0; b < 2 * Cfg::KA; ++b)
       tma_load_2d(kron + (size_t)b * Cfg::NFP * 128, &tmKron, kron_bar, 0, b * Cfg::NFP);
   }
+  // A producer's unit: its channel blocks, tile positions and images.  The divisions for the first unit
+  // come before the wait for the preceding kernel, those for the others before the wait for the stage.
+  int cb[2], tw[2], th[2], img[2], halves = 0;
+  auto locate = [&](uint32_t local) {
+    const unsigned u = blockIdx.x + local * gridDim.x;
+    halves = 2 * u + 1 < num_sub ? 2 : 1;                  // the last unit of an odd count has one half
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned sidx = 2 * u + h, pl = sidx / CB64, p = (unsigned)p0 + pl, q = p / (unsigned)Tw, im = q / (unsigned)Th;
+      cb[h] = (int)(sidx - pl * CB64);
+      tw[h] = (int)(p - q * (unsigned)Tw);
+      th[h] = (int)(q - im * (unsigned)Th);
+      img[h] = (int)im;
+    }
+  };
+  if (warp < kProdWarps) locate(warp);
   // The product kernel may be scheduled from here on; it relies on everything before this kernel
   // having completed by then (it fetches U before its own wait), hence after the wait.
   pdl_wait();
@@ -170,21 +187,16 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
   if (warp < kProdWarps) {
     // ---------------- TMA producers
     for (uint32_t local = warp; local < n_local && !timed_out; local += kProdWarps) {
-      const unsigned u = blockIdx.x + local * gridDim.x;
       const uint32_t stage = local % kStages, phase = (local / kStages) & 1;
+      if (local != (uint32_t)warp) locate(local);
       if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, abort_flag)) { timed_out = true; break; }
       if (lane == 0) {
         uint8_t* dst = ring + (size_t)stage * Cfg::kStageBytes;
-        const int halves = 2 * u + 1 < num_sub ? 2 : 1;      // the last unit of an odd count has one half
         mbar_expect_tx(&full_bar[stage], halves * Cfg::NF * 128);
-        for (int h = 0; h < halves; ++h) {
-          const unsigned sidx = 2 * u + h;
-          const int cb = (int)(sidx % CB64);
-          const unsigned p = (unsigned)p0 + sidx / CB64;
-          const int tw = (int)(p % (unsigned)Tw), th = (int)((p / (unsigned)Tw) % (unsigned)Th);
-          const int img = (int)(p / ((unsigned)Tw * (unsigned)Th));
-          tma_load_4d(dst + h * Cfg::kHalfBytes, &tmX, &full_bar[stage], cb * 64, M * tw - Cfg::PAD, M * th - Cfg::PAD, img);
-        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (h < halves)
+            tma_load_4d(dst + h * Cfg::kHalfBytes, &tmX, &full_bar[stage], cb[h] * 64, M * tw[h] - Cfg::PAD, M * th[h] - Cfg::PAD, img[h]);
       }
       __syncwarp();
     }

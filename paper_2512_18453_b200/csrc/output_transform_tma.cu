@@ -73,6 +73,7 @@ output_transform_tma_kernel(const __grid_constant__ CUtensorMap tmM, const __gri
   const unsigned num_units = (unsigned)TG * (unsigned)KG;
   const uint32_t n_local = num_units > blockIdx.x ? (num_units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
 
+  if (threadIdx.x == 32) tma_prefetch(&tmM);
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 4); }
     *abort_flag = 0;

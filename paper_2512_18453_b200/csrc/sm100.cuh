@@ -97,6 +97,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   return mbar_wait(bar, parity, abort_flag);
 }
 
+// Fetch a tensor map ahead of its first use, which would otherwise wait for it.  A kernel parameter
+// may be fetched before the wait for the preceding kernel.
+__device__ __forceinline__ void tma_prefetch(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
                                             int y, int z) {
   asm volatile(

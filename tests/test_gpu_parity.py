@@ -395,6 +395,27 @@ def test_product_work_splits_match_the_cuda_core_product(kind, m, shape):
     assert conv.rel_l2(ya, yb) < 0.05 * conv.rel_l2(yb, conv.direct_conv_fp64(x, g)) + 2.0 ** -13
 
 
+@pytest.mark.parametrize("kind,m,shape", [
+    ("nova", 4, (1, 3, 2, 8, 16)),          # one tile, one stage: boxes of 8 rows
+    ("nova", 4, (1, 32, 16, 520, 64)),      # 32 tiles, 9 pieces of 64 channels: one more than the ring has stages
+    ("nova", 4, (1, 508, 4, 136, 264)),     # 127 tiles: boxes of 128 rows, the last of them zero
+    ("std", 2, (2, 16, 16, 512, 304)),      # 128 tiles, 8 pieces in a ring of 3 or 4 stages
+    ("nova", 6, (1, 258, 18, 264, 512))])   # 129 tiles: a second row block of one tile
+def test_product_first_loads_match_the_cuda_core_product(kind, m, shape):
+    # the first item's loads are issued by other warps than the rest, in boxes of the tiles there are; the bound
+    # is that of the work splits above, and repeated calls give the same bits
+    N, H, W, C, K = shape
+    x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=485 + m)
+    pts = point_set(kind, m)
+    ya, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, nv.GEMM_TCGEN05)
+    yb, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, nv.GEMM_SIMT)
+    assert np.isfinite(ya.astype(np.float32)).all()
+    assert conv.rel_l2(ya, yb) < 0.05 * conv.rel_l2(yb, conv.direct_conv_fp64(x, g)) + 2.0 ** -13
+    for _ in range(3):
+        yc, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, nv.GEMM_TCGEN05)
+        assert np.array_equal(ya.view(np.int16), yc.view(np.int16))
+
+
 def test_gpu_is_close_to_emulation_elementwise():
     x, g = make_conv_inputs(2, 24, 24, 64, 64, "fp16", True, True, seed=410)
     pts = point_set("nova", 4)
