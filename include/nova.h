@@ -233,7 +233,9 @@ int nova_conv2d_fwd(const nova_plan* plan, const void* x_dev, const void* U_dev,
  * on `stream` around each kernel; synchronises the stream and writes the summed
  * device time in milliseconds of the three kernel classes to kernel_ms_host[0..2]
  * (input transform, transformed-domain product, output transform); the one-kernel
- * path of C = 8 reports its time as the product's and 0 for the transforms.
+ * paths (C = 8 in half mode; fp32 mode with up to 8 points) report their time as the
+ * product's and 0 for the transforms, and where product and output transform are one
+ * kernel its time is the product's.
  */
 int nova_conv2d_fwd_timed(const nova_plan* plan, const void* x_dev, const void* U_dev, void* y_dev,
                           int N, int H, int W, int C, int K,

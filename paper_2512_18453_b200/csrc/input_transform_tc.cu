@@ -8,7 +8,11 @@
 // stores it as hi + lo (two half matrices, hi = fl16(prod), lo = fl16(prod - hi)) and the
 // kernel issues the MMAs of both into the same accumulator: the result is the float
 // accumulation of exact products of the rounded coefficients with the inputs, i.e. the
-// same quantity the CUDA-core transform evaluates, in a different summation order.
+// same quantity the CUDA-core transform evaluates, in a different summation order.  Where all
+// products of a point set are exact in half (0, +-1, +-2; or 0, +-1/2, +-1, +-2), lo is zero and its MMAs are
+// left out.  Whole call, with / without them, F(6,3): 8 x 56 x 56, 64 -> 64 14.9 / 14.5 us; 32 x 112 x 112,
+// 128 -> 128 206 / 201; 32 x 224 x 224, 64 -> 64 357 / 354.  (Leaving out single slabs of 16 columns for the
+// other sets was slower: the loop over a mask costs more than the one or two MMAs it saves.)
 //
 // One work unit = two (tile, block of 64 channels) pairs, one per half of the 128 TMEM lanes; the
 // pairs are numbered tile-major, so a unit is a tile's two neighbouring channel blocks when C is a
@@ -94,7 +98,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
 // pass's qparts / 127 where qgiven is 0, and is left in *qslot for the output transform.  (A cleared
 // word, atomics and a kernel that made the scale of it were two more launches per call, and neither
 // could overlap its neighbours.)
-template <int M, int QMODE, int R = 3>
+// LO: the table has a part lo (see above).  A variant, not a branch: the issue of a unit's MMAs is straight-line code.
+template <int M, int QMODE, int R, bool LO>
 __global__ void __launch_bounds__(kTcThreads, 1)
 input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmKron,
                           void* __restrict__ Vout, int C, int Th, int Tw, long long p0, int pc, int pc_pad,
@@ -159,8 +164,9 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
   // the constant Kronecker table belongs to the plan: it may be fetched while the preceding
   // kernel of the stream is still draining; everything else waits for that kernel
   if (warp == 0 && lane == 0) {
-    mbar_expect_tx(kron_bar, Cfg::kKronBytes);
-    for (int b = 0; b < 2 * Cfg::KA; ++b)
+    constexpr int parts = LO ? 2 : 1;
+    mbar_expect_tx(kron_bar, parts * (Cfg::kKronBytes / 2));
+    for (int b = 0; b < parts * Cfg::KA; ++b)
       tma_load_2d(kron + (size_t)b * Cfg::NFP * 128, &tmKron, kron_bar, 0, b * Cfg::NFP);
   }
   // A producer's unit: its channel blocks, tile positions and images.  The divisions for the first unit
@@ -214,9 +220,9 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
       if (lane == 0) {
         const uint32_t sa = smem_u32(ring + (size_t)stage * Cfg::kStageBytes);
         const uint32_t tmem_d = tmem_base + acc * kAccCols;
-const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
+        const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);
 #pragma unroll
-        for (int hl = 0; hl < 2; ++hl)
+        for (int hl = 0; hl < (LO ? 2 : 1); ++hl)
 #pragma unroll
           for (int ks = 0; ks < Cfg::KP / 16; ++ks) {
             const uint64_t ad = umma_desc_advance(ad0, ks * 2048);
@@ -334,7 +340,8 @@ template <int M, int QMODE, int R = 3>
 int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0, int pc, int pc_pad,
              float* qslot, float* qparts, float qgiven, cudaStream_t stream) {
   using Cfg = TcCfg<M, R>;
-  if (cudaError_t e = allow_dynamic_smem(input_transform_tc_kernel<M, QMODE, R>, Cfg::kTotal); e != cudaSuccess) return (int)e;
+  const auto kernel = plan->kron_lo ? input_transform_tc_kernel<M, QMODE, R, true> : input_transform_tc_kernel<M, QMODE, R, false>;
+  if (cudaError_t e = allow_dynamic_smem(kernel, Cfg::kTotal); e != cudaSuccess) return (int)e;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return (int)cudaErrorUnknown;
   CUtensorMap tmX, tmK;
@@ -361,7 +368,7 @@ int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long 
   const int sms = plan->sm_count;
   const long long units = ((long long)pc * ((g.C + 63) / 64) + 1) / 2;   // two (tile, 64-channel block) pairs each
   const int grid = (int)(units < sms ? units : sms);
-  return (int)launch_overlapped(input_transform_tc_kernel<M, QMODE, R>, grid, kTcThreads, Cfg::kTotal, stream, tmX, tmK,
+  return (int)launch_overlapped(kernel, grid, kTcThreads, Cfg::kTotal, stream, tmX, tmK,
                                 V, g.C, g.Th, g.Tw, p0, pc, pc_pad, plan->status_dev, qslot, qparts, qgiven);
 }
 
@@ -372,9 +379,11 @@ size_t kron_table_halves(int n) {
   return (size_t)2 * ka * kp * 64;
 }
 
-// Host image of the device table: [hi|lo][K atom][frequency row, padded][64 halves].
-void build_kron_table(const nova_plan* plan, unsigned short* out) {
+// Host image of the device table: [hi|lo][K atom][frequency row, padded][64 halves].  Returns whether
+// its lo part holds anything but zeros.
+int build_kron_table(const nova_plan* plan, unsigned short* out) {
   const int n = plan->n, nf = n * n, kp = (nf + 15) / 16 * 16, ka = (kp + 63) / 64;
+  int used = 0;
   for (size_t i = 0; i < kron_table_halves(plan->n); ++i) out[i] = 0;
   for (int xi = 0; xi < n; ++xi)
     for (int nu = 0; nu < n; ++nu)
@@ -389,7 +398,9 @@ void build_kron_table(const nova_plan* plan, unsigned short* out) {
           const size_t at = ((size_t)(k / 64) * kp + f) * 64 + (k % 64);
           out[at] = __half_as_ushort(hi);
           out[(size_t)ka * kp * 64 + at] = __half_as_ushort(lo);
+          if (__half_as_ushort(lo) & 0x7fff) used = 1;
         }
+  return used;
 }
 
 int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0,

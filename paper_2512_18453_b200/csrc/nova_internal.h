@@ -55,6 +55,7 @@ struct nova_plan {
   int sm_count;                           // multiprocessors of that device
   int l2_bytes;                           // size of its L2
   unsigned long long* prof_dev;           // 8 wait counters per multiprocessor (NOVA_PROFILE_WAITS; may be null)
+  int kron_lo;                            // kron_dev's lo part is not all zero
 };
 
 namespace nova {
@@ -85,7 +86,7 @@ int launch_input_transform_n4(const nova_plan* plan, const Geom& g, const void* 
 int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* x, void* V,
                               long long p0, int pc, int pc_pad, void* stream);
 size_t kron_table_halves(int n);   // n points
-void build_kron_table(const nova_plan* plan, unsigned short* out);
+int build_kron_table(const nova_plan* plan, unsigned short* out);   // returns kron_lo
 int launch_output_transform(const nova_plan* plan, const Geom& g, const void* M, void* y,
                             long long p0, int pc, int pc_pad, int relu, void* stream);
 // scale_U / scale_V non-null: M holds int32 sums of the int8 pipeline, dequantised on load
