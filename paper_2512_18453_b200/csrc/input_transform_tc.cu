@@ -379,27 +379,34 @@ size_t kron_table_halves(int n) {
   return (size_t)2 * ka * kp * 64;
 }
 
-// Host image of the device table: [hi|lo][K atom][frequency row, padded][64 halves].  Returns whether
-// its lo part holds anything but zeros.
+// Host image of the device table: [hi|lo][K atom][frequency row, padded][64 halves].  Returns whether its lo part
+// holds anything but zeros, or -1 where hi + lo does not stand for the products: one of them beyond half's range (hi
+// would be infinite, and infinity times a zero of the patch is NaN), or a row so far down in half's range that its
+// step of 2^-24 shows.  2^-16 of the row's largest product is a sixteenth of what rounding V to half costs.
 int build_kron_table(const nova_plan* plan, unsigned short* out) {
   const int n = plan->n, nf = n * n, kp = (nf + 15) / 16 * 16, ka = (kp + 63) / 64;
   int used = 0;
   for (size_t i = 0; i < kron_table_halves(plan->n); ++i) out[i] = 0;
   for (int xi = 0; xi < n; ++xi)
-    for (int nu = 0; nu < n; ++nu)
+    for (int nu = 0; nu < n; ++nu) {
+      double largest = 0.0, missed = 0.0;
       for (int a = 0; a < n; ++a)
         for (int b = 0; b < n; ++b) {
           const int f = xi * n + nu, k = a * n + b;
           const double prod = (double)plan->kcoefs.BT[xi][a] * (double)plan->kcoefs.BT[nu][b];
           const __half hi = __double2half(prod);
           const double hid = (double)__half2float(hi);
-          __half lo = __float2half(0.f);
-          if (hid - hid == 0.0) lo = __double2half(prod - hid);      // hi finite
+          if (!(hid - hid == 0.0)) return -1;                        // hi is not finite
+          const __half lo = __double2half(prod - hid);
+          largest = fmax(largest, fabs(prod));
+          missed = fmax(missed, fabs(prod - hid - (double)__half2float(lo)));
           const size_t at = ((size_t)(k / 64) * kp + f) * 64 + (k % 64);
           out[at] = __half_as_ushort(hi);
           out[(size_t)ka * kp * 64 + at] = __half_as_ushort(lo);
           if (__half_as_ushort(lo) & 0x7fff) used = 1;
         }
+      if (missed * 65536.0 > largest) return -1;
+    }
   return used;
 }
 

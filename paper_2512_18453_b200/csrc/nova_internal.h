@@ -49,7 +49,7 @@ struct nova_plan {
   nova::CoefsD kcoefs_d;                  // B^T and A^T of kcoefs
   int perm[nova::kMaxN];
   int symmetric;
-  void* kron_dev;                         // device table of the tensor-core input transform (may be null)
+  void* kron_dev;                         // device table of the tensor-core input transform (null where half cannot hold it)
   int* status_dev;                        // device status word (null without a device)
   int device;                             // device that owns status_dev
   int sm_count;                           // multiprocessors of that device
@@ -86,7 +86,7 @@ int launch_input_transform_n4(const nova_plan* plan, const Geom& g, const void* 
 int launch_input_transform_tc(const nova_plan* plan, const Geom& g, const void* x, void* V,
                               long long p0, int pc, int pc_pad, void* stream);
 size_t kron_table_halves(int n);   // n points
-int build_kron_table(const nova_plan* plan, unsigned short* out);   // returns kron_lo
+int build_kron_table(const nova_plan* plan, unsigned short* out);   // returns kron_lo, or -1: no table
 int launch_output_transform(const nova_plan* plan, const Geom& g, const void* M, void* y,
                             long long p0, int pc, int pc_pad, int relu, void* stream);
 // scale_U / scale_V non-null: M holds int32 sums of the int8 pipeline, dequantised on load

@@ -696,6 +696,19 @@ def test_unpaired_scales_take_the_dense_transforms_and_stay_correct():
     check_fp16(y, x, g, 6, pts, scales=(sg, sb))
 
 
+@pytest.mark.parametrize("C", [16, 48, 72])
+@pytest.mark.parametrize("e", [9, -6])
+def test_scales_whose_coefficient_products_do_not_fit_half(e, C):
+    # Every row of B^T times 2^e (A^T undoes it), the input times 2^-e: with e = 9 products of two coefficients pass
+    # 65504, with e = -6 they are so small that half's smallest step shows, while V and y stay in range
+    m, pts = 4, point_set("nova", 4)
+    x, g = make_conv_inputs(2, 21, 18, C, 40, "fp16", True, True, seed=330 + C)
+    x = (x.astype(np.float32) * 2.0 ** -e).astype(np.float16)
+    sc = (None, [(2 ** e, 1) if e > 0 else (1, 2 ** -e)] * len(pts))
+    y, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, scales=sc)
+    check_fp16(y, x, g, m, pts, scales=sc)
+
+
 # ---------------------------------------------------------------- INT8 Winograd-domain pipeline
 def gpu_conv_int8(x, g, m, pts, quant=nv.QUANT_PER_TENSOR, scale_U=None, scale_V=0.0, flags=0, coef=nv.COEF_FP32,
                   scales=(None, None)):
