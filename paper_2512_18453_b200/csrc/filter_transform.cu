@@ -3,9 +3,8 @@
 //
 // What bounds it: the stores of U, n*n / (R*R) times the bytes of g.  A thread owns one filter, four consecutive
 // channels (eight-byte accesses, a warp's store 256 contiguous bytes) and two rows of the n x n frequencies, so that
-// a small layer still spreads over the SMs; the threads that share a filter's taps find them in the L1 or L2 (F(4,5),
-// 512 x 512: 12.6 us with two rows, 13.6 with half of the rows per thread).  Launched as a programmatic dependent: a
-// plain launch costs the host up to twice as much and nothing of it overlaps.
+// a small layer still spreads over the SMs, or all rows, so that the taps of a large one are read once (see the launcher).
+// Launched as a programmatic dependent: a plain launch costs the host up to twice as much and nothing of it overlaps.
 // Against one thread per channel pair and whole filter, launched plainly: F(6,3) 512 x 512 (38 MB) 7.5 -> 7.2 us back to
 // back, 64 x 64 3.4 -> 2.1; F(8,3) 512 x 512 (57 MB) 10.9 -> 9.9; per call 11.2 -> 6.0 us wherever the host is the bound.
 #include <cuda_fp16.h>
@@ -22,7 +21,7 @@ using namespace xf;
 
 constexpr int kFtThreads = 256;
 
-template <int N, int R>
+template <int N, int R, int ROWS>
 __global__ void __launch_bounds__(kFtThreads)
 filter_transform_half_kernel(const __grid_constant__ Coefs cf, const __half* __restrict__ g, __half* __restrict__ U, int K, int C) {
   sm100::pdl_wait();
@@ -43,9 +42,9 @@ filter_transform_half_kernel(const __grid_constant__ Coefs cf, const __half* __r
     }
   const size_t f_stride = (size_t)K * C;
   __half* dst = U + (size_t)k * C + c;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int p = 2 * (int)blockIdx.y + e;
+#pragma unroll 2
+  for (int e = 0; e < ROWS; ++e) {
+    const int p = ROWS * (int)blockIdx.y + e;
     float2 t[2][R];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -71,11 +70,11 @@ filter_transform_half_kernel(const __grid_constant__ Coefs cf, const __half* __r
   }
 }
 
-template <int N, int R>
-int go(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
+template <int N, int R, int ROWS>
+int start(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
   const long long work = (long long)K * (C / 4);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / 2);
+  cfg.gridDim = dim3((unsigned)((work + kFtThreads - 1) / kFtThreads), N / ROWS);
   cfg.blockDim = dim3(kFtThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -83,7 +82,15 @@ int go(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return (int)cudaLaunchKernelEx(&cfg, filter_transform_half_kernel<N, R>, plan->kcoefs, (const __half*)g, (__half*)U, K, C);
+  return (int)cudaLaunchKernelEx(&cfg, filter_transform_half_kernel<N, R, ROWS>, plan->kcoefs, (const __half*)g, (__half*)U, K, C);
+}
+
+// All n rows per thread from 2^17 threads on, where they fill the chip by themselves.  Two rows / all rows: 3 x 3, 1024 x
+// 1024: F(2,3) 9.3 / 7.8 us, F(4,3) 19.0 / 15.7, F(6,3) 28.6 / 26.3; 2048 x 2048: F(6,3) 111 / 98, F(6,5) 246 / 215; 1024 x 512:
+// F(6,3) 13.5 / 11.9, F(8,3) 21.5 / 19.1.  Below: 512 x 512 F(6,3) 7.6 / 8.7, F(8,3) 10.3 / 13.5; 64 x 64 F(6,5) 6.5 / 7.8.
+template <int N, int R>
+int go(const nova_plan* plan, const void* g, int K, int C, void* U, cudaStream_t s) {
+  return (long long)K * (C / 4) >= 1 << 17 ? start<N, R, N>(plan, g, K, C, U, s) : start<N, R, 2>(plan, g, K, C, U, s);
 }
 
 }  // namespace

@@ -174,6 +174,19 @@ def test_filter_transform_matches_emulation(kind, m):
     assert (d > 0).mean() < 0.02                # and almost always identical
 
 
+@pytest.mark.parametrize("m,key,r", [(2, ("std", 2), 3), (4, ("nova", 4), 3), (6, ("half", 6), 3), (8, ("nova", 8), 3),
+                                     (2, ("nova", 4), 5), (4, ("asym", 6), 5), (6, ("nova", 8), 5)])
+def test_filter_transform_of_a_large_layer_gives_the_bits_of_its_parts(m, key, r):
+    # 1032 x 520: a thread has a filter's whole transform; 344 of its filters: two rows of it
+    K, C = 1032, 520
+    plan = nv.Plan(m, point_set(*key), r=r)
+    gen = torch.Generator(device="cuda").manual_seed(210 + m)
+    g = torch.randn(K, r, r, C, generator=gen, device="cuda").half()
+    whole = plan.filter_transform(g)
+    parts = torch.cat([plan.filter_transform(g[k:k + 344].contiguous()) for k in range(0, K, 344)], dim=1)
+    assert torch.equal(whole.view(torch.int16), parts.view(torch.int16))
+
+
 # ---------------------------------------------------------------- fp16 mode, both product kernels
 SHAPES16 = [(2, 13, 11, 16, 8), (1, 5, 3, 8, 8), (2, 30, 30, 64, 64), (3, 20, 20, 72, 136), (1, 17, 23, 136, 264)]
 
