@@ -310,10 +310,13 @@ HostPipe* host_pipe() {
 
 // Groups the batch is cut into.  A group costs some 15 us of copy set-up, fewer groups leave more of the first copy
 // in and the last copy out uncovered: T / G + 15 us * G for T, the slower direction's bytes at the 43 GB/s that
-// each direction gets when both run.  Copies alone, 12.8 MB each way: 497, 402, 367, 415, 544 us with 1, 2, 4, 8, 16 groups.
+// each direction gets when both run, but two from 1 MB on, where that model is too careful.  Whole calls by groups, MB
+// each way (us with 1, 2, 3, 4, 6, 8): 0.8 55, 56; 1.2 80, 74, 74; 1.6 90, 79, 81, 87, 101, 112; 3.2 160, 145, 148, 154, 160,
+// 171; 12.8 510, 427, 418, 431, 430, 456; 51 1954, 1537, 1422, 1393, 1380, 1406.  The rule is within 4 % of the best of each;
+// the figures are those of one host's link.
 int host_groups(int N, size_t bytes) {
   const double t = (double)bytes / 43e3;                // us
-  int groups = 1;
+  int groups = bytes >= 1000000 ? 2 : 1;
   while (groups < kHostGroups && t / (groups + 1) + 15.0 * (groups + 1) < t / groups + 15.0 * groups) ++groups;
   return groups < N ? groups : N;
 }

@@ -528,27 +528,49 @@ def test_host_buffer_entry_point():
     assert np.array_equal(yh.numpy(), y_dev)
 
 
-@pytest.mark.parametrize("C", [64, 8])
-def test_host_buffer_entry_point_pipelines_ragged_groups(C):
-    # 11 images: groups of 2, 2, 2, 2, 2, 1 overlap their copies and kernels; two calls in a row reuse
-    # the internal streams and events; the result must be that of the device-resident call, bit for bit
-    # (C = 8: each group runs the one-kernel path)
-    N, H, W, K = 11, 26, 22, 72
-    pts = point_set("nova", 4)
-    plan = nv.Plan(4, pts)
+def host_groups(N, nbytes):
+    """The groups that nova_conv2d_fwd_host cuts a batch into (nbytes: the larger direction), restated."""
+    t, n = nbytes / 43e3, 2 if nbytes >= 1000000 else 1
+    while n < 8 and t / (n + 1) + 15.0 * (n + 1) < t / n + 15.0 * n:
+        n += 1
+    return min(n, N)
+
+
+@pytest.mark.parametrize("N,H,W,C,K,pool,groups", [
+    (11, 26, 22, 64, 72, False, 1),       # stays on the caller's stream
+    (7, 40, 32, 64, 72, False, 2),        # images 4 + 3
+    (11, 80, 64, 64, 72, False, 4),       # 3 + 3 + 3 + 2, workspace and internal streams used in turn
+    (9, 80, 80, 64, 72, False, 4),        # 3 + 3 + 3: the fourth group would be empty
+    (11, 80, 64, 8, 72, False, 4),        # each group runs the one-kernel path
+    (10, 128, 96, 64, 72, True, 5),       # pooled
+    (17, 160, 160, 8, 72, True, 5)])      # 4 + 4 + 4 + 4 + 1
+def test_host_buffer_entry_point_pipelines_ragged_groups(N, H, W, C, K, pool, groups):
+    # Two calls in a row, with new inputs, reuse the internal streams and events, and nothing waits in between; the
+    # result must be that of the device-resident call, bit for bit
+    Ho, Wo = (H // 2, W // 2) if pool else (H, W)
+    assert host_groups(N, 2 * N * max(H * W * C, Ho * Wo * K)) == groups
+    flags = nv.RELU | (nv.POOL2X2 if pool else 0)
+    plan = nv.Plan(4, point_set("nova", 4))
     xs = torch.empty(N, H, W, C, dtype=torch.float16, device="cuda")
-    ys = torch.empty(N, H, W, K, dtype=torch.float16, device="cuda")
+    ys = torch.empty(N, Ho, Wo, K, dtype=torch.float16, device="cuda")
     ws = torch.empty(plan.workspace_bytes(N, H, W, C, K), dtype=torch.uint8, device="cuda")
+    calls = []
     for seed in (461, 462):
-        x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=seed)
-        U = plan.filter_transform(torch.from_numpy(g).cuda())
-        xh = torch.from_numpy(x).pin_memory()
-        yh = torch.full((N, H, W, K), float("nan"), dtype=torch.float16).pin_memory()
-        plan.conv2d_host(xh, U, yh, xs, ys, ws, flags=nv.RELU)
-        torch.cuda.synchronize()
-        y_dev, _, _ = gpu_conv(x, g, 4, pts, nv.FP16_F32ACC, flags=nv.RELU)
-        assert np.array_equal(yh.numpy(), y_dev)
-        assert plan.device_status() == 0
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        xd = torch.randn(N, H, W, C, generator=gen, device="cuda").relu_().half()
+        U = plan.filter_transform((torch.randn(K, 3, 3, C, generator=gen, device="cuda") * 0.05).half())
+        xh = xd.cpu().pin_memory()
+        yh = torch.full((N, Ho, Wo, K), float("nan"), dtype=torch.float16).pin_memory()
+        calls.append((xd, U, xh, yh))
+    torch.cuda.synchronize()
+    for _, U, xh, yh in calls:
+        plan.conv2d_host(xh, U, yh, xs, ys, ws, flags=flags)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0
+    for xd, U, _, yh in calls:
+        y_dev = plan.conv2d(xd, U, flags=flags).cpu()
+        assert torch.isfinite(yh.float()).all()
+        assert torch.equal(yh.view(torch.int16), y_dev.view(torch.int16))
 
 
 # ---------------------------------------------------------------- the workload configurations at full size
