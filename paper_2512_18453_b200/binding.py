@@ -133,16 +133,19 @@ _fastcall = None
 
 def _fast():
     """The CPython extension that makes the hot calls (csrc/fastcall.c), bound to libnova's functions; False
-    where the build had no Python headers, and the calls go through ctypes then."""
+    where the build had no Python headers, and the calls go through ctypes then (as they do without a GPU,
+    to be refused there like any wrong argument)."""
     global _fastcall
     if _fastcall is None:
         L = lib()
+        import torch
+        if not torch.cuda.is_available():
+            return False
         try:
             from . import _fastcall as ext
         except ImportError:
             _fastcall = False
             return False
-        import torch
         torch.cuda.current_stream()                  # initialises CUDA
         get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
         if get is None or dev is None:

@@ -242,3 +242,20 @@ def test_binding_constants_agree_with_the_header():
     assert len(set(flags)) == len(flags) and all(a & b == 0 for i, a in enumerate(flags) for b in flags[i + 1:])
     m = re.search(r"#define\s+NOVA_STATIC_SCRATCH_BYTES\s+\(\(size_t\)(\d+)\s*<<\s*(\d+)\)", text)
     assert m and (int(m.group(1)) << int(m.group(2))) == nv.STATIC_SCRATCH_BYTES
+
+
+def test_tensors_that_are_not_on_a_gpu_are_refused_as_arguments():
+    # with or without a GPU: an AssertionError about the tensor, not an error of CUDA's initialisation
+    torch = pytest.importorskip("torch")
+    plan = nv.Plan(4, point_set("nova", 4))
+    x = torch.zeros(1, 8, 8, 8, dtype=torch.float16)
+    U = torch.zeros(36, 8, 8, dtype=torch.float16)
+    ws = torch.zeros(1024, dtype=torch.uint8)
+    with pytest.raises(AssertionError):
+        plan.conv2d(x, U)
+    with pytest.raises(AssertionError):
+        plan.conv2d(x, U, torch.zeros_like(x), ws)
+    with pytest.raises(AssertionError):
+        plan.filter_transform(torch.zeros(8, 3, 3, 8, dtype=torch.float16))
+    with pytest.raises(AssertionError):
+        plan.conv2d_int8(x, U.to(torch.int8), torch.zeros(8), 0.0, torch.zeros_like(x), ws)
