@@ -75,6 +75,7 @@ struct PoArgs {
   int H, W, C, K, Th, Tw, pc, pc_pad;
   long long p0;
   int F, num_kb, items, clusters, nacc, relu, stages, box_rows;
+  uint32_t none;                       // 0, which the compiler does not know
 };
 
 __device__ __forceinline__ bool test_cluster(uint64_t* bar, uint32_t parity) {
@@ -112,9 +113,12 @@ __device__ __forceinline__ uint32_t peer(uint32_t a, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
-// Relaxed: it says that registers hold what was read, and must not wait for the stores of y before it to be performed.
+// "I have read my exchange buffer", to another CTA.  What orders the reads before it is that it depends on their values
+// (see the finish warps): a store that follows from the arrival cannot be what they saw.  A release at cluster scope
+// would also wait for the stores of y issued before: 32 x 112 x 112, 64 -> 128, F(2,3) 203 -> 282 us, and 241 with one
+// warp per buffer that passes a local arrive on.
 __device__ __forceinline__ void arrive_peer(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
 // 16 bytes to ANOTHER CTA's shared memory (the instruction is not defined for the executing CTA's own), counted on that
 // CTA's barrier when they are there.  (Plain remote stores and one release per slice cost 3 to 4 thousand cycles per
@@ -400,19 +404,21 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
         const int slot = w >> 1, t8 = (w & 1) * 4 + tt;
         const int pl = pb * kRows + (slot * N + (int)rank) * 8 + t8;
         float2 Y[M][M];
+        uint32_t seen = 0;
         const bool mine = slot < my_oct && pl < args.pc && k < args.K;
         if (mine) {
           const uint32_t base = smem_u32(smem + Cfg::kOffZ) + b * Cfg::kBuf +
                                 (uint32_t)(slot * (M * 512) + (fp >> 1) * 128 + ((t8 ^ ((fp >> 1) << 1)) << 4) + (fp & 1) * 8);
           accumulate_rows<M, SYM, float2, N>(cf, ExchangeRows<M, R>{base}, Y);
-          // the sums are complete, hence everything that this warp reads of the buffer is in registers
+          // every value read of the buffer is in a sum of the first or the last row: the arrival below waits for all of
+          // them (args.none is 0; 0 to 2 % of the call)
 #pragma unroll
-          for (int i = 0; i < M; ++i)
+          for (int i = 0; i < M; i += M - 1)
 #pragma unroll
-            for (int j = 0; j < M; ++j) asm volatile("" : "+f"(Y[i][j].x), "+f"(Y[i][j].y));
+            for (int j = 0; j < M; ++j) seen |= __float_as_uint(Y[i][j].x) | __float_as_uint(Y[i][j].y);
         }
-        __syncwarp();
-        if (lane < N) arrive_peer(tell);
+        const bool unread = __any_sync(0xffffffffu, (seen & args.none) != 0u);
+        if (lane < N && !unread) arrive_peer(tell);
         if (mine) {
           const unsigned p = (unsigned)(args.p0 + pl);
           const unsigned tw = p % (unsigned)args.Tw, q2 = p / (unsigned)args.Tw;
@@ -489,6 +495,7 @@ int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void*
   a.clusters = a.items < slots ? a.items : slots;
   a.nacc = 2 * Cfg::N * F <= 512 ? 2 : 1;
   a.relu = relu;
+  a.none = 0;
   a.stages = Cfg::stages(F);
   const int smem = Cfg::total(F);
   if (cudaError_t e = allow_dynamic_smem(kernel, smem); e != cudaSuccess) return (int)e;

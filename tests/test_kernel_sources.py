@@ -1,0 +1,20 @@
+"""Rules of the kernels' hand-overs that no run can show broken, read off the sources (no GPU)."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2512_18453_b200", "csrc")
+SOURCES = sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
+
+
+def code(path):
+    text = open(path).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_no_barrier_arrival_is_relaxed(path):
+    # a relaxed arrival orders nothing that the arriving thread did before it
+    assert "arrive.relaxed" not in code(path)
