@@ -123,7 +123,9 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
+// The barriers below are aligned ones: a warp comes to them as a whole, after stores that only some of its threads did.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void mma884(Dbl2& d, float a, float b) {
@@ -262,6 +264,10 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
           if (nb < args.nb)
             sts_d2(base + (uint32_t)((nu * kTiles + g) * Cfg::F + ((((h * args.nb + nb) * 8) ^ ((g & 3) << 3)) + 2 * t)) * 8, acc[i][nb]);
       };
+      auto product_sync = [] {
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"n"(Cfg::kProductThreads) : "memory");
+      };
       const int kb = (int)(blk % (unsigned)args.num_kb);
       const int fp_log = 31 - __clz(f_run >> 1);
       const int pairs = kTiles * (f_run >> 1);
@@ -274,7 +280,7 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
         for (int i = 0; i < M; ++i) {
           const uint32_t zr = zb + (i & 1) * Cfg::kZRow;
           put_columns(zr, i);
-          asm volatile("bar.sync 1, %0;" ::"n"(Cfg::kProductThreads));
+          product_sync();
           if ((int)threadIdx.x < pairs && k < args.K) {
             const FcRec rt = rc[tl];
             Dbl2 in[N], yv[M];
@@ -288,7 +294,7 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
         // the cluster's CTAs hold the sums of different channels: all rows to shared memory (over the operand
         // buffers, which no one reads any more), then each CTA adds and finishes its share of the outputs
         const uint32_t z0 = smem_u32(smem);
-        asm volatile("bar.sync 1, %0;" ::"n"(Cfg::kProductThreads));
+        product_sync();
 #pragma unroll
         for (int i = 0; i < M; ++i) put_columns(z0 + i * Cfg::kZRow, i);
         cluster_sync();

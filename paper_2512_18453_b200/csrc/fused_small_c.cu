@@ -52,7 +52,10 @@ constexpr int kProductRegs = 216;
 constexpr int kHelperRegs = 72;
 
 // barrier of the helper warps only
-__device__ __forceinline__ void helper_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kHelperWarps * 32) : "memory"); }
+__device__ __forceinline__ void helper_sync() {
+  __syncwarp();                          // an aligned barrier: a warp comes to it as a whole
+  asm volatile("bar.sync 1, %0;" ::"n"(kHelperWarps * 32) : "memory");
+}
 
 // Tiles of a large group.  A group costs some 3000 cycles of hand-overs between the roles whatever it holds, so it is
 // as large as shared memory (and, for the copies of y, 128 helper threads) allow: 64, 32, 16, 8.  The product takes 16 of

@@ -127,7 +127,10 @@ __device__ __forceinline__ void store_peer(uint32_t a, uint32_t bar, float x, fl
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();                          // an aligned barrier: a warp comes to it as a whole
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
@@ -339,6 +342,7 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
         if ((int)(gs & 1) != grp) continue;
         const uint32_t b = gs & 1;
         wait_cluster(&z_free[b], ((gs >> 1) & 1) ^ 1, abort_flag);
+        __syncwarp();                                // the loads of tensor memory are a whole warp's
         if (live) {
 #pragma unroll 1
           for (int fq = 0; fq < 4; ++fq) {
@@ -439,7 +443,6 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
 
   if (*abort_flag && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
   tc_fence_before();
-  __syncwarp();
   cluster_arrive();                                  // nobody leaves while another CTA may still write to or signal it
   cluster_wait();
   if (warp == 1) {

@@ -18,3 +18,11 @@ def code(path):
 def test_no_barrier_arrival_is_relaxed(path):
     # a relaxed arrival orders nothing that the arriving thread did before it
     assert "arrive.relaxed" not in code(path)
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_aligned_barriers_follow_a_reconvergence(path):
+    # bar.sync and barrier.cluster.arrive .aligned want whole warps, and the code before them branches by thread
+    text = code(path)
+    for m in re.finditer(r'asm volatile\(\s*"(bar\.sync|barrier\.cluster\.arrive)', text):
+        assert re.search(r"__syncwarp\(\);\s*$", text[:m.start()]), text[m.start() - 80:m.end() + 40]
