@@ -68,7 +68,7 @@ fabric_probe_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size
       for (int it = 0; it < iters && !timed_out; ++it)
         for (size_t p = blockIdx.x; p < pieces; p += gridDim.x) {
           if (issued >= (uint32_t)depth) {
-            if (!mbar_wait(&full[stage], phase, abort_flag)) { timed_out = true; break; }
+            if (!mbar_wait_warp(&full[stage], phase, abort_flag)) { timed_out = true; break; }
             if (stage == depth - 1) phase ^= 1;
           }
           // `stage` was just drained (or never used): refill it
@@ -84,7 +84,7 @@ fabric_probe_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size
       const uint32_t pending = issued < (uint32_t)depth ? issued : (uint32_t)depth;
       if (issued < (uint32_t)depth) { stage = 0; phase = 0; }   // the ring never wrapped: oldest is slot 0
       for (uint32_t i = 0; i < pending && !timed_out; ++i) {
-        if (!mbar_wait(&full[stage], phase, abort_flag)) { timed_out = true; break; }
+        if (!mbar_wait_warp(&full[stage], phase, abort_flag)) { timed_out = true; break; }
         if (stage == depth - 1) phase ^= 1;
         if (++stage == depth) stage = 0;
       }
@@ -122,6 +122,7 @@ fabric_probe_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size
   if (timed_out) {
     *abort_flag = 1;
     if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
   }
 }
 

@@ -417,7 +417,10 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
     }
     if (split > 1) { cluster_sync(); cluster_sync(); }
   }
-  if (*abort_flag && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+  if (*abort_flag) {
+    if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
+  }
 }
 
 template <int M, int R, bool SYM>

@@ -375,7 +375,10 @@ fused_small_c_kernel(const __grid_constant__ Coefs cf, const __grid_constant__ C
     }
     bulk_wait_read<0>();
   }
-  if (*abort_flag && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+  if (*abort_flag) {
+    if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
+  }
 }
 
 template <int M, int GT, bool SYM>

@@ -301,6 +301,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
   if (timed_out) {
     *abort_flag = 1;
     if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

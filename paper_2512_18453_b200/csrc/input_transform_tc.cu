@@ -326,6 +326,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
   if (timed_out) {
     *abort_flag = 1;
     if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
   }
   tc_fence_before();
   __syncthreads();

@@ -158,6 +158,7 @@ output_transform_tma_kernel(const __grid_constant__ CUtensorMap tmM, const __gri
   if (timed_out) {
     *abort_flag = 1;
     if (lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+    settle_after_timeout();
   }
 }
 

@@ -441,10 +441,12 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
     }
   }
 
-  if (*abort_flag && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
+  const bool expired = *abort_flag != 0;
+  if (expired && lane == 0) atomicExch(status, NOVA_ERR_DEVICE_TIMEOUT);
   tc_fence_before();
   cluster_arrive();                                  // nobody leaves while another CTA may still write to or signal it
   cluster_wait();
+  if (expired) settle_after_timeout();               // also for what the others sent here and nobody waited for
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, tmem_cols);

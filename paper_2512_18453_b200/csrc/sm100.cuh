@@ -96,6 +96,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return mbar_wait(bar, parity, abort_flag);
 }
+// For a warp that leaves after an expired wait: copies and MMAs that were under way may still write to the CTA's shared
+// and tensor memory, which must not be given to the next CTA before they have.  One millisecond, a hundred times what
+// the slowest of them takes.
+__device__ __forceinline__ void settle_after_timeout() {
+  const uint64_t t0 = global_ns();
+  for (int i = 0; i < 4096 && global_ns() - t0 < 1000000ull; ++i) __nanosleep(2000);
+}
 
 // Fetch a tensor map ahead of its first use, which would otherwise wait for it.  A kernel parameter
 // may be fetched before the wait for the preceding kernel.

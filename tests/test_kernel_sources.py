@@ -26,3 +26,11 @@ def test_aligned_barriers_follow_a_reconvergence(path):
     text = code(path)
     for m in re.finditer(r'asm volatile\(\s*"(bar\.sync|barrier\.cluster\.arrive)', text):
         assert re.search(r"__syncwarp\(\);\s*$", text[:m.start()]), text[m.start() - 80:m.end() + 40]
+
+
+@pytest.mark.parametrize("path", [p for p in SOURCES if p.endswith(".cu")], ids=os.path.basename)
+def test_kernels_with_bounded_waits_let_their_copies_land(path):
+    # after an expired wait a kernel ends only when nothing is under way to its shared or tensor memory any more
+    text = code(path)
+    if re.search(r"tma_load_\w+\(|bulk_g2s\(|umma_\w+\(", text):
+        assert "settle_after_timeout();" in text
