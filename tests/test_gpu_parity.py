@@ -744,6 +744,31 @@ def test_scales_whose_coefficient_products_do_not_fit_half(e, C):
     check_fp16(y, x, g, m, pts, scales=sc)
 
 
+@pytest.mark.parametrize("m,key,shape", [(4, ("nova", 4), (5, 114, 110, 8, 24)), (6, ("asym", 6), (9, 202, 206, 8, 16))])
+def test_eight_channels_and_many_tiles_with_pooled_stores(m, key, shape):
+    # 4060 and 10710 tiles: the input transform changes kernels on these two lines; a few images of the same call are
+    # on the other side.  Both evaluate V in float and round once, so that y differs by flips of last bits, amplified as
+    # any rounding of V is: judged against the error of the emulation, as everywhere
+    N, H, W, C, K = shape
+    x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=340 + m)
+    plan = nv.Plan(m, point_set(*key))
+    U = plan.filter_transform(torch.from_numpy(g).cuda())
+    xd = torch.from_numpy(x).cuda()
+    flags = nv.RELU | nv.POOL2X2
+    whole = plan.conv2d(xd, U, flags=flags)
+    parts = torch.cat([plan.conv2d(xd[i:i + 2].contiguous(), U, flags=flags) for i in range(0, N, 2)])
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0
+    n = 2
+    y1 = np.maximum(conv.direct_conv_fp64(x[:n], g), 0.0)
+    ye = conv.winograd_conv_emulated(x[:n], g, m, point_set(*key), "fp16", apply_relu=True).astype(np.float64)
+    pool = lambda a: a.reshape(a.shape[0], H // 2, 2, W // 2, 2, K).max(axis=(2, 4))
+    e_emu = np.linalg.norm(pool(ye) - pool(y1))
+    for y in (whole, parts):
+        assert np.linalg.norm(y[:n].cpu().numpy().astype(np.float64) - pool(ye)) <= EMU_CLOSE * e_emu
+    assert torch.linalg.vector_norm(whole.double() - parts.double()) <= 2 * EMU_CLOSE * e_emu * (N / n) ** 0.5
+
+
 # ---------------------------------------------------------------- INT8 Winograd-domain pipeline
 def gpu_conv_int8(x, g, m, pts, quant=nv.QUANT_PER_TENSOR, scale_U=None, scale_V=0.0, flags=0, coef=nv.COEF_FP32,
                   scales=(None, None)):
