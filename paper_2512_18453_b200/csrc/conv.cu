@@ -82,14 +82,14 @@ bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
 // 24 -> 64: 38.7 -> 37.3, 49.8 -> 35.2, 65.4 -> 34.1.  With 4 points its units are too small to pay below 64
 // channels once a layer has many tiles (98 tiles 8.0 -> 6.7 us, 1568 tiles 11.8 -> 12.1, 12544 tiles 24.3 -> 35.5); the
 // half pipeline has a kernel of its own for them, so that the line matters to the INT8 pipeline alone.  Eight channels
-// use an eighth of a unit: with 6 points (CUDA cores / tensor cores, 8 -> 64 pooled) 1568 tiles 17.2 / 15.6 us, 6272 34.9 /
-// 38.1, 25088 85.2 / 98.9; with 8 points 5776 tiles 59.5 / 50.0, 11552 95.3 / 97.3, 23328 161 / 168; with 10 points 6272 tiles 109 /
-// 85; sixteen channels 25088 tiles with 6 points 94.3 / 87.3.
+// use an eighth of a unit.  With 6 points (CUDA cores / tensor cores, 8 -> 64 pooled): 392 tiles 12.9 / 12.1 us, 1568 tiles 17.2 /
+// 15.6, 6272 34.9 / 38.1, 25088 85.2 / 98.9; with 8: 800 tiles 21.4 / 15.3, 5776 59.5 / 50.0, 23328 161 / 168; with 10: 6272 tiles
+// 109 / 85; sixteen channels, 6 points: 25088 tiles 94.3 / 87.3.  The line does not depend on the batch: a part of a batch
+// has the bits of the whole.
 bool tensor_core_input(const nova_plan* p, const Geom& g, int flags) {
   if (!p->kron_dev || (flags & NOVA_TRANSFORM_SIMT)) return false;
   if (p->n == 4) return g.C >= 64 || g.P <= 1024;
-  if (g.C == 8) return p->n == 10 || g.P <= (p->n == 6 ? 4000 : 10000);
-  return true;
+  return p->n > 6 || g.C > 8;
 }
 
 // Product and output transform in one kernel, for callers with the recommended workspace (a smaller one asks for the
