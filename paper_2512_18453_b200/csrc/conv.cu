@@ -22,6 +22,7 @@ struct Chunking {
   int pc;            // tiles per chunk
   int pc_pad;        // row stride of V and M inside the workspace
   int chunks;
+  int ldv;           // row pitch of V in elements
   size_t v_bytes, m_bytes;
 };
 
@@ -42,6 +43,7 @@ bool choose_chunking(const nova_plan* p, const Geom& g, size_t bytes, Chunking* 
   c->pc = (int)(pc < g.P ? pc : g.P);
   c->pc_pad = (int)pc;
   c->chunks = (int)((g.P + pc - 1) / pc);
+  c->ldv = g.C;
   c->v_bytes = round_up((size_t)g.n * g.n * c->pc_pad * g.C * elt_bytes(p->mode), kAlign);
   c->m_bytes = round_up((size_t)g.n * g.n * c->pc_pad * g.K * 4, kAlign);
   return c->v_bytes + c->m_bytes <= bytes;
@@ -92,12 +94,23 @@ bool tensor_core_input(const nova_plan* p, const Geom& g, int flags) {
   return p->n > 6 || g.C > 8;
 }
 
+// Row pitch of V for product_output.cu: whole sectors of 32 bytes where a row takes several of that kernel's 128-byte
+// boxes.  It fetches V once per block of filters, and rows that start anywhere cost a sector and often a line more per box.
+// Pitch of C / this pitch: F(4,5) 32 x 56 x 56, 120 -> 256 204 / 172 us; F(2,5) 8 x 56 x 56, 104 -> 256 128 / 119; F(6,3) 32 x 56 x 56,
+// 104 -> 512 238 / 226; F(2,3) 8 x 56 x 56, 520 -> 256 108 / 100; INT8 F(4,5) 240 -> 128 156 / 139.  A row of a single box, or of
+// two with 4 points, only gets longer (F(2,3) 24 -> 64 17.8 / 18.7, F(4,5) 40 -> 128 33.7 / 34.0).
+int padded_pitch(int n, int C, int bytes) {
+  return C * bytes <= (n == 4 ? 256 : 128) ? C : (C * bytes + 31) / 32 * 32 / bytes;
+}
+
 // Product and output transform in one kernel, for callers with the recommended workspace (a smaller one asks for the
 // chunked three kernels); only V is in it then, in as many chunks as it takes.
 bool two_kernels(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags, Chunking* c) {
   if ((flags & kThreeKernelFlags) || !use_product_output(p, g, false)) return false;
   if (ws_bytes < nova_conv2d_workspace_bytes(p, g.N, g.H, g.W, g.C, g.K)) return false;
-  const size_t v_tile = (size_t)g.n * g.n * g.C * elt_bytes(p->mode);
+  // the CUDA-core transform of more than 4 points writes rows of C
+  const int ldv = p->n == 4 || tensor_core_input(p, g, flags) ? padded_pitch(p->n, g.C, 2) : g.C;
+  const size_t v_tile = (size_t)g.n * g.n * ldv * elt_bytes(p->mode);
   long long pc = (long long)(ws_bytes / v_tile) / 128 * 128;
   const long long p_pad = round_up_ll(g.P, 128);
   if (pc > p_pad) pc = p_pad;
@@ -105,6 +118,7 @@ bool two_kernels(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags, 
   c->pc = (int)(pc < g.P ? pc : g.P);
   c->pc_pad = (int)pc;
   c->chunks = (int)((g.P + pc - 1) / pc);
+  c->ldv = ldv;
   c->v_bytes = (size_t)pc * v_tile;
   c->m_bytes = 0;
   return true;
@@ -200,6 +214,7 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
   const bool tc = use_tcgen05(p, flags);
   if (tc && !p->status_dev) return NOVA_ERR_CUDA;
   const bool two = two_kernels(p, g, ws_bytes, flags, &c);
+  g.ldv = c.ldv;
   char* Vb = static_cast<char*>(ws);
   float* Mb = reinterpret_cast<float*>(Vb + c.v_bytes);
   const int nfreq = g.n * g.n;
@@ -446,7 +461,7 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
   if ((flags & NOVA_POOL2X2) && ((H | W) & 1)) return NOVA_ERR_INVALID_ARG;
   if (!p->status_dev) return NOVA_ERR_CUDA;
   if (!on_plan_device(p)) return NOVA_ERR_INVALID_ARG;
-  const Geom g = make_geom(p, N, H, W, C, K);
+  Geom g = make_geom(p, N, H, W, C, K);
   if (g.P >= (1ll << 24)) return NOVA_ERR_UNSUPPORTED;
   const Int8Layout l = int8_layout(g);
   if (ws_bytes < l.total) return NOVA_ERR_WORKSPACE;
@@ -460,10 +475,13 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
   // The tensor-core transform needs the exact hi + lo table of half-rounded coefficients; plans
   // with float32 coefficients (and narrow layers) use the CUDA-core transform.
   const bool tc_in = tensor_core_input(p, g, flags);
+  const bool two = use_product_output(p, g, true) && !(flags & kThreeKernelFlags);
+  if (two && tc_in) g.ldv = padded_pitch(p->n, C, 1);           // into the room of M, which is not used then
   if (ev) cudaEventRecord(ev[0], s);
   // s_V is given, or max|V| / 127 over the batch, which costs one more pass of the input transform
   if (tc_in) {
-    float* parts = reinterpret_cast<float*>(Mb);      // one word per CTA, read before the product writes M
+    // one word per CTA in the last bytes of M, read before the product writes there (the rows of V end before)
+    float* parts = reinterpret_cast<float*>(base + l.total) - p->sm_count;
     if (!(scale_V > 0.f)) e = launch_input_transform_tc_int8(p, g, x, Vq, slot, parts, 0.f, 0, 0, pc, l.pad, stream);
     if (!e) e = launch_input_transform_tc_int8(p, g, x, Vq, slot, parts, scale_V, 1, 0, pc, l.pad, stream);
   } else {
@@ -477,7 +495,7 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
     if (!e) e = launch_input_transform_int8(p, g, x, Vq, slot, 1, 0, pc, l.pad, stream);
   }
   if (ev) cudaEventRecord(ev[1], s);
-  if (!e && use_product_output(p, g, true) && !(flags & kThreeKernelFlags)) {
+  if (!e && two) {
     e = launch_product_output(p, g, Vq, Uq, y, 0, pc, l.pad, store_flags(flags), stream, scale_U, slot);
     if (ev) { cudaEventRecord(ev[2], s); cudaEventRecord(ev[3], s); }
     if (e) g_last_cuda_error = e;

@@ -34,7 +34,7 @@ __device__ __forceinline__ uint32_t pack2(float2 v) {
 template <bool SYM>
 __global__ void __launch_bounds__(kN4Threads)
 input_transform_n4_kernel(const __grid_constant__ Coefs cf, const __half* __restrict__ x, __half* __restrict__ V, int H, int W,
-                          int C, int Th, int Tw, long long p0, int pc, int pc_pad) {
+                          int C, int ldv, int Th, int Tw, long long p0, int pc, int pc_pad) {
   constexpr int N = 4;
   sm100::pdl_wait();
   sm100::pdl_launch_dependents();
@@ -81,8 +81,8 @@ input_transform_n4_kernel(const __grid_constant__ Coefs cf, const __half* __rest
       for (int xi = 0; xi < N; ++xi) o[e][xi][nu] = pack2(out[xi]);
     }
   }
-  const size_t f_stride = (size_t)pc_pad * C;
-  __half* dst = V + (size_t)pl * C + c;
+  const size_t f_stride = (size_t)pc_pad * ldv;
+  __half* dst = V + (size_t)pl * ldv + c;
 #pragma unroll
   for (int xi = 0; xi < N; ++xi)
 #pragma unroll
@@ -99,9 +99,9 @@ int launch_input_transform_n4(const nova_plan* plan, const Geom& g, const void* 
   cudaStream_t s = (cudaStream_t)stream;
   return (int)(plan->symmetric
                    ? launch_overlapped(input_transform_n4_kernel<true>, grid, kN4Threads, 0, s, plan->kcoefs, (const __half*)x,
-                                       (__half*)V, g.H, g.W, g.C, g.Th, g.Tw, p0, pc, pc_pad)
+                                       (__half*)V, g.H, g.W, g.C, g.ldv, g.Th, g.Tw, p0, pc, pc_pad)
                    : launch_overlapped(input_transform_n4_kernel<false>, grid, kN4Threads, 0, s, plan->kcoefs, (const __half*)x,
-                                       (__half*)V, g.H, g.W, g.C, g.Th, g.Tw, p0, pc, pc_pad));
+                                       (__half*)V, g.H, g.W, g.C, g.ldv, g.Th, g.Tw, p0, pc, pc_pad));
 }
 
 }  // namespace nova

@@ -102,7 +102,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
 template <int M, int QMODE, int R, bool LO>
 __global__ void __launch_bounds__(kTcThreads, 1)
 input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmKron,
-                          void* __restrict__ Vout, int C, int Th, int Tw, long long p0, int pc, int pc_pad,
+                          void* __restrict__ Vout, int C, int ldv, int Th, int Tw, long long p0, int pc, int pc_pad,
                           int* __restrict__ status, float* __restrict__ qslot, float* __restrict__ qparts, float qgiven) {
   using Cfg = TcCfg<M, R>;
   static_assert(TcCfgCheck<M, R>::ok, "");
@@ -239,7 +239,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     // ---------------- epilogue
     const int quad = warp & 3;                    // the TMEM lane quadrant this warp may read
     const int group = (warp - kProdWarps - kMmaWarps) >> 2;
-    const size_t f_stride = (size_t)pc_pad * C;
+    const size_t f_stride = (size_t)pc_pad * ldv;
     float qs = 1.f, amax = 0.f;
     if constexpr (QMODE == 2) {
       qs = qgiven;
@@ -263,8 +263,8 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
       if (!mbar_wait_warp(&tmem_full[acc], acc_phase, abort_flag)) { timed_out = true; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * kAccCols;
-      __half* dst = reinterpret_cast<__half*>(Vout) + (size_t)pl * C + c;
-      int8_t* dst8 = reinterpret_cast<int8_t*>(Vout) + (size_t)pl * C + c;
+      __half* dst = reinterpret_cast<__half*>(Vout) + (size_t)pl * ldv + c;
+      int8_t* dst8 = reinterpret_cast<int8_t*>(Vout) + (size_t)pl * ldv + c;
 #pragma unroll
       for (int col0 = 0; col0 < Cfg::NFP; col0 += 64) {
         constexpr int kMaxCols = 64;
@@ -370,7 +370,7 @@ int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long 
   const long long units = ((long long)pc * ((g.C + 63) / 64) + 1) / 2;   // two (tile, 64-channel block) pairs each
   const int grid = (int)(units < sms ? units : sms);
   return (int)launch_overlapped(kernel, grid, kTcThreads, Cfg::kTotal, stream, tmX, tmK,
-                                V, g.C, g.Th, g.Tw, p0, pc, pc_pad, plan->status_dev, qslot, qparts, qgiven);
+                                V, g.C, g.ldv, g.Th, g.Tw, p0, pc, pc_pad, plan->status_dev, qslot, qparts, qgiven);
 }
 
 }  // namespace

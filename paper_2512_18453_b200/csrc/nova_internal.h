@@ -66,6 +66,7 @@ inline size_t elt_bytes(int mode) { return mode == NOVA_FP32 ? 4 : 2; }
 struct Geom {
   int N, H, W, C, K, m, n, Th, Tw;
   long long P;   // total tiles
+  int ldv;       // row pitch of V in elements: C, or more where product_output.cu reads it
 };
 inline Geom make_geom(const nova_plan* p, int N, int H, int W, int C, int K) {
   Geom g;
@@ -73,6 +74,7 @@ inline Geom make_geom(const nova_plan* p, int N, int H, int W, int C, int K) {
   g.Th = (H + p->m - 1) / p->m;
   g.Tw = (W + p->m - 1) / p->m;
   g.P = (long long)N * g.Th * g.Tw;
+  g.ldv = C;
   return g;
 }
 

@@ -453,13 +453,13 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
   }
 }
 
-// [nfreq][rows][inner] elements, 128-byte swizzled boxes of box_rows rows of two neighbouring frequencies
-bool make_map(CUtensorMap* map, bool i8, const void* base, int inner, int rows, long long freq_stride, int nfreq, int box_rows) {
+// [nfreq][rows][inner] elements, rows `pitch` elements apart, 128-byte swizzled boxes of box_rows rows of two neighbouring frequencies
+bool make_map(CUtensorMap* map, bool i8, const void* base, int inner, int pitch, int rows, long long freq_stride, int nfreq, int box_rows) {
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return false;
   const int esize = i8 ? 1 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)nfreq};
-  cuuint64_t strides[2] = {(cuuint64_t)inner * esize, (cuuint64_t)freq_stride * esize};
+  cuuint64_t strides[2] = {(cuuint64_t)pitch * esize, (cuuint64_t)freq_stride * esize};
   cuuint32_t box[3] = {(cuuint32_t)(kRowBytes / esize), (cuuint32_t)box_rows, 2};
   cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides,
@@ -489,8 +489,8 @@ int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void*
   // their sums are not sent)
   a.box_rows = pc < kRows ? (pc + 7) & ~7 : kRows;
   CUtensorMap tmV, tmU;
-  if (!make_map(&tmV, I8, V, g.C, pc, (long long)pc_pad * g.C, Cfg::N * Cfg::N, a.box_rows) ||
-      !make_map(&tmU, I8, U, g.C, g.K, (long long)g.K * g.C, Cfg::N * Cfg::N, F))
+  if (!make_map(&tmV, I8, V, g.C, g.ldv, pc, (long long)pc_pad * g.ldv, Cfg::N * Cfg::N, a.box_rows) ||
+      !make_map(&tmU, I8, U, g.C, g.C, g.K, (long long)g.K * g.C, Cfg::N * Cfg::N, F))
     return (int)cudaErrorUnknown;
   a.H = g.H; a.W = g.W; a.C = g.C; a.K = g.K; a.Th = g.Th; a.Tw = g.Tw; a.pc = pc; a.pc_pad = pc_pad; a.p0 = p0;
   a.F = F;
@@ -535,20 +535,28 @@ int block_filters(int n, int K, int num_ks) {
 
 // Against product and output transform as two kernels.  What this kernel saves is M (n*n floats per tile and filter,
 // written and read); what it costs is V once per F filters instead of once per 256, and an exchange at 17 bytes per
-// clock and SM.  So it pays where M is large and the channels few: num_ks = 128-byte rows of channels.  Whole calls, three
-// kernels / two kernels, by MB of M:
-//   n = 4          3 MB 0.96 .. 1.09, 12 MB 1.04 .. 1.20, 49 MB 1.12 .. 1.34, 98 MB 1.26 .. 1.59, 392 MB 1.80 .. 2.41
-//   n = 6, m = 2   55 MB 1.22, 110 MB 1.12, 220 MB 1.59, 441 MB 1.50 (up to two rows)
-//   n = 6, m = 4   one row: 13 MB 0.93, 55 MB 1.00, 220 MB 1.13 .. 1.24, 882 MB 1.72; two rows: 110 MB 0.93, 441 MB 1.25;
-//                  four rows 0.83 .. 1.05
-//   n = 8, m = 4   one row: 24 MB 1.05, 98 MB 1.15; two rows: 98 MB 0.93, 196 MB 1.05, 392 MB 1.15; four rows 0.89
-//   n = 8, m = 6   90 MB 0.86, 180 MB 0.97 .. 1.05, 361 MB 1.07 .. 1.12, 757 MB 1.27 (up to two rows); four rows 0.79
+// clock and SM.  So it pays where M is large and the channels few: num_ks = 128-byte rows of channels.  Whole calls, time of
+// three kernels / of two, by MB of M, over 1100 layers of 1 .. 32 images of 28 x 28 .. 112 x 112:
+//   n = 4          up to two rows: 13 MB 1.0 .. 1.3, 26 MB 1.1 .. 1.4, 103 MB 1.3 .. 1.5, 411 MB 1.5 .. 2.2
+//                  more: one filter block 1.04 .. 1.2; several: 8 rows 26 MB 1.0, 51 MB 0.94 .. 1.12, 103 MB 1.0 .. 1.1, 411 MB 1.35; 12 rows
+//                  51 MB 0.85 .. 1.1, 103 MB 0.91; 16 rows 26 .. 103 MB 0.81 .. 0.95: the more rows, the more of M it takes
+//   n = 6, m = 2   one row 29 MB 1.14, 58 MB 1.04 .. 1.24; two rows 58 MB 1.04 .. 1.14, 116 MB 1.1 .. 1.2, 462 MB 1.4
+//   n = 6, m = 4   one row: 14 .. 58 MB 0.96 .. 1.02, 116 MB 1.0 .. 1.06, 231 MB and more 1.07 .. 1.7; two rows: 116 MB 0.93 .. 1.06,
+//                  173 MB 0.95, 231 MB 0.97 (256 filters) .. 1.18 (64), 462 MB 1.16 .. 1.24
+//   n = 8, m = 4   one row: 26 MB 1.06, 103 MB 1.18; two rows: 103 MB 0.96 .. 1.06, 206 MB 0.98 .. 1.03, 411 MB 1.07 .. 1.26
+//   n = 8, m = 6   one row: 95 MB 0.96, 189 MB 1.01, 419 MB 1.05; two rows: 105 MB 0.87, 379 MB 1.04 .. 1.07, 757 MB 1.13, but with 512
+//                  filters 419 MB 0.97
+// Rows of channels that are not whole 32-byte sectors lose 5 to 10 % more here, because those of U keep their pitch: 72 or 104
+// channels 0.87 .. 0.96 at two rows, 24 or 40 channels 0.9 .. 0.97 near the line of n = 8, m = 4.
 // INT8 lines up with half at the same number of rows (32 x 56 x 56, 256 -> 256: 132 -> 123 us).
 bool use_product_output(const nova_plan* plan, const Geom& g, bool int8) {
   if (plan->mode != NOVA_FP16_F32ACC || plan->n > 8 || !plan->status_dev || plan->sm_count < 64 || g.P >= (1ll << 31)) return false;
   const int num_ks = (g.C * (int8 ? 1 : 2) + kRowBytes - 1) / kRowBytes;
   const double m_mb = 4e-6 * plan->n * plan->n * (double)g.P * g.K;
-  if (plan->n == 4) return m_mb >= 12;
+  if (plan->n == 4) {
+    const int F = block_filters(4, g.K, num_ks), num_kb = (g.K + F - 1) / F;
+    return m_mb >= 12 && (num_kb == 1 || m_mb * (num_kb == 2 ? 4 : 2) >= num_ks * num_ks);
+  }
   if (num_ks > 2) return false;
   if (plan->n == 6) return m_mb >= (plan->m == 2 ? 50 : 100 * num_ks);
   return m_mb >= (plan->m == 6 ? 300 : num_ks == 1 ? 20 : 150);
