@@ -75,7 +75,8 @@ bool use_fused_small_c(const nova_plan* p, const Geom& g, int flags) {
 int store_flags(int flags) { return ((flags & NOVA_RELU) ? 1 : 0) | ((flags & NOVA_POOL2X2) ? 2 : 0); }
 
 bool one_kernel(const nova_plan* p, const Geom& g, int flags) {
-  return fused_fp32_applies(p) || use_fused_small_c(p, g, flags);
+  if (p->mode == NOVA_FP32) return !(flags & (NOVA_GEMM_SIMT | NOVA_TRANSFORM_SIMT)) && fused_fp32_applies(p);
+  return use_fused_small_c(p, g, flags);
 }
 
 // Input transform on the tensor cores or on CUDA cores.  The tensor-core kernel computes 64 channels

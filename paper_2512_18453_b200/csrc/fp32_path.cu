@@ -7,7 +7,8 @@
 // tile on well-conditioned points sits at a relative error of 1.2e-4 .. 1.7e-4; this way it stays
 // below 1e-4.  The kernels are plain dense products with the plan's tables (internal point
 // order).  Tiles of up to 8 points run steps 2-4 in fused_fp32.cu; the input and output
-// transforms here serve 10 points, whose sums do not fit a block of that kernel.
+// transforms here serve 10 points, whose sums do not fit a block of that kernel, and the others where a flag asks for
+// the separate kernels.
 #include <cuda_runtime.h>
 
 #include "nova_internal.h"
@@ -179,15 +180,11 @@ int launch_filter_transform_f32(const nova_plan* plan, const void* g, int K, int
 }
 int launch_input_transform_f32(const nova_plan* plan, const Geom& g, const void* x, void* V, long long p0, int pc,
                                int pc_pad, void* stream) {
-  if (plan->n != 10) return (int)cudaErrorInvalidValue;
-  return plan->r == 3 ? input_go<10, 3>(plan, g, x, V, p0, pc, pc_pad, (cudaStream_t)stream)
-                      : input_go<10, 5>(plan, g, x, V, p0, pc, pc_pad, (cudaStream_t)stream);
+  NOVA_F32_DISPATCH(input_go, plan, g, x, V, p0, pc, pc_pad, (cudaStream_t)stream);
 }
 int launch_output_transform_f32(const nova_plan* plan, const Geom& g, const void* M, void* y, long long p0, int pc,
                                 int pc_pad, int relu, void* stream) {
-  if (plan->n != 10) return (int)cudaErrorInvalidValue;
-  return plan->r == 3 ? output_go<10, 3>(plan, g, M, y, p0, pc, pc_pad, relu, (cudaStream_t)stream)
-                      : output_go<10, 5>(plan, g, M, y, p0, pc, pc_pad, relu, (cudaStream_t)stream);
+  NOVA_F32_DISPATCH(output_go, plan, g, M, y, p0, pc, pc_pad, relu, (cudaStream_t)stream);
 }
 
 }  // namespace nova

@@ -423,6 +423,17 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
   }
 }
 
+// setmaxnreg draws on the registers the block was launched with: a build whose register count is not what the split was
+// computed for does without this kernel.
+template <int M, int R, bool SYM>
+bool built() {
+  static const int regs = [] {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, fused_fp32_kernel<M, R, SYM>) == cudaSuccess ? at.numRegs : 0;
+  }();
+  return regs >= Fc32<M, R>::kLaunchRegs;
+}
+
 template <int M, int R, bool SYM>
 int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, int nb, int split,
        cudaStream_t stream) {
@@ -430,13 +441,7 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return (int)cudaErrorUnknown;
   auto kernel = fused_fp32_kernel<M, R, SYM>;
-  // setmaxnreg draws on the registers the block was launched with: refuse a build whose register count
-  // is not what the split was computed for
-  static const int built_regs = [kernel] {
-    cudaFuncAttributes at;
-    return cudaFuncGetAttributes(&at, kernel) == cudaSuccess ? at.numRegs : 0;
-  }();
-  if (built_regs < Cfg::kLaunchRegs) return (int)cudaErrorInvalidConfiguration;
+  if (!built<M, R, SYM>()) return (int)cudaErrorInvalidConfiguration;
   const int f_run = 8 * nb * Cfg::NH;
   CUtensorMap tmX, tmU;
   cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -513,7 +518,20 @@ void choose_blocks(int n, const Geom& g, int sms, int* nb_out, int* split_out) {
 
 }  // namespace
 
-bool fused_fp32_applies(const nova_plan* plan) { return plan->mode == NOVA_FP32 && plan->n <= 8; }
+bool fused_fp32_applies(const nova_plan* plan) {
+  if (plan->mode != NOVA_FP32 || plan->n > 8) return false;
+  if (plan->device < 0) return true;                   // plans made without a device only answer questions
+  const int key = plan->r * 10 + plan->m;
+  const bool sym = plan->symmetric != 0;
+  switch (key) {
+    case 32: return sym ? built<2, 3, true>() : built<2, 3, false>();
+    case 34: return sym ? built<4, 3, true>() : built<4, 3, false>();
+    case 36: return sym ? built<6, 3, true>() : built<6, 3, false>();
+    case 52: return sym ? built<2, 5, true>() : built<2, 5, false>();
+    case 54: return sym ? built<4, 5, true>() : built<4, 5, false>();
+  }
+  return false;
+}
 
 int launch_fused_fp32(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;

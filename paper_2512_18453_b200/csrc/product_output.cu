@@ -472,18 +472,38 @@ int cluster_slots(int n, int sms) {                  // clusters of n CTAs that 
   return s < 1 ? 1 : s;
 }
 
+// setmaxnreg draws on the registers the block was launched with: a build whose register count is not what the split was
+// computed for does without this kernel.
+template <int M, int R, bool SYM, bool I8>
+bool built() {
+  static const int regs = [] {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, product_output_kernel<M, R, SYM, I8>) == cudaSuccess ? at.numRegs : 0;
+  }();
+  return regs >= PoCfg<M, R>::kLaunchRegs;
+}
+template <int M, int R>
+bool built(bool sym, bool i8) {
+  return i8 ? (sym ? built<M, R, true, true>() : built<M, R, false, true>()) : (sym ? built<M, R, true, false>() : built<M, R, false, false>());
+}
+bool built(const nova_plan* plan, bool i8) {
+  const bool sym = plan->symmetric != 0;
+  switch (plan->r * 10 + plan->m) {
+    case 32: return built<2, 3>(sym, i8);
+    case 34: return built<4, 3>(sym, i8);
+    case 36: return built<6, 3>(sym, i8);
+    case 52: return built<2, 5>(sym, i8);
+    case 54: return built<4, 5>(sym, i8);
+  }
+  return false;
+}
+
 template <int M, int R, bool SYM, bool I8>
 int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void* y, long long p0, int pc, int pc_pad, int relu, int F,
        const float* scale_U, const float* scale_V, cudaStream_t stream) {
   using Cfg = PoCfg<M, R>;
   auto kernel = product_output_kernel<M, R, SYM, I8>;
-  // setmaxnreg draws on the registers the block was launched with: refuse a build whose register count
-  // is not what the split was computed for
-  static const int built_regs = [kernel] {
-    cudaFuncAttributes at;
-    return cudaFuncGetAttributes(&at, kernel) == cudaSuccess ? at.numRegs : 0;
-  }();
-  if (built_regs < Cfg::kLaunchRegs) return (int)cudaErrorInvalidConfiguration;
+  if (!built<M, R, SYM, I8>()) return (int)cudaErrorInvalidConfiguration;
   PoArgs a;
   // rows of a box of V: a layer of fewer than 128 tiles fetches no zero fill (the rows beyond hold what they held:
   // their sums are not sent)
@@ -551,6 +571,7 @@ int block_filters(int n, int K, int num_ks) {
 // INT8 lines up with half at the same number of rows (32 x 56 x 56, 256 -> 256: 132 -> 123 us).
 bool use_product_output(const nova_plan* plan, const Geom& g, bool int8) {
   if (plan->mode != NOVA_FP16_F32ACC || plan->n > 8 || !plan->status_dev || plan->sm_count < 64 || g.P >= (1ll << 31)) return false;
+  if (!built(plan, int8)) return false;
   const int num_ks = (g.C * (int8 ? 1 : 2) + kRowBytes - 1) / kRowBytes;
   const double m_mb = 4e-6 * plan->n * plan->n * (double)g.P * g.K;
   if (plan->n == 4) {

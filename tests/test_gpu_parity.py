@@ -138,6 +138,27 @@ def test_fp32_one_kernel_blocks_match_direct(m, key, r, shape):
     assert conv.rel_l2(y.cpu().numpy(), y1) <= 1.5 * e_emu + 1e-7
 
 
+@pytest.mark.parametrize("m,key,r", [(2, ("std", 2), 3), (4, ("asym", 4), 3), (6, ("half", 6), 3), (2, ("nova", 4), 5),
+                                     (4, ("half", 6), 5)])
+@pytest.mark.parametrize("flag", [nv.GEMM_SIMT, nv.TRANSFORM_SIMT])
+def test_fp32_mode_in_three_kernels_where_a_flag_asks_for_them(m, key, r, flag):
+    # the second GPU path of the mode: the same double sums, M rounded to float between the kernels
+    N, H, W, C, K = 2, 21, 17, 24, 40
+    x, g = make_conv_inputs(N, H, W, C, K, "fp32", True, True, seed=150 + m, r=r)
+    pts = point_set(*key)
+    plan = nv.Plan(m, pts, nv.FP32, r=r)
+    ws = plan.workspace_bytes(N, H, W, C, K)
+    assert plan.launch_count(N, H, W, C, K, ws) == 1 and plan.launch_count(N, H, W, C, K, ws, flag) == 3
+    xd, U = torch.from_numpy(x).cuda(), plan.filter_transform(torch.from_numpy(g).cuda())
+    y1 = np.maximum(conv.direct_conv_fp64(x, g), 0.0)
+    e_emu = conv.rel_l2(conv.winograd_conv_emulated(x, g, m, pts, "fp32", apply_relu=True), y1)
+    for flags in (nv.RELU, nv.RELU | flag):
+        y = plan.conv2d(xd, U, flags=flags)
+        torch.cuda.synchronize()
+        assert plan.device_status() == 0
+        assert conv.rel_l2(y.cpu().numpy(), y1) <= 1.5 * e_emu + 1e-7
+
+
 def test_cfg1_fp32_standard_f2():
     c = CONFIGS["cfg1"]
     x, g = make_conv_inputs(c.N, c.H, c.W, c.C, c.K, c.dtype, c.relu_inputs, c.he_weights, c.seed)
