@@ -8,7 +8,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnova.so")
-EXT = os.path.join(HERE, "_fastcall.so")
+# named for this interpreter's ABI: another one does not import it and goes through ctypes
+EXT = os.path.join(HERE, "_fastcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["plan.cpp", "transforms.cu", "filter_transform.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "input_transform_n4.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "product_output.cu", "conv.cu"]
 
 
@@ -28,10 +29,13 @@ def needs_build():
 
 
 def build_ext():
-    """The CPython extension of the binding's hot calls; without Python headers the binding uses ctypes."""
+    """The CPython extension of the binding's hot calls; without headers of Python 3.9 or newer the binding uses ctypes."""
     src, inc = os.path.join(CSRC, "fastcall.c"), sysconfig.get_paths()["include"]
-    if not os.path.exists(os.path.join(inc, "Python.h")):
-        sys.stderr.write("no Python headers in %s: calls go through ctypes\n" % inc)
+    untagged = os.path.join(HERE, "_fastcall.so")           # an earlier build's name, which any interpreter would import
+    if untagged != EXT and os.path.exists(untagged):
+        os.remove(untagged)
+    if sys.version_info < (3, 9) or not os.path.exists(os.path.join(inc, "Python.h")):
+        sys.stderr.write("no headers of Python 3.9 or newer in %s: calls go through ctypes\n" % inc)
         return
     newest = max(os.path.getmtime(f) for f in (src, os.path.join(ROOT, "include", "nova.h")))
     if not os.path.exists(EXT) or os.path.getmtime(EXT) < newest:

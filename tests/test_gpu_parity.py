@@ -208,6 +208,35 @@ def test_filter_transform_of_a_large_layer_gives_the_bits_of_its_parts(m, key, r
     assert torch.equal(whole.view(torch.int16), parts.view(torch.int16))
 
 
+def test_calls_through_ctypes_give_the_bits_of_the_extensions(monkeypatch):
+    # a build without Python headers, or another interpreter's, has no extension
+    from paper_2512_18453_b200 import binding
+    x, g = make_conv_inputs(2, 14, 18, 48, 40, "fp16", True, True, seed=221)
+    g8 = make_conv_inputs(1, 4, 4, 48, 48, "fp16", True, True, seed=222)[1]
+    plan = nv.Plan(4, point_set("nova", 4))
+    xd, gd, g8d = (torch.from_numpy(a).cuda() for a in (x, g, g8))
+
+    def calls():
+        U = plan.filter_transform(gd)
+        Uq, sU = plan.filter_transform_int8(g8d)
+        y = torch.full((2, 14, 18, 40), float("nan"), dtype=torch.float16, device="cuda")
+        ws = torch.empty(plan.workspace_bytes(2, 14, 18, 48, 40), dtype=torch.uint8, device="cuda")
+        out = [U, plan.conv2d(xd, U, y, ws, nv.RELU), plan.conv2d(xd, U), plan.conv2d_int8(xd, Uq, sU, 0.0),
+               plan.conv2d_int8(xd, Uq, sU, 0.02, flags=nv.RELU)]
+        with pytest.raises(AssertionError):
+            plan.conv2d(xd.float(), U, y, ws)
+        with pytest.raises(nv.NovaError):
+            plan.conv2d(xd, U, y, ws[:256])
+        torch.cuda.synchronize()
+        return out
+    assert binding._fast()
+    a = calls()
+    monkeypatch.setattr(binding, "_fastcall", False)
+    b = calls()
+    for u, v in zip(a, b):
+        assert torch.equal(u.view(torch.int16), v.view(torch.int16)) and torch.isfinite(u).all()
+
+
 # ---------------------------------------------------------------- fp16 mode, both product kernels
 SHAPES16 = [(2, 13, 11, 16, 8), (1, 5, 3, 8, 8), (2, 30, 30, 64, 64), (3, 20, 20, 72, 136), (1, 17, 23, 136, 264)]
 

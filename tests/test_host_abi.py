@@ -259,3 +259,22 @@ def test_tensors_that_are_not_on_a_gpu_are_refused_as_arguments():
         plan.filter_transform(torch.zeros(8, 3, 3, 8, dtype=torch.float16))
     with pytest.raises(AssertionError):
         plan.conv2d_int8(x, U.to(torch.int8), torch.zeros(8), 0.0, torch.zeros_like(x), ws)
+
+
+def test_the_extension_carries_its_interpreters_abi_in_its_name():
+    import sysconfig
+    from paper_2512_18453_b200 import build
+    assert os.path.basename(build.EXT) == "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX")
+    if os.path.exists(build.EXT):
+        from paper_2512_18453_b200 import _fastcall
+        assert os.path.samefile(_fastcall.__file__, build.EXT)
+
+
+def test_an_extension_under_the_untagged_name_is_not_left_behind(tmp_path, monkeypatch):
+    from paper_2512_18453_b200 import build
+    monkeypatch.setattr(build, "HERE", str(tmp_path))
+    monkeypatch.setattr(build, "EXT", str(tmp_path / "_fastcall.tag.so"))
+    (tmp_path / "_fastcall.so").write_bytes(b"")
+    monkeypatch.setattr(build.sysconfig, "get_paths", lambda: {"include": str(tmp_path)})     # no headers
+    build.build_ext()
+    assert list(tmp_path.iterdir()) == []
