@@ -1189,14 +1189,22 @@ def test_eight_channel_layers_run_in_one_kernel_and_match_the_emulation(kind, m,
     assert whole <= EMU_CLOSE and tile <= EMU_CLOSE_TILE, (whole, tile)
 
 
-@pytest.mark.parametrize("kind,m,N", [("std", 2, 1), ("asym", 2, 1), ("nova", 4, 1), ("asym", 4, 1), ("half", 6, 4),
-                                      ("asym", 6, 4)])
+def takes_large_groups(m, P, K):
+    """Whether the one-kernel path of 8 channels walks its large groups of tiles: the launcher's rule, restated."""
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count // -(-K // 64)
+    rounds = lambda tiles: -(-(-(-P // tiles)) // ctas)
+    return rounds(8) >= 4 and rounds({2: 64, 4: 32, 6: 16}[m]) * {2: 310, 4: 280, 6: 175}[m] < rounds(8) * 100
+
+
+@pytest.mark.parametrize("kind,m,N", [("std", 2, 1), ("asym", 2, 1), ("nova", 4, 1), ("asym", 4, 1), ("half", 6, 9),
+                                      ("asym", 6, 9)])
 def test_one_kernel_path_in_large_groups_matches_the_three_kernels(kind, m, N):
     # Nine filter blocks leave 16 CTAs each, so that groups of 64, 32 and 16 tiles are taken (m = 2, 4, 6); the last group
     # and the last filter block are ragged, and so are the tiles.  Judged against the three kernels, the same roundings
     # with sums in another order.  Per tile the bound is twice EMU_CLOSE_TILE: either side may be that far from the
     # emulation (triangle inequality), and a flipped rounding of one V reaches every output of its tile.
     H, W, C, K = 81, 85, 8, 520
+    assert takes_large_groups(m, N * -(-H // m) * -(-W // m), K)
     x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=305 + m)
     pts = point_set(kind, m)
     y, _, _ = gpu_conv(x, g, m, pts, nv.FP16_F32ACC, flags=nv.RELU)
@@ -1318,6 +1326,52 @@ def test_product_and_output_in_one_kernel_give_the_bits_of_two(op, m, key, r, sh
         assert plan.device_status() == 0
         assert torch.equal(got.view(torch.int16), want.view(torch.int16))
         assert torch.isfinite(got.float()).all()
+
+
+@pytest.mark.parametrize("op,m,key,r,shape,launches", [
+    # one block of filters and whole rows of channels: V's lines are dropped after their last read; more blocks of tiles
+    # than clusters, so that the ring goes on from one to the next
+    ("conv", 2, ("std", 2), 3, (8, 56, 56, 128, 64), 2),
+    ("conv", 4, ("nova", 4), 3, (32, 112, 112, 64, 32), 2),
+    ("conv", 4, ("nova", 4), 3, (32, 148, 148, 128, 32), 2),
+    ("conv", 6, ("half", 6), 3, (32, 204, 204, 64, 32), 2),
+    ("conv", 2, ("nova", 4), 5, (8, 76, 76, 64, 32), 2),
+    ("conv", 4, ("half", 6), 5, (8, 100, 100, 64, 32), 2),
+    ("conv", 4, ("half", 6), 5, (32, 96, 96, 128, 32), 2),
+    ("int8", 4, ("dyadic", 4), 3, (32, 112, 112, 128, 32), 2),
+    # blocks of 16 filters: one slice each, so that the two row groups take turns by block
+    ("conv", 2, ("std", 2), 3, (16, 56, 56, 64, 16), 2),
+    ("conv", 2, ("asym", 2), 3, (32, 56, 56, 72, 8), 2),
+    ("conv", 4, ("nova", 4), 3, (32, 148, 148, 64, 16), 2),
+    ("conv", 4, ("half", 6), 5, (8, 100, 100, 40, 16), 2),
+    # two chunks of tiles
+    ("conv", 2, ("std", 2), 3, (11, 162, 162, 512, 16), 4)])
+def test_product_and_output_in_one_kernel_by_blocks_and_chunks(op, m, key, r, shape, launches):
+    # bit for bit the separate kernels, several calls in a row on one workspace
+    N, H, W, C, K = shape
+    plan = nv.Plan(m, point_set(*key), r=r)
+    gen = torch.Generator(device="cuda").manual_seed(81 + m)
+    x = torch.randn(N, H, W, C, generator=gen, device="cuda", dtype=torch.float16).relu_()
+    g = (torch.randn(K, r, r, C, generator=gen, device="cuda") * (2.0 / (r * r * C)) ** 0.5).half()
+    if op == "conv":
+        U = plan.filter_transform(g)
+        nbytes = plan.workspace_bytes(N, H, W, C, K)
+        assert plan.launch_count(N, H, W, C, K, nbytes) == launches
+        run = lambda y, flags: plan.conv2d(x, U, y, ws, flags)
+    else:
+        U, sU = plan.filter_transform_int8(g, nv.QUANT_PER_CHANNEL)
+        nbytes = plan.int8_workspace_bytes(N, H, W, C, K)
+        run = lambda y, flags: plan.conv2d_int8(x, U, sU, 0.0, y, ws, flags)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    ys = [torch.full((N, H, W, K), float("nan"), dtype=torch.float16, device="cuda") for _ in range(4)]
+    for y in ys[:3]:
+        run(y, nv.RELU)
+    run(ys[3], nv.RELU | nv.GEMM_TCGEN05)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0
+    assert torch.isfinite(ys[3]).all()
+    for y in ys[:3]:
+        assert torch.equal(y.view(torch.int16), ys[3].view(torch.int16))
 
 
 def test_pooled_output_through_the_int8_and_host_entry_points():
