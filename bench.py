@@ -320,6 +320,29 @@ def whole_job_value(world, direct_flops_per_rank, ms_per_step):
     return world * direct_flops_per_rank / (ms_per_step * 1e-3) / 1e12
 
 
+def chunks_and_kernels(launches, launches_separate):
+    """(chunks, kernels per chunk) of a call: `launches` of it, `launches_separate` of the same call with the separate
+    kernels forced.  One kernel for everything; product and output transform in one, whose chunks are no more than
+    those of the separate kernels (only V is in the workspace); or all three."""
+    if launches == 1:
+        return 1, 1
+    per = 3 if launches == launches_separate else 2
+    return launches // per, per
+
+
+def kernel_classes(per_chunk, kms, flops, x_bytes, v_bytes, m_bytes, y_bytes, tensor_peak, hbm_peak, product, in_name, out_name):
+    """[(name, ms, bound, work)] of the kernel classes a step runs, with the algorithmic bytes or operations of each.  A merged
+    kernel's bound is the slower of its operations and the bytes it cannot do without (M stays on the chip)."""
+    def merged(nbytes):
+        return ("tensor", flops) if flops / (tensor_peak * 1e12) > nbytes / (hbm_peak * 1e9) else ("hbm", nbytes)
+    if per_chunk == 1:
+        return [("one_kernel", sum(kms)) + merged(x_bytes + y_bytes)]
+    if per_chunk == 2:
+        return [(in_name, kms[0], "hbm", x_bytes + v_bytes), (product + "_and_output", kms[1] + kms[2]) + merged(v_bytes + y_bytes)]
+    return [(in_name, kms[0], "hbm", x_bytes + v_bytes), (product, kms[1], "tensor", flops),
+            (out_name, kms[2], "hbm", m_bytes + y_bytes)]
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -459,19 +482,14 @@ def run_ours(args):
         return
 
     peaks = read_peaks()
-    chunks = launches // 3
-    names = ["input_transform", "product_tcgen05" if flags != nv.GEMM_SIMT else "product_simt", "output_transform"]
+    separate = plan.launch_count(c.N, c.H, c.W, c.C, c.K, ws_bytes, flags | nv.GEMM_TCGEN05)
+    chunks, per_chunk = chunks_and_kernels(launches, separate)
     n2 = (c.m + FILTER_R - 1) ** 2
-    elt = 2
-    # algorithmic bytes / flops per step of each kernel class
-    alg = [
-        ("hbm", 2.0 * c.N * c.H * c.W * c.C + elt * n2 * P * c.C),        # read x, write V
-        ("tensor", actual),                                                # 2 n^2 K C P flop
-        ("hbm", 4.0 * n2 * P * c.K + 2.0 * c.N * c.H * c.W * c.K),         # read M, write y
-    ]
-    dom = max(range(3), key=lambda i: kms[i])
-    bound, work = alg[dom]
-    dur_launch = kms[dom] * 1e-3 / chunks
+    classes = kernel_classes(per_chunk, kms, actual, 2.0 * c.N * c.H * c.W * c.C, 2.0 * n2 * P * c.C, 4.0 * n2 * P * c.K,
+                             2.0 * c.N * c.H * c.W * c.K, peaks["tflops_burst"], peaks["hbm_gbs"],
+                             "product_simt" if flags == nv.GEMM_SIMT else "product_tcgen05", "input_transform", "output_transform")
+    dom_name, dom_ms, bound, work = max(classes, key=lambda k: k[1])
+    dur_launch = dom_ms * 1e-3 / chunks
     if bound == "tensor":
         achieved, peak, runit = work / chunks / dur_launch / 1e12, peaks["tflops_burst"], "TFLOP/s"
     else:
@@ -499,10 +517,10 @@ def run_ours(args):
                           "tensor_us": actual / (peaks["tflops_burst"] * 1e12) * 1e6,
                           "hbm_us": min_bytes / (peaks["hbm_gbs"] * 1e9) * 1e6,
                           "alu_us": alu["alu_us"], "alu": alu},
-        "kernels_ms_per_step": {n_: v for n_, v in zip(names, kms) if n_ != "-"},
+        "kernels_ms_per_step": {k[0]: k[1] for k in classes},
         "single_step": step_stats,
         "filter_transform_ms": filter_ms,
-        "roofline": {"kernel": names[dom], "bound": bound, "achieved": achieved, "peak": peak, "unit": runit,
+        "roofline": {"kernel": dom_name, "bound": bound, "achieved": achieved, "peak": peak, "unit": runit,
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_note": "null: DRAM counters are taken under ncu, never in a timed run",
                      "peak_source": peaks["source"], "launch_us": dur_launch * 1e6},
@@ -651,24 +669,21 @@ def run_int8(args):
 
     peaks = read_peaks()
     passes = 1 if scale_V > 0 else 2
-    names = ["input_transform_int8 (%d pass%s)" % (passes, "" if passes == 1 else "es"), "product_tcgen05_i8",
-             "output_transform_dequant"]
-    # algorithmic work per step of each kernel class; the int8 tensor peak is twice the measured
-    # bf16 one (nominal ratio of the dense peaks)
-    alg = [("hbm", passes * 2.0 * c.N * c.H * c.W * c.C + 1.0 * n2 * P * c.C),
-           ("tensor", actual),
-           ("hbm", 4.0 * n2 * P * c.K + 2.0 * c.N * c.H * c.W * c.K)]
-    dom = max(range(3), key=lambda i: kms[i])
-    bound, work = alg[dom]
-    dur = kms[dom] * 1e-3
+    # the int8 tensor peak is twice the measured bf16 one (nominal ratio of the dense peaks)
     i8_peak = 2.0 * peaks["tflops_burst"]
+    launches = plan.int8_launch_count(c.N, c.H, c.W, c.C, c.K, scale_V)
+    separate = plan.int8_launch_count(c.N, c.H, c.W, c.C, c.K, scale_V, nv.GEMM_TCGEN05)
+    classes = kernel_classes(3 if launches == separate else 2, kms[:3], actual, passes * 2.0 * c.N * c.H * c.W * c.C,
+                             1.0 * n2 * P * c.C, 4.0 * n2 * P * c.K, 2.0 * c.N * c.H * c.W * c.K, i8_peak, peaks["hbm_gbs"],
+                             "product_tcgen05_i8", "input_transform_int8 (%d pass%s)" % (passes, "" if passes == 1 else "es"),
+                             "output_transform_dequant")
+    dom_name, dom_ms, bound, work = max(classes, key=lambda k: k[1])
+    dur = dom_ms * 1e-3
     if bound == "tensor":
         achieved, peak, runit = work / dur / 1e12, i8_peak, "TOP/s"
     else:
         achieved, peak, runit = work / dur / 1e9, peaks["hbm_gbs"], "GB/s"
     roof_s = max(actual / (i8_peak * 1e12), min_bytes / (peaks["hbm_gbs"] * 1e9))
-    # input transform once or twice, product, output transform; the CUDA-core input transform has a scale kernel besides
-    launches = (4 if scale_V == 0 else 3) + (1 if args.int8_coef == "fp32" else 0)
     out = {
         "metric": METRIC.replace("fp16", "int8"), "value": whole_job_value(world, direct, ms_per_step), "unit": UNIT,
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
@@ -686,9 +701,9 @@ def run_int8(args):
         "tops_actual": world * actual / (ms_per_step * 1e-3) / 1e12,
         "path_roofline": {"roofline_us": roof_s * 1e6, "achieved_us": ms_per_step * 1e3,
                           "frac": roof_s / (ms_per_step * 1e-3), "peaks": peaks["source"] + "; int8 tensor peak = 2 x bf16"},
-        "kernels_ms_per_step": dict(zip(names, kms[:3])),
+        "kernels_ms_per_step": {k[0]: k[1] for k in classes},
         "filter_transform_ms": filter_ms,
-        "roofline": {"kernel": names[dom], "bound": bound, "achieved": achieved, "peak": peak, "unit": runit,
+        "roofline": {"kernel": dom_name, "bound": bound, "achieved": achieved, "peak": peak, "unit": runit,
                      "frac": achieved / peak, "traffic": None, "peak_source": peaks["source"], "launch_us": dur * 1e6},
         "e2e": {"value": world * direct / (e2e_ms * 1e-3) / 1e12, "unit": UNIT, "ms_per_step": e2e_ms,
                 "h2d_bytes_per_step": int(x_np.nbytes), "d2h_bytes_per_step": int(yh.numel() * 2)},

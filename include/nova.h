@@ -53,7 +53,7 @@ enum { NOVA_COEF_ROUND_TO_MODE = 0, NOVA_COEF_FP32 = 1 };
 /* nova_conv2d_fwd flags (bitwise or). */
 enum {
   NOVA_RELU = 1,            /* y = (v < 0) ? 0 : v after the output transform */
-  NOVA_GEMM_SIMT = 1 << 8,  /* force the CUDA-core product kernel (fp16 mode; testing) */
+  NOVA_GEMM_SIMT = 1 << 8,  /* force the CUDA-core product kernel (testing); fp32 mode: the separate kernels */
   NOVA_GEMM_TCGEN05 = 2 << 8, /* force the tcgen05 tensor-core product kernel */
   NOVA_PROFILE_WAITS = 1 << 13, /* measurement aid: the tensor-core product kernel (half mode, K > 128) runs in a
                                    variant that sums the cycles its warps spend waiting; read them with
@@ -66,7 +66,7 @@ enum {
                                the INT8 entry points */
   NOVA_TRANSFORM_SIMT = 1 << 10 /* plain transform kernels: the input transform on CUDA cores even
                                    where the tensor-core formulation applies, the output transform
-                                   without TMA staging (testing) */
+                                   without TMA staging (testing); fp32 mode: the separate kernels */
 };
 
 /* How nova_filter_transform_int8 obtains the scales of the transformed filter. */
@@ -222,7 +222,11 @@ size_t nova_conv2d_min_workspace_bytes(const nova_plan* plan, int N, int H, int 
  * With C = 8 (NOVA_FP16_F32ACC, 3-tap filters, none of NOVA_GEMM_SIMT, NOVA_GEMM_TCGEN05,
  * NOVA_TRANSFORM_SIMT, NOVA_PROFILE_WAITS) the three steps run in ONE kernel that keeps V and M
  * on the SM: same arithmetic and rounding points, one launch, workspace checked but not touched
- * (problems of 2^31 tiles or more stay on the three-kernel path).
+ * (problems of 2^31 tiles or more stay on the three-kernel path).  The same holds for the fp32 mode with
+ * up to 8 points and neither NOVA_GEMM_SIMT nor NOVA_TRANSFORM_SIMT.  In half mode with up to 8 points, layers
+ * of few channels and a large M run the product and the output transform in one kernel (same bits), which needs V
+ * alone; this path too is taken only with nova_conv2d_workspace_bytes() or more, a smaller workspace
+ * (nova_conv2d_fwd_static's for a large problem) gets the chunked three kernels.
  */
 int nova_conv2d_fwd(const nova_plan* plan, const void* x_dev, const void* U_dev, void* y_dev,
                     int N, int H, int W, int C, int K,
@@ -296,6 +300,8 @@ int nova_conv2d_fwd_static(const nova_plan* plan, const void* x_dev, const void*
  * and workspace size (negative = error). */
 int nova_conv2d_launch_count(const nova_plan* plan, int N, int H, int W, int C, int K,
                              size_t workspace_bytes, int flags);
+/* The same for one nova_conv2d_fwd_int8 call (scale_V as there: 0 derives it from the data). */
+int nova_conv2d_int8_launch_count(const nova_plan* plan, int N, int H, int W, int C, int K, float scale_V, int flags);
 
 /*
  * INT8 Winograd-domain pipeline (Section 5.1 "INT8 Setup"; appendix "INT8 Convolution Error

@@ -24,7 +24,7 @@ EXPORTED_SYMBOLS = (
     "nova_plan_get_matrices_rational", "nova_plan_kappa_matrices", "nova_symmetric_search",
     "nova_selftest_wait_timeout", "nova_probe_fabric", "nova_plan_wait_profile",
     "nova_filter_transform_int8_bytes", "nova_filter_transform_int8", "nova_conv2d_int8_workspace_bytes",
-    "nova_conv2d_fwd_int8", "nova_conv2d_fwd_int8_timed",
+    "nova_conv2d_fwd_int8", "nova_conv2d_fwd_int8_timed", "nova_conv2d_int8_launch_count",
 )
 QUANT_PER_TENSOR, QUANT_PER_CHANNEL, QUANT_GIVEN = 0, 1, 2
 STATIC_SCRATCH_BYTES = 32 << 20
@@ -118,6 +118,8 @@ def lib():
     L.nova_conv2d_fwd_int8_timed.restype = i
     L.nova_conv2d_launch_count.argtypes = [vp, i, i, i, i, i, sz, i]
     L.nova_conv2d_launch_count.restype = i
+    L.nova_conv2d_int8_launch_count.argtypes = [vp, i, i, i, i, i, cf, i]
+    L.nova_conv2d_int8_launch_count.restype = i
     L.nova_maxpool2x2.argtypes = [vp, vp, i, i, i, i, i, vp]
     L.nova_maxpool2x2.restype = i
     L.nova_last_device_status.argtypes = [vp, vp]
@@ -436,6 +438,9 @@ class Plan:
 
     def int8_workspace_bytes(self, N, H, W, C, K):
         return lib().nova_conv2d_int8_workspace_bytes(self._h, N, H, W, C, K)
+
+    def int8_launch_count(self, N, H, W, C, K, scale_V=0.0, flags=0):
+        return lib().nova_conv2d_int8_launch_count(self._h, N, H, W, C, K, float(scale_V), flags)
 
     def conv2d_int8(self, x, Uq, scale_U, scale_V=0.0, y=None, workspace=None, flags=0, timed=False):
         """x [N,H,W,C] half -> y [N,H,W,K] half.  scale_V = 0 derives the input scale from the data.

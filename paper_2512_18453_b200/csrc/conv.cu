@@ -452,6 +452,10 @@ Int8Layout int8_layout(const Geom& g) {
   return l;
 }
 
+bool two_kernels_int8(const nova_plan* p, const Geom& g, int flags) {
+  return !(flags & kThreeKernelFlags) && use_product_output(p, g, true);
+}
+
 int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const float* scale_U, float scale_V,
                      void* y, int N, int H, int W, int C, int K, void* ws, size_t ws_bytes, int flags,
                      nova_stream stream, cudaEvent_t* ev) {
@@ -476,7 +480,7 @@ int conv2d_int8_impl(const nova_plan* p, const void* x, const void* Uq, const fl
   // The tensor-core transform needs the exact hi + lo table of half-rounded coefficients; plans
   // with float32 coefficients (and narrow layers) use the CUDA-core transform.
   const bool tc_in = tensor_core_input(p, g, flags);
-  const bool two = use_product_output(p, g, true) && !(flags & kThreeKernelFlags);
+  const bool two = two_kernels_int8(p, g, flags);
   if (two && tc_in) g.ldv = padded_pitch(p->n, C, 1);           // into the room of M, which is not used then
   if (ev) cudaEventRecord(ev[0], s);
   // s_V is given, or max|V| / 127 over the batch, which costs one more pass of the input transform
@@ -544,6 +548,15 @@ extern "C" int nova_conv2d_fwd_int8(const nova_plan* p, const void* x, const voi
                                     float scale_V, void* y, int N, int H, int W, int C, int K, void* ws,
                                     size_t ws_bytes, int flags, nova_stream stream) {
   return conv2d_int8_impl(p, x, Uq, scale_U, scale_V, y, N, H, W, C, K, ws, ws_bytes, flags, stream, nullptr);
+}
+
+extern "C" int nova_conv2d_int8_launch_count(const nova_plan* p, int N, int H, int W, int C, int K, float scale_V, int flags) {
+  if (!p || !(scale_V >= 0.f)) return NOVA_ERR_INVALID_ARG;
+  if (!int8_shape_ok(p, N, H, W, C, K)) return p->mode != NOVA_FP16_F32ACC || !device_plan(p) ? NOVA_ERR_UNSUPPORTED : NOVA_ERR_INVALID_ARG;
+  const Geom g = make_geom(p, N, H, W, C, K);
+  // the tensor-core input transform carries the scale itself; the CUDA-core one has a kernel that sets it
+  const int input = (scale_V > 0.f ? 1 : 2) + (tensor_core_input(p, g, flags) ? 0 : 1);
+  return input + (two_kernels_int8(p, g, flags) ? 1 : 2);
 }
 
 extern "C" int nova_conv2d_fwd_int8_timed(const nova_plan* p, const void* x, const void* Uq, const float* scale_U,

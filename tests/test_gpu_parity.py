@@ -1374,6 +1374,16 @@ def test_product_and_output_in_one_kernel_by_blocks_and_chunks(op, m, key, r, sh
         assert torch.equal(y.view(torch.int16), ys[3].view(torch.int16))
 
 
+def test_int8_launch_count_follows_the_path():
+    large, small = (2, 104, 106, 112, 528), (1, 20, 20, 112, 48)
+    plan = nv.Plan(4, point_set("dyadic", 4))
+    assert plan.int8_launch_count(*large) == 3                       # two passes, product and output in one kernel
+    assert plan.int8_launch_count(*large, 0.02) == 2
+    assert plan.int8_launch_count(*large, 0.0, nv.GEMM_TCGEN05) == 4
+    assert plan.int8_launch_count(*small) == 4
+    assert nv.Plan(4, point_set("dyadic", 4), coef=nv.COEF_FP32).int8_launch_count(*small) == 5
+
+
 def test_pooled_output_through_the_int8_and_host_entry_points():
     m, N, H, W, C, K = 4, 3, 20, 24, 64, 80
     x, g = make_conv_inputs(N, H, W, C, K, "fp16", True, True, seed=421)
