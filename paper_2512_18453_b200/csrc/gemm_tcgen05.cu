@@ -197,7 +197,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_consta
         if (!mbar_wait_warp(&full_bar[stage], phase, abort_flag)) { timed_out = true; break; }
         w_ops.stop();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (lane == 0) {
+        if (elect_one()) {
           const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
           const uint32_t sb = sa + L::kABytes;
           const uint64_t ad0 = umma_desc_sw128(sa), bd0 = umma_desc_sw128(sb);

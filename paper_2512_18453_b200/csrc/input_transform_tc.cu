@@ -98,7 +98,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
 // pass's qparts / 127 where qgiven is 0, and is left in *qslot for the output transform.  (A cleared
 // word, atomics and a kernel that made the scale of it were two more launches per call, and neither
 // could overlap its neighbours.)
-// LO: the table has a part lo (see above).  A variant, not a branch: the issue of a unit's MMAs is straight-line code.
+// LO: the table has a part lo (see above).
 template <int M, int QMODE, int R, bool LO>
 __global__ void __launch_bounds__(kTcThreads, 1)
 input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmKron,
@@ -217,7 +217,7 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
       if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1, abort_flag)) { timed_out = true; break; }
       if (!mbar_wait_warp(&full_bar[stage], phase, abort_flag)) { timed_out = true; break; }
       tc_fence_after();
-      if (lane == 0) {
+      if (elect_one()) {
         const uint32_t sa = smem_u32(ring + (size_t)stage * Cfg::kStageBytes);
         const uint32_t tmem_d = tmem_base + acc * kAccCols;
         const uint64_t ad0 = umma_desc_mn_sw128(sa, Cfg::kHalfBytes);

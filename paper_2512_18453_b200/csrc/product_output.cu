@@ -275,7 +275,8 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
       // ---------------- MMA issuers: one thread of warp 1 + e issues the columns nu of parity e.  (One issuer alone
       // took 660 cycles per stage, more than the loads.)
       pdl_wait();
-      if (lane == 0) {
+      __syncwarp();
+      if (elect_one()) {
         const int e = warp - 1;
         const uint32_t idesc = I8 ? umma_idesc_i8(kRows, F) : umma_idesc_f16(kRows, F);
         const uint64_t desc0 = umma_desc_sw128(smem_u32(smem) + Cfg::kOffRing + e * args.box_rows * kRowBytes);

@@ -104,6 +104,15 @@ __device__ __forceinline__ void settle_after_timeout() {
   for (int i = 0; i < 4096 && global_ns() - t0 < 1000000ull; ++i) __nanosleep(2000);
 }
 
+// The thread of a (converged) warp that issues its MMAs and commits: always the same one.  Their operands are the warp's,
+// not the thread's, and a comparison of the lane's number does not tell the compiler that: with a branch between the MMAs
+// of such a region the input transform gave wrong results (rel-L2 0.3 to 0.9, no barrier passed twice), with elect.sync the
+// same branch gives the bits of straight-line code.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one != 0;
+}
 // Fetch a tensor map ahead of its first use, which would otherwise wait for it.  A kernel parameter
 // may be fetched before the wait for the preceding kernel.
 __device__ __forceinline__ void tma_prefetch(const CUtensorMap* map) {

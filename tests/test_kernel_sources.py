@@ -34,3 +34,12 @@ def test_kernels_with_bounded_waits_let_their_copies_land(path):
     text = code(path)
     if re.search(r"tma_load_\w+\(|bulk_g2s\(|umma_\w+\(", text):
         assert "settle_after_timeout();" in text
+
+
+@pytest.mark.parametrize("path", [p for p in SOURCES if p.endswith(".cu")], ids=os.path.basename)
+def test_mmas_are_issued_by_the_elected_thread(path):
+    # the block that an MMA stands in is entered by elect.sync, not by a comparison of the lane's number
+    text = code(path)
+    for m in re.finditer(r"\bumma_(f16|f16_c<\w+>|i8|commit)\(", text):
+        entered = re.findall(r"if \((lane == 0|elect_one\(\))\) \{", text[:m.start()])
+        assert entered and entered[-1] == "elect_one()", text[m.start() - 200:m.end()]
