@@ -395,12 +395,14 @@ int build_kron_table(const nova_plan* plan, unsigned short* out) {
         for (int b = 0; b < n; ++b) {
           const int f = xi * n + nu, k = a * n + b;
           const double prod = (double)plan->kcoefs.BT[xi][a] * (double)plan->kcoefs.BT[nu][b];
+          if (prod == 0.0) continue;
           const __half hi = __double2half(prod);
           const double hid = (double)__half2float(hi);
           if (!(hid - hid == 0.0)) return -1;                        // hi is not finite
           const __half lo = __double2half(prod - hid);
-          largest = fmax(largest, fabs(prod));
-          missed = fmax(missed, fabs(prod - hid - (double)__half2float(lo)));
+          const double size = fabs(prod), miss = fabs(prod - hid - (double)__half2float(lo));
+          if (size > largest) largest = size;
+          if (miss > missed) missed = miss;
           const size_t at = ((size_t)(k / 64) * kp + f) * 64 + (k % 64);
           out[at] = __half_as_ushort(hi);
           out[(size_t)ka * kp * 64 + at] = __half_as_ushort(lo);
