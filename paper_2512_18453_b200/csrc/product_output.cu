@@ -18,8 +18,8 @@
 //   warps 1, 2    tcgen05.mma (M = 128, N = F), accumulator nu at column nu * F; two sets of accumulators where 512
 //                 columns hold them
 //   warps 4-11    row transform, two groups that take alternate slices of 16 filters: tcgen05.ld of the n
-//                 accumulators, A^T along nu, stores into the owner CTA's exchange buffer (one of two)
-//   the rest      finish, one group per exchange buffer, a warp per 4 of the CTA's own tiles: A^T along xi, y (or the
+//                 accumulators, A^T along nu, stores into the owner CTA's exchange buffers (two or four, in turn)
+//   the rest      finish, two groups that take alternate slices, a warp per 4 of the CTA's own tiles: A^T along xi, y (or the
 //                 pooled y)
 // The arithmetic and its order are the three-kernel path's, so the results are the same bits.
 // Every wait is bounded by the clock; after one has expired no role of the CTA waits any more and all run to their end.
@@ -40,7 +40,6 @@ using namespace xf;
 constexpr int kRows = 128;             // tiles of a block: TMEM lanes
 constexpr int kRowBytes = 128;         // one swizzle row of channels per stage: 64 halves or 128 int8
 constexpr int kUmmaBytes = 32;
-constexpr int kMaxF = 64;
 constexpr int kSliceF = 16;            // filters exchanged at a time
 constexpr int kVBytes = kRows * kRowBytes;
 
@@ -59,22 +58,28 @@ struct PoCfg {
   static constexpr int kFinishRegs = (N == 4) ? 72 : (N == 6) ? 80 : 128;
   static_assert(128 * kIssueRegs + 256 * kRowRegs + 64 * kFinish * kFinishRegs <= kThreads * kLaunchRegs, "register split");
   static constexpr int kOffZ = 0;
-  static constexpr int kOffRing = 2 * kBuf;
-  static_assert(kOffRing % 1024 == 0, "swizzled operands");
+  static_assert(2 * kBuf % 1024 == 0, "swizzled operands");
   // A stage holds the operands of two columns nu, one per MMA issuer; each issuer uses every stage, so that no one
   // gets two phases ahead of a barrier that it waits on by parity.
   static constexpr int stage_bytes(int F) { return 2 * (kVBytes + F * kRowBytes); }
-  static constexpr int stages(int F) {
-    return (232448 - kOffRing - 2048) / stage_bytes(F) < 4 ? (232448 - kOffRing - 2048) / stage_bytes(F) : 4;
+  static constexpr int stages(int F, int bufs) {
+    return (232448 - bufs * kBuf - 2048) / stage_bytes(F) < 4 ? (232448 - bufs * kBuf - 2048) / stage_bytes(F) : 4;
   }
-  static constexpr int total(int F) { return kOffRing + stages(F) * stage_bytes(F) + 256 + 1024; }
-  static_assert(total(kMaxF) <= 227 * 1024 && stages(kMaxF) >= 2, "shared memory of one CTA");
+  static constexpr int total(int F, int bufs) { return bufs * kBuf + stages(F, bufs) * stage_bytes(F) + 256 + 1024; }
+  static constexpr int kMaxF = (N == 4) ? 64 : 32;               // see block_filters
+  static_assert(total(kMaxF, 2) <= 227 * 1024 && stages(kMaxF, 2) >= 2, "shared memory of one CTA");
+  // Exchange buffers: four for few channels, where the ring of operands can spare a stage.  With two, a row group waits for the
+  // buffer that it filled a slice ago to be read in all CTAs.  Whole call, two / four: F(2,3) 32 x 56 x 56, 128 -> 128 75.6 / 70.7 us,
+  // 32 x 112 x 112, 64 -> 64 136 / 133; F(4,3) 32 x 112 x 112, 64 -> 128 152.8 / 147.7, 8 x 112 x 112, 64 -> 256 75.3 / 70.9.  With more channels
+  // the stage is worth more: F(2,3) 8 x 56 x 56, 256 -> 64 29.4 / 30.2, F(4,3) 32 x 112 x 112, 128 -> 128 202 / 235, F(2,5) 8 x 56 x 56, 128 -> 256
+  // 66.1 / 69.9; with 8 points 32 x 56 x 56, 64 -> 128, F(4,5) 62.4 / 64.9.
+  static constexpr int bufs(int F, int num_ks) { return N <= 6 && num_ks <= (N == 4 ? 2 : 1) && stages(F, 4) >= 2 ? 4 : 2; }
 };
 
 struct PoArgs {
   int H, W, C, K, Th, Tw, pc, pc_pad;
   long long p0;
-  int F, num_kb, items, clusters, nacc, relu, stages, box_rows;
+  int F, num_kb, items, clusters, nacc, relu, stages, box_rows, bufs;
   uint32_t none;                       // 0, which the compiler does not know
 };
 
@@ -177,17 +182,18 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
                       const uint8_t* __restrict__ Vdrop) {
   using Cfg = PoCfg<M, R>;
   constexpr int N = Cfg::N;
+  const int bufs = args.bufs, off_ring = bufs * Cfg::kBuf;
   const int ST = args.stages, kStageBytes = 2 * (kVBytes + args.F * kRowBytes);
   constexpr int BLOCK_K = I8 ? kRowBytes : kRowBytes / 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + Cfg::kOffRing + ST * kStageBytes);
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + off_ring + ST * kStageBytes);
   uint64_t* empty_bar = full_bar + ST;
   uint64_t* tmem_full = empty_bar + ST;             // [2]
   uint64_t* tmem_empty = tmem_full + 2;             // [2]
-  uint64_t* z_full = tmem_empty + 2;                // [2] rows of all CTAs have arrived in the exchange buffer
-  uint64_t* z_free = z_full + 2;                    // [2] every owner has read its buffer
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(z_free + 2);
+  uint64_t* z_full = tmem_empty + 2;                // [4] rows of all CTAs have arrived in the exchange buffer
+  uint64_t* z_free = z_full + 4;                    // [4] every owner has read its buffer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(z_free + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -211,8 +217,10 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tmem_full[a], 2);
       mbar_init(&tmem_empty[a], 8);
-      mbar_init(&z_full[a], (uint32_t)(1 + my_oct));   // what the other CTAs send, and the own rows per owned octet
-      mbar_init(&z_free[a], (uint32_t)(N * Cfg::kFinish));
+    }
+    for (int b = 0; b < 4; ++b) {
+      mbar_init(&z_full[b], (uint32_t)(1 + my_oct));   // what the other CTAs send, and the own rows per owned octet
+      mbar_init(&z_free[b], (uint32_t)(N * Cfg::kFinish));
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -248,7 +256,7 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
           for (int ks = 0; ks < num_ks; ++ks) {
             wait_local(&empty_bar[stage], phase ^ 1, abort_flag);
             if (lane == 0 && !*abort_flag) {
-              uint8_t* dst = smem + Cfg::kOffRing + stage * kStageBytes;
+              uint8_t* dst = smem + off_ring + stage * kStageBytes;
               mbar_expect_tx(&full_bar[stage], tx);
               if (is_v) tma_load_3d(dst, &tmV, &full_bar[stage], ks * BLOCK_K, pb * kRows, (int)rank * N + nu);
               else tma_load_3d(dst + 2 * kVBytes, &tmU, &full_bar[stage], ks * BLOCK_K, kb * F, (int)rank * N + nu);
@@ -279,7 +287,7 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
       if (elect_one()) {
         const int e = warp - 1;
         const uint32_t idesc = I8 ? umma_idesc_i8(kRows, F) : umma_idesc_f16(kRows, F);
-        const uint64_t desc0 = umma_desc_sw128(smem_u32(smem) + Cfg::kOffRing + e * args.box_rows * kRowBytes);
+        const uint64_t desc0 = umma_desc_sw128(smem_u32(smem) + off_ring + e * args.box_rows * kRowBytes);
         const uint32_t b_off = (uint32_t)(2 * kVBytes - e * args.box_rows * kRowBytes + e * F * kRowBytes);
         uint32_t stage = 0, phase = 0;
         for (uint32_t local = 0; local < n_local; ++local) {
@@ -341,8 +349,8 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)(N * F);
       for (int s = 0; s < slices; ++s, ++gs) {
         if ((int)(gs & 1) != grp) continue;
-        const uint32_t b = gs & 1;
-        wait_cluster(&z_free[b], ((gs >> 1) & 1) ^ 1, abort_flag);
+        const uint32_t b = gs & (uint32_t)(bufs - 1);
+        wait_cluster(&z_free[b], ((gs & (uint32_t)bufs) ? 1u : 0u) ^ 1u, abort_flag);
         __syncwarp();                                // the loads of tensor memory are a whole warp's
         if (live) {
 #pragma unroll 1
@@ -385,25 +393,26 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
       if (lane == 0) mbar_arrive(&tmem_empty[acc]);
     }
   } else {
-    // ---------------- finish: group b reads exchange buffer b
+    // ---------------- finish: group e takes the slices whose running number is e modulo 2, hence always the same buffers
     set_registers<Cfg::kFinishRegs, Cfg::kLaunchRegs>();
-    const uint32_t b = warp - 12 >= Cfg::kFinish ? 1u : 0u;
-    const int w = warp - 12 - (int)b * Cfg::kFinish;
+    const uint32_t grp = warp - 12 >= Cfg::kFinish ? 1u : 0u;
+    const int w = warp - 12 - (int)grp * Cfg::kFinish;
     const int fp = lane & 7, tt = lane >> 3;
-    const uint32_t tell = peer(smem_u32(&z_free[b]), lane < N ? (uint32_t)lane : 0u);
+    const uint32_t tell = peer(smem_u32(z_free), lane < N ? (uint32_t)lane : 0u);
     pdl_wait();
     uint32_t gs = 0;
     for (uint32_t local = 0; local < n_local; ++local) {
       int pb, kb;
       item_of(local, pb, kb);
       for (int s = 0; s < slices; ++s, ++gs) {
-        if ((gs & 1) != b) continue;
+        if ((gs & 1) != grp) continue;
+        const uint32_t b = gs & (uint32_t)(bufs - 1);
         if (w == 0 && lane == 0) {                   // what the other CTAs send for the octets of this CTA that exist
           int live = 0;
           for (int slot = 0; slot < my_oct; ++slot) live += pb * kRows + (slot * N + (int)rank) * 8 < args.pc ? 1 : 0;
           mbar_expect_tx(&z_full[b], (uint32_t)(live * (N - 1) * M * 512));
         }
-        wait_cluster(&z_full[b], (gs >> 1) & 1, abort_flag);
+        wait_cluster(&z_full[b], (gs & (uint32_t)bufs) ? 1u : 0u, abort_flag);
         const int k = kb * F + s * kSliceF + 2 * fp;
         // a warp has 4 of the CTA's tiles x 16 filters (the last warps of a CTA that owns fewer octets have none)
         const int slot = w >> 1, t8 = (w & 1) * 4 + tt;
@@ -423,7 +432,7 @@ product_output_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_cons
             for (int j = 0; j < M; ++j) seen |= __float_as_uint(Y[i][j].x) | __float_as_uint(Y[i][j].y);
         }
         const bool unread = __any_sync(0xffffffffu, (seen & args.none) != 0u);
-        if (lane < N && !unread) arrive_peer(tell);
+        if (lane < N && !unread) arrive_peer(tell + b * 8);
         if (mine) {
           const unsigned p = (unsigned)(args.p0 + pl);
           const unsigned tw = p % (unsigned)args.Tw, q2 = p / (unsigned)args.Tw;
@@ -522,8 +531,9 @@ int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void*
   a.nacc = 2 * Cfg::N * F <= 512 ? 2 : 1;
   a.relu = relu;
   a.none = 0;
-  a.stages = Cfg::stages(F);
-  const int smem = Cfg::total(F);
+  a.bufs = Cfg::bufs(F, (g.C * (I8 ? 1 : 2) + kRowBytes - 1) / kRowBytes);
+  a.stages = Cfg::stages(F, a.bufs);
+  const int smem = Cfg::total(F, a.bufs);
   if (cudaError_t e = allow_dynamic_smem(kernel, smem); e != cudaSuccess) return (int)e;
   const int esize = I8 ? 1 : 2;
   const bool drop = a.num_kb == 1 && ((size_t)g.C * esize) % kRowBytes == 0 && (reinterpret_cast<uintptr_t>(V) % kRowBytes) == 0;

@@ -1344,6 +1344,11 @@ def test_product_and_output_in_one_kernel_give_the_bits_of_two(op, m, key, r, sh
     ("conv", 2, ("asym", 2), 3, (32, 56, 56, 72, 8), 2),
     ("conv", 4, ("nova", 4), 3, (32, 148, 148, 64, 16), 2),
     ("conv", 4, ("half", 6), 5, (8, 100, 100, 40, 16), 2),
+    # four exchange buffers and two of them, by the channels; blocks whose slices are no multiple of four
+    ("conv", 2, ("std", 2), 3, (8, 56, 56, 136, 48), 2),
+    ("conv", 2, ("nova", 4), 5, (8, 76, 76, 72, 48), 2),
+    ("conv", 4, ("asym", 4), 3, (32, 112, 112, 40, 48), 2),
+    ("int8", 4, ("dyadic", 4), 3, (32, 112, 112, 144, 48), 2),
     # two chunks of tiles
     ("conv", 2, ("std", 2), 3, (11, 162, 162, 512, 16), 4)])
 def test_product_and_output_in_one_kernel_by_blocks_and_chunks(op, m, key, r, shape, launches):
