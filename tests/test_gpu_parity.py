@@ -959,6 +959,27 @@ def test_int8_degenerate_inputs():
         assert conv.rel_l2(y, ref) <= 2.0 * conv.rel_l2(ye, ref) + 1e-6
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_int8_quantiser_with_the_datas_scale_gives_the_codes_of_the_same_scale_given(value):
+    # the pass with the data's own scale rounds by an addition, the one with a caller's scale by the saturating conversion;
+    # NaN becomes code 0 in both, and an infinity makes the scale infinite
+    plan = nv.Plan(4, point_set("dyadic", 4))
+    gen = torch.Generator(device="cuda").manual_seed(99)
+    x = torch.randn(2, 22, 19, 80, generator=gen, device="cuda").half()
+    g = (torch.randn(32, 3, 3, 80, generator=gen, device="cuda") * 0.05).half()
+    Uq, sU = plan.filter_transform_int8(g, nv.QUANT_PER_CHANNEL)
+    ws = torch.empty(plan.int8_workspace_bytes(2, 22, 19, 80, 32), dtype=torch.uint8, device="cuda")
+    for bad in (False, True):
+        if bad:
+            x[1, 7, 3, 5] = value
+        y = plan.conv2d_int8(x, Uq, sU, 0.0, workspace=ws)
+        scale = float(ws[:4].view(torch.float32)[0])
+        given = plan.conv2d_int8(x, Uq, sU, scale)
+        torch.cuda.synchronize()
+        assert plan.device_status() == 0 and (scale == float("inf")) == (bad and value == float("inf"))
+        assert torch.equal(y.view(torch.int16), given.view(torch.int16))
+
+
 # ---------------------------------------------------------------- 5 x 5 filters (F(2,5), F(4,5), F(6,5))
 R5_CASES = [(2, ("std", 4)), (4, ("std", 6)), (4, ("nova", 6)), (4, ("half", 6)), (6, ("nova", 8))]
 
