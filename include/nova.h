@@ -224,8 +224,9 @@ size_t nova_conv2d_min_workspace_bytes(const nova_plan* plan, int N, int H, int 
  * on the SM: same arithmetic and rounding points, one launch, workspace checked but not touched
  * (problems of 2^31 tiles or more stay on the three-kernel path).  The same holds for the fp32 mode with
  * up to 8 points and neither NOVA_GEMM_SIMT nor NOVA_TRANSFORM_SIMT.  In half mode with up to 8 points, layers
- * of few channels and a large M run the product and the output transform in one kernel (same bits), which needs V
- * alone; this path too is taken only with nova_conv2d_workspace_bytes() or more, a smaller workspace
+ * of few channels and a large M, and small layers (few tiles and channels), run the product and the output transform in
+ * one kernel (same bits), which needs V alone; small F(2,3) layers the input transform too.  These paths are taken
+ * only with nova_conv2d_workspace_bytes() or more, a smaller workspace
  * (nova_conv2d_fwd_static's for a large problem) gets the chunked three kernels.
  */
 int nova_conv2d_fwd(const nova_plan* plan, const void* x_dev, const void* U_dev, void* y_dev,
@@ -237,7 +238,7 @@ int nova_conv2d_fwd(const nova_plan* plan, const void* x_dev, const void* U_dev,
  * on `stream` around each kernel; synchronises the stream and writes the summed
  * device time in milliseconds of the three kernel classes to kernel_ms_host[0..2]
  * (input transform, transformed-domain product, output transform); the one-kernel
- * paths (C = 8 in half mode; fp32 mode with up to 8 points) report their time as the
+ * paths (C = 8 and small F(2,3) layers in half mode; fp32 mode with up to 8 points) report their time as the
  * product's and 0 for the transforms, and where product and output transform are one
  * kernel its time is the product's.
  */

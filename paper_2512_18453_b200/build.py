@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnova.so")
 # named for this interpreter's ABI: another one does not import it and goes through ctypes
 EXT = os.path.join(HERE, "_fastcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
-SOURCES = ["plan.cpp", "transforms.cu", "filter_transform.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "input_transform_n4.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "product_output.cu", "conv.cu"]
+SOURCES = ["plan.cpp", "transforms.cu", "filter_transform.cu", "gemm_simt.cu", "fp32_path.cu", "gemm_tcgen05.cu", "input_transform_tc.cu", "input_transform_n4.cu", "output_transform_tma.cu", "fabric_probe.cu", "fused_small_c.cu", "fused_fp32.cu", "product_output.cu", "few_tiles.cu", "conv.cu"]
 
 
 def _nvcc():

@@ -125,6 +125,13 @@ bool two_kernels(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags, 
   return true;
 }
 
+// The kernels of few_tiles.cu, for the same callers: 0, or few_tiles_blocks' variant.
+int few_tiles(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags) {
+  if (p->mode != NOVA_FP16_F32ACC || (flags & kThreeKernelFlags) || use_product_output(p, g, false)) return 0;
+  if (ws_bytes < nova_conv2d_workspace_bytes(p, g.N, g.H, g.W, g.C, g.K)) return 0;
+  return few_tiles_blocks(p, g);
+}
+
 bool use_tcgen05(const nova_plan* p, int flags) {
   if (p->mode == NOVA_FP32) return false;
   return (flags & NOVA_GEMM_SIMT) == 0;
@@ -177,7 +184,8 @@ extern "C" int nova_conv2d_launch_count(const nova_plan* p, int N, int H, int W,
   if (!choose_chunking(p, g, workspace_bytes, &c)) return NOVA_ERR_WORKSPACE;
   if (one_kernel(p, g, flags)) return 1;
   if (two_kernels(p, g, workspace_bytes, flags, &c)) return 2 * c.chunks;
-  return 3 * c.chunks;
+  const int few = few_tiles(p, g, workspace_bytes, flags);
+  return few > 10 ? 1 : few > 0 ? 2 * c.chunks : 3 * c.chunks;
 }
 
 namespace {
@@ -214,6 +222,16 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
   }
   const bool tc = use_tcgen05(p, flags);
   if (tc && !p->status_dev) return NOVA_ERR_CUDA;
+  const int few = few_tiles(p, g, ws_bytes, flags);
+  if (few > 10) {
+    if (ev) cudaEventRecord(ev[0], (cudaStream_t)stream);
+    if (int e = launch_few_tiles_n4(p, g, x, U, y, store_flags(flags), few - 10, stream)) {
+      g_last_cuda_error = e;
+      return NOVA_ERR_CUDA;
+    }
+    if (ev) cudaEventRecord(ev[1], (cudaStream_t)stream);
+    return NOVA_OK;
+  }
   const bool two = two_kernels(p, g, ws_bytes, flags, &c);
   g.ldv = c.ldv;
   char* Vb = static_cast<char*>(ws);
@@ -233,8 +251,9 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
                 : launch_input_transform(p, g, x, Vb, p0, pc, c.pc_pad, stream))
       return NOVA_ERR_CUDA;
     if (ev) cudaEventRecord(ev[4 * ci + 1], s);
-    if (two) {
-      if (int e = launch_product_output(p, g, Vb, U, y, p0, pc, c.pc_pad, store_flags(flags), stream)) {
+    if (two || few) {
+      if (int e = two ? launch_product_output(p, g, Vb, U, y, p0, pc, c.pc_pad, store_flags(flags), stream)
+                      : launch_few_tiles(p, g, Vb, U, y, p0, pc, c.pc_pad, store_flags(flags), few, stream)) {
         g_last_cuda_error = e;
         return NOVA_ERR_CUDA;
       }
@@ -283,7 +302,8 @@ extern "C" int nova_conv2d_fwd_timed(const nova_plan* p, const void* x, const vo
     return st1;
   }
   Chunking two;                      // two kernels per chunk: the second one's time is reported as the product's
-  const int chunks = two_kernels(p, make_geom(p, N, H, W, C, K), ws_bytes, flags, &two) ? two.chunks : launches / 3;
+  const Geom g = make_geom(p, N, H, W, C, K);
+  const int chunks = two_kernels(p, g, ws_bytes, flags, &two) ? two.chunks : launches / (few_tiles(p, g, ws_bytes, flags) ? 2 : 3);
   cudaEvent_t* ev = new cudaEvent_t[4 * chunks];
   for (int i = 0; i < 4 * chunks; ++i) cudaEventCreate(&ev[i]);
   int st = conv2d_fwd_impl(p, x, U, y, N, H, W, C, K, ws, ws_bytes, flags, stream, ev);

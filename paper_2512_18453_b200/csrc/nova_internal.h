@@ -130,6 +130,14 @@ int launch_fused_fp32(const nova_plan* plan, const Geom& g, const void* x, const
 bool use_product_output(const nova_plan* plan, const Geom& g, bool int8);
 int launch_product_output(const nova_plan* plan, const Geom& g, const void* V, const void* U, void* y, long long p0, int pc,
                           int pc_pad, int relu, void* stream, const float* scale_U = nullptr, const float* scale_V = nullptr);
+// Layers of few tiles and channels (half mode): product and output transform in one kernel without clusters, with 4 points the
+// input transform too.  few_tiles_blocks names the variant (0: none; above 10: input transform included), `blocks8` takes its
+// last digit.  V has rows of C.
+int few_tiles_blocks(const nova_plan* plan, const Geom& g);
+int launch_few_tiles(const nova_plan* plan, const Geom& g, const void* V, const void* U, void* y, long long p0, int pc, int pc_pad,
+                     int relu, int blocks8, void* stream);
+int launch_few_tiles_n4(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, int blocks8,
+                        void* stream);
 int launch_maxpool2x2(const void* x, void* y, int N, int H, int W, int C, int mode, void* stream);
 
 }  // namespace nova

@@ -1400,6 +1400,74 @@ def test_product_and_output_in_one_kernel_by_blocks_and_chunks(op, m, key, r, sh
         assert torch.equal(y.view(torch.int16), ys[3].view(torch.int16))
 
 
+# ---------------------------------------------------------------- layers of few tiles: merged kernels without clusters
+@pytest.mark.parametrize("m,key,r,shape,launches", [
+    # F(2,3), input transform included: blocks of 16 and of 32 filters
+    (2, ("std", 2), 3, (1, 1, 1, 16, 8), 1),             # one tile, one output
+    (2, ("asym", 2), 3, (1, 8, 8, 64, 24), 1),           # 16 tiles: one whole block; the second block of filters half there
+    (2, ("std", 2), 3, (1, 34, 2, 72, 40), 1),           # 17 tiles; 64 + 8 channels
+    (2, ("asym", 2), 3, (2, 30, 32, 56, 200), 1),        # 32 filters a block, the last one 8
+    (2, ("std", 2), 3, (3, 50, 90, 64, 16), 1),          # more blocks than SMs
+    # F(2,3), after the input transform: 32, 16 and 8 filters
+    (2, ("std", 2), 3, (2, 24, 24, 128, 136), 2), (2, ("asym", 2), 3, (1, 17, 23, 200, 24), 2), (2, ("std", 2), 3, (1, 10, 10, 328, 40), 2),
+    # F(4,3): 8, 16 and 32 filters; one, two and three pieces of 64 channels (the ring of four stages wraps)
+    (4, ("nova", 4), 3, (1, 3, 2, 16, 8), 2), (4, ("asym", 4), 3, (1, 16, 16, 64, 72), 2), (4, ("nova", 4), 3, (3, 38, 40, 24, 40), 2),
+    (4, ("dyadic", 4), 3, (2, 40, 36, 48, 296), 2), (4, ("nova", 4), 3, (8, 56, 56, 64, 64), 2), (4, ("asym", 4), 3, (4, 56, 56, 40, 64), 2),
+    (4, ("nova", 4), 3, (2, 20, 22, 72, 24), 2), (4, ("std", 4), 3, (2, 60, 60, 72, 40), 2), (4, ("nova", 4), 3, (3, 60, 60, 72, 72), 2),
+    (4, ("asym", 4), 3, (1, 60, 60, 136, 8), 2), (4, ("std", 4), 3, (4, 60, 60, 136, 16), 2),
+    # F(6,3), and 5 x 5 filters on 6 and 8 points
+    (6, ("nova", 6), 3, (1, 13, 7, 64, 16), 2), (6, ("asym", 6), 3, (2, 50, 44, 40, 136), 2), (6, ("half", 6), 3, (6, 60, 62, 128, 16), 2),
+    (6, ("nova", 6), 3, (3, 70, 70, 32, 72), 2), (6, ("nova", 6), 3, (3, 70, 70, 40, 136), 2), (6, ("asym", 6), 3, (3, 70, 70, 72, 72), 2),
+    (2, ("asym", 4), 5, (2, 13, 11, 72, 24), 2), (4, ("nova", 6), 5, (1, 33, 21, 16, 48), 2), (4, ("asym", 6), 5, (5, 32, 32, 88, 32), 2)])
+def test_few_tiles_kernels_give_the_bits_of_three(m, key, r, shape, launches):
+    # the same sums in the same order, of registers' mma.sync instead of tcgen05: bit for bit the separate kernels (which a
+    # flag names), plain and pooled, NaN and infinities included
+    N, H, W, C, K = shape
+    plan = nv.Plan(m, point_set(*key), r=r)
+    gen = torch.Generator(device="cuda").manual_seed(83 + m)
+    x = torch.randn(N, H, W, C, generator=gen, device="cuda").half()
+    g = (torch.randn(K, r, r, C, generator=gen, device="cuda") * (2.0 / (r * r * C)) ** 0.5).half()
+    U = plan.filter_transform(g)
+    nbytes = plan.workspace_bytes(N, H, W, C, K)
+    assert plan.launch_count(N, H, W, C, K, nbytes, nv.RELU) == launches
+    assert plan.launch_count(N, H, W, C, K, nbytes, nv.GEMM_TCGEN05) == 3
+    for bad in (None, float("inf"), float("nan")):
+        if bad is not None:
+            x[-1, H // 2, W // 2, C - 1] = bad
+        for flags in (0, nv.RELU) + ((nv.RELU | nv.POOL2X2,) if H % 2 == 0 and W % 2 == 0 else ()):
+            y = torch.full((N, H // 2, W // 2, K) if flags & nv.POOL2X2 else (N, H, W, K), 7.0, dtype=torch.float16, device="cuda")
+            got = plan.conv2d(x, U, y, flags=flags)
+            want = plan.conv2d(x, U, flags=flags | nv.GEMM_TCGEN05)
+            torch.cuda.synchronize()
+            assert plan.device_status() == 0
+            assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+            assert torch.isfinite(got.float()).all() == (bad is None)
+    y1 = conv.direct_conv_fp64(x[:1].nan_to_num(0, 0, 0).cpu().numpy(), g.cpu().numpy())
+    y = plan.conv2d(x[:1].nan_to_num(0, 0, 0).contiguous(), U).cpu().numpy()
+    assert conv.rel_l2(y, y1) < (0.1 if m + r - 1 == 8 else 0.02)
+
+
+def test_few_tiles_kernels_follow_each_other_and_other_layers_on_one_workspace():
+    # calls in a row without a wait between them, each fed by the one before, the filters made just before: the kernels start
+    # before their predecessor has ended
+    gen = torch.Generator(device="cuda").manual_seed(89)
+    chans, plans = (16, 64, 64, 40, 256, 24, 64), [nv.Plan(m, point_set("std", m)) for m in (2, 4, 2, 4, 4, 2)]
+    ws = torch.empty(max(p.workspace_bytes(2, 20, 24, a, b) for p, a, b in zip(plans, chans, chans[1:])), dtype=torch.uint8, device="cuda")
+    x = torch.randn(2, 20, 24, 16, generator=gen, device="cuda").half()
+    g = [(torch.randn(b, 3, 3, a, generator=gen, device="cuda") * (2.0 / (9 * a)) ** 0.5).half() for a, b in zip(chans, chans[1:])]
+    outs = []
+    for flags in (nv.RELU, nv.RELU | nv.GEMM_TCGEN05):
+        for _ in range(3):
+            a = x
+            for p, w in zip(plans, g):
+                a = p.conv2d(a, p.filter_transform(w), workspace=ws, flags=flags)
+            outs.append(a)
+    torch.cuda.synchronize()
+    assert all(p.device_status() == 0 for p in plans) and torch.isfinite(outs[0]).all()
+    for o in outs[1:]:
+        assert torch.equal(o.view(torch.int16), outs[0].view(torch.int16))
+
+
 def test_int8_launch_count_follows_the_path():
     large, small = (2, 104, 106, 112, 528), (1, 20, 20, 112, 48)
     plan = nv.Plan(4, point_set("dyadic", 4))
