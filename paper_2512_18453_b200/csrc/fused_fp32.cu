@@ -60,11 +60,16 @@ struct Fc32 {
   static constexpr int kVBytes = N * kVRow;
   static constexpr int kStage = N * F * kRowBytes;
   static constexpr int kZRow = N * kTiles * F * 8;
+  // Output rows that meet in shared memory at a time.  Row by row, in two buffers in turn, most product warps wait at a barrier
+  // per row: a block's end took as long as one of its chunks.  Whole call, row by row / this: F(4,3) 8 x 56 x 56, 64 -> 64 34.6 / 33.9 us,
+  // 3 x 46 x 46, 32 -> 32 9.9 / 9.1; F(6,3) 61 x 107, 32 -> 256 28.3 / 26.9.  Two output rows stay with it: 8 x 56 x 56, 64 -> 64, F(2,3) 55.8 / 58.7.
+  static constexpr int kZRows = (M == 2) ? 1 : (N == 8) ? 2 : M;
+  static_assert(M % kZRows == 0, "");
   static constexpr int kOffX = 0;
   static constexpr int kOffV = kOffX + kXBytes;
   static constexpr int kOffU = kOffV + 2 * kVBytes;
   static constexpr int kOffZ = kOffU + kStages * kStage;
-  static constexpr int kOffRec = kOffZ + 2 * kZRow;
+  static constexpr int kOffRec = kOffZ + (kZRows == 1 ? 2 : kZRows) * kZRow;
   static constexpr int kOffBar = kOffRec + kRecRing * kTiles * 16;
   static constexpr int kTotal = kOffBar + 8 * (2 * kStages + 2 + 4) + 16 + 128;
   static_assert(kTotal <= 227 * 1024, "shared memory of one CTA");
@@ -273,21 +278,44 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
       const int pairs = kTiles * (f_run >> 1);
       const FcRec* rc = rec + (it % kRecRing) * kTiles;
       if (split == 1) {
-        static_assert(kTiles * Cfg::F / 2 <= Cfg::kProductThreads, "one (tile, filter pair) per thread");
-        const int tl = threadIdx.x >> fp_log, fc = (threadIdx.x & ((f_run >> 1) - 1)) * 2;
-        const int k = kb * f_run + fc;
+        if constexpr (Cfg::kZRows == 1) {
+          static_assert(kTiles * Cfg::F / 2 <= Cfg::kProductThreads, "one (tile, filter pair) per thread");
+          const int tl = threadIdx.x >> fp_log, fc = (threadIdx.x & ((f_run >> 1) - 1)) * 2;
+          const int k = kb * f_run + fc;
 #pragma unroll
-        for (int i = 0; i < M; ++i) {
-          const uint32_t zr = zb + (i & 1) * Cfg::kZRow;
-          put_columns(zr, i);
-          product_sync();
-          if ((int)threadIdx.x < pairs && k < args.K) {
-            const FcRec rt = rc[tl];
-            Dbl2 in[N], yv[M];
+          for (int i = 0; i < M; ++i) {
+            const uint32_t zr = zb + (i & 1) * Cfg::kZRow;
+            put_columns(zr, i);
+            product_sync();
+            if ((int)threadIdx.x < pairs && k < args.K) {
+              const FcRec rt = rc[tl];
+              Dbl2 in[N], yv[M];
 #pragma unroll
-            for (int a = 0; a < N; ++a) in[a] = lds_d2(zr + (uint32_t)((a * kTiles + tl) * Cfg::F + (fc ^ ((tl & 3) << 3))) * 8);
-            at_apply<M, SYM, Dbl2, N>(cf, in, yv);
-            put_row<M>(i, yv, y + rt.ybase + k, rt, args);
+              for (int a = 0; a < N; ++a) in[a] = lds_d2(zr + (uint32_t)((a * kTiles + tl) * Cfg::F + (fc ^ ((tl & 3) << 3))) * 8);
+              at_apply<M, SYM, Dbl2, N>(cf, in, yv);
+              put_row<M>(i, yv, y + rt.ybase + k, rt, args);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int i0 = 0; i0 < M; i0 += Cfg::kZRows) {
+            product_sync();         // the rows before have been read
+#pragma unroll
+            for (int r = 0; r < Cfg::kZRows; ++r) put_columns(zb + r * Cfg::kZRow, i0 + r);
+            product_sync();
+            for (int u = threadIdx.x; u < pairs * Cfg::kZRows; u += Cfg::kProductThreads) {
+              const int r = u >> (fp_log + 3), idx = u & (pairs - 1);
+              const int tl = idx >> fp_log, fc = (idx & ((f_run >> 1) - 1)) * 2;
+              const int k = kb * f_run + fc;
+              if (k >= args.K) continue;
+              const FcRec rt = rc[tl];
+              Dbl2 in[N], yv[M];
+#pragma unroll
+              for (int a = 0; a < N; ++a)
+                in[a] = lds_d2(zb + (uint32_t)r * Cfg::kZRow + (uint32_t)((a * kTiles + tl) * Cfg::F + (fc ^ ((tl & 3) << 3))) * 8);
+              at_apply<M, SYM, Dbl2, N>(cf, in, yv);
+              put_row<M>(i0 + r, yv, y + rt.ybase + k, rt, args);
+            }
           }
         }
       } else {
