@@ -394,9 +394,10 @@ FtArgs make_args(const Geom& g, long long p0, int pc, int pc_pad, int relu, int 
   return a;
 }
 
+constexpr int kOwnSm = 120 * 1024;
 // Shared memory that keeps two CTAs off one SM while another SM has none.  Without it CTAs that become resident while the
 // input transform still runs share SMs: F(4,3), 2 x 26 x 20, 344 -> 104, 65 CTAs 27.7 / 13.4 us; 4 x 97 x 37, 184 -> 16 21.1 / 12.9.
-int own_sm(int bytes, int grid, int sms) { return bytes < 120 * 1024 && grid <= sms ? 120 * 1024 : bytes; }
+int own_sm(int bytes, int grid, int sms) { return bytes < kOwnSm && grid <= sms ? kOwnSm : bytes; }
 
 template <int M, int R, bool SYM, int NB>
 int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void* y, long long p0, int pc, int pc_pad, int relu, cudaStream_t s) {
@@ -404,14 +405,14 @@ int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void*
   const auto kernel = few_tiles_kernel<M, R, SYM, NB>;
   const FtArgs a = make_args(g, p0, pc, pc_pad, relu, Cfg::KB);
   const int grid = (pc + kT - 1) / kT * a.num_kb, smem = own_sm(Cfg::kTotal, grid, plan->sm_count);
-  if (cudaError_t e = allow_dynamic_smem(kernel, smem); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<(Cfg::kTotal > kOwnSm ? Cfg::kTotal : kOwnSm)>(kernel); e != cudaSuccess) return (int)e;
   return (int)launch_overlapped(kernel, grid, Cfg::kThreads, smem, s, plan->kcoefs, (const __half*)V, (const __half*)U, (__half*)y, a);
 }
 template <bool SYM, int NB>
 int go_n4(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, cudaStream_t s) {
   using Cfg = N4Cfg<NB>;
   const auto kernel = few_tiles_n4_kernel<SYM, NB>;
-  if (cudaError_t e = allow_dynamic_smem(kernel, Cfg::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<Cfg::kTotal>(kernel); e != cudaSuccess) return (int)e;
   const FtArgs a = make_args(g, 0, (int)g.P, (int)g.P, relu, Cfg::KB);
   const int grid = ((int)g.P + kT - 1) / kT * a.num_kb;
   return (int)launch_overlapped(kernel, grid, Cfg::kThreads, Cfg::kTotal, s, plan->kcoefs, (const __half*)x, (const __half*)U, (__half*)y, a);

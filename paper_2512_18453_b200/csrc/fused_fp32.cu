@@ -491,7 +491,7 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return (int)cudaErrorUnknown;
   }
-  if (cudaError_t e = allow_dynamic_smem(kernel, Cfg::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<Cfg::kTotal>(kernel); e != cudaSuccess) return (int)e;
   FcArgs a;
   a.H = g.H; a.W = g.W; a.K = g.K; a.Th = g.Th; a.Tw = g.Tw;
   a.P = g.P;

@@ -395,7 +395,7 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return (int)cudaErrorUnknown;
-  if (cudaError_t e = allow_dynamic_smem(fused_small_c_kernel<M, GT, SYM>, L::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<L::kTotal>(fused_small_c_kernel<M, GT, SYM>); e != cudaSuccess) return (int)e;
   const int num_kb = (g.K + kFilterBlock - 1) / kFilterBlock;
   const long long groups = (g.P + L::kGroupTiles - 1) / L::kGroupTiles;
   long long per_kb = plan->sm_count / num_kb;

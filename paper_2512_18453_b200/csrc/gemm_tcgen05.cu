@@ -362,8 +362,9 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
   const bool lean = nfreq <= 16 && BLOCK_N < 256;
   const int stages = lean ? (BLOCK_N == 64 ? 4 : 3) : L::kMaxStages;
   size_t smem = (size_t)L::total(stages);
+  static_assert(L::total(L::kMaxStages) >= 118 * 1024, "the attribute below covers the padding");
   if (lean && smem < 118 * 1024) smem = 118 * 1024;
-  if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8>, (int)smem); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<L::total(L::kMaxStages)>(gemm_tcgen05_kernel<BLOCK_N, I8>); e != cudaSuccess) return (int)e;
   CUtensorMap tmV, tmU;
   const CUtensorMapDataType dt = I8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   constexpr int esize = I8 ? 1 : 2;
@@ -397,7 +398,7 @@ int launch_n(int sms, int l2_bytes, const void* V, const void* U, float* M, int 
   // the wait-profiling variant exists for the half product with 256-wide filter blocks only
   if constexpr (BLOCK_N == 256 && !I8) {
     if (prof) {
-      if (cudaError_t e = allow_dynamic_smem(gemm_tcgen05_kernel<BLOCK_N, I8, true>, (int)smem); e != cudaSuccess) return (int)e;
+      if (cudaError_t e = allow_dynamic_smem<L::total(L::kMaxStages)>(gemm_tcgen05_kernel<BLOCK_N, I8, true>); e != cudaSuccess) return (int)e;
       // CTAs beyond this launch's grid must read as "did not run"
       if (cudaError_t e = cudaMemsetAsync(prof, 0, sizeof(unsigned long long) * 8 * sms, stream); e != cudaSuccess) return (int)e;
       return (int)launch_overlapped(gemm_tcgen05_kernel<BLOCK_N, I8, true>, grid, kThreads, smem, stream, tmV, tmU, M,

@@ -356,7 +356,7 @@ int launch_m(const nova_plan* plan, const Geom& g, const void* x, void* V, long 
              float* qslot, float* qparts, float qgiven, cudaStream_t stream) {
   using Cfg = TcCfg<M, R>;
   const auto kernel = plan->kron_lo ? input_transform_tc_kernel<M, QMODE, R, true> : input_transform_tc_kernel<M, QMODE, R, false>;
-  if (cudaError_t e = allow_dynamic_smem(kernel, Cfg::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<Cfg::kTotal>(kernel); e != cudaSuccess) return (int)e;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return (int)cudaErrorUnknown;
   CUtensorMap tmX, tmK;

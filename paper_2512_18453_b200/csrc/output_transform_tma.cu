@@ -166,7 +166,7 @@ template <int M, typename T, bool SYM, int VEC, bool QUANT, int R = 3>
 int launch_one(const nova_plan* plan, const Geom& g, const CUtensorMap& tmM, const float* Mb, void* y, long long p0, int pc,
                int pc_pad, int relu, const float* scale_U, const float* scale_V, cudaStream_t stream) {
   using Cfg = OtCfg<M, VEC, R>;
-  if (cudaError_t e = allow_dynamic_smem(output_transform_tma_kernel<M, T, SYM, VEC, QUANT, R>, Cfg::kTotal); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<Cfg::kTotal>(output_transform_tma_kernel<M, T, SYM, VEC, QUANT, R>); e != cudaSuccess) return (int)e;
   const long long units = (long long)((pc + 7) / 8) * ((g.K + 16 * VEC - 1) / (16 * VEC));
   const int grid = (int)(units < plan->sm_count ? units : plan->sm_count);
   return (int)launch_overlapped(output_transform_tma_kernel<M, T, SYM, VEC, QUANT, R>, grid, kOtThreads, Cfg::kTotal,

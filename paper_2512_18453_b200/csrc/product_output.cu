@@ -67,7 +67,9 @@ struct PoCfg {
   }
   static constexpr int total(int F, int bufs) { return bufs * kBuf + stages(F, bufs) * stage_bytes(F) + 256 + 1024; }
   static constexpr int kMaxF = (N == 4) ? 64 : 32;               // see block_filters
-  static_assert(total(kMaxF, 2) <= 227 * 1024 && stages(kMaxF, 2) >= 2, "shared memory of one CTA");
+  static constexpr int kMaxTotal = 227 * 1024;                   // stages() fills up to it, whatever F and the buffers
+  static_assert(total(kMaxF, 2) <= kMaxTotal && total(kMaxF, 4) <= kMaxTotal && total(16, 2) <= kMaxTotal && total(16, 4) <= kMaxTotal &&
+                total(32, 2) <= kMaxTotal && total(32, 4) <= kMaxTotal && stages(kMaxF, 2) >= 2, "shared memory of one CTA");
   // Exchange buffers: four for few channels, where the ring of operands can spare a stage.  With two, a row group waits for the
   // buffer that it filled a slice ago to be read in all CTAs.  Whole call, two / four: F(2,3) 32 x 56 x 56, 128 -> 128 75.6 / 70.7 us,
   // 32 x 112 x 112, 64 -> 64 136 / 133; F(4,3) 32 x 112 x 112, 64 -> 128 152.8 / 147.7, 8 x 112 x 112, 64 -> 256 75.3 / 70.9.  With more channels
@@ -534,7 +536,7 @@ int go(const nova_plan* plan, const Geom& g, const void* V, const void* U, void*
   a.bufs = Cfg::bufs(F, (g.C * (I8 ? 1 : 2) + kRowBytes - 1) / kRowBytes);
   a.stages = Cfg::stages(F, a.bufs);
   const int smem = Cfg::total(F, a.bufs);
-  if (cudaError_t e = allow_dynamic_smem(kernel, smem); e != cudaSuccess) return (int)e;
+  if (cudaError_t e = allow_dynamic_smem<Cfg::kMaxTotal>(kernel); e != cudaSuccess) return (int)e;
   const int esize = I8 ? 1 : 2;
   const bool drop = a.num_kb == 1 && ((size_t)g.C * esize) % kRowBytes == 0 && (reinterpret_cast<uintptr_t>(V) % kRowBytes) == 0;
   cudaLaunchConfig_t cfg = {};

@@ -25,12 +25,13 @@ inline EncodeTiledFn tensor_map_encoder() {
   return fn;
 }
 
-// Opt a kernel in to `bytes` of dynamic shared memory.  The attribute belongs to the (function,
-// device) pair, so it is set on every launch path rather than remembered per process: the call
-// is a few hundred nanoseconds of host time.
-template <typename Kernel>
-inline cudaError_t allow_dynamic_smem(Kernel kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+// Opt a kernel in to BYTES of dynamic shared memory, the most that any of its launches takes.  The attribute
+// belongs to the (function, device) pair, so it is set on every launch path rather than remembered per process:
+// the call is a few hundred nanoseconds of host time.  It is the same number every time, hence a template argument:
+// another thread that launches the same kernel with less must not lower the limit between this call and its launch.
+template <int BYTES, typename Kernel>
+inline cudaError_t allow_dynamic_smem(Kernel kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES);
 }
 
 // Launch a kernel that may be scheduled while the preceding kernel of the stream is still

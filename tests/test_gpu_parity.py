@@ -1468,6 +1468,50 @@ def test_few_tiles_kernels_follow_each_other_and_other_layers_on_one_workspace()
         assert torch.equal(o.view(torch.int16), outs[0].view(torch.int16))
 
 
+@pytest.mark.parametrize("a,b", [
+    # pairs of layers that launch one and the same kernel with different amounts of shared memory: product and output of few tiles
+    # (padded to an SM of its own or not), of many (four exchange buffers or two), the separate product (lean or full ring)
+    ((4, (8, 56, 56, 64, 64)), (4, (8, 28, 28, 64, 64))),
+    ((2, (32, 56, 56, 128, 128)), (2, (32, 56, 56, 256, 128))),
+    ((2, (2, 56, 56, 512, 64)), (4, (2, 56, 56, 512, 64)))])
+def test_host_threads_launch_one_kernel_with_different_shared_memory(a, b):
+    # the limit on a kernel's shared memory belongs to the kernel, not to the call: with a limit set to what each call needs,
+    # one thread's call failed now and then because another's had lowered it in between
+    import threading
+    failed = []
+
+    def layer(m, shape, seed):
+        N, H, W, C, K = shape
+        plan = nv.Plan(m, point_set("std", m))
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.randn(N, H, W, C, generator=gen, device="cuda").half()
+        U = plan.filter_transform((torch.randn(K, 3, 3, C, generator=gen, device="cuda") * (2.0 / (9 * C)) ** 0.5).half())
+        want = plan.conv2d(x, U)
+        ws = torch.empty(plan.workspace_bytes(*shape), dtype=torch.uint8, device="cuda")
+        return plan, x, U, torch.empty_like(want), ws, want
+
+    def work(plan, x, U, y, ws, want):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(400):
+                    plan.conv2d(x, U, y, ws)
+            stream.synchronize()
+            if not torch.equal(y.view(torch.int16), want.view(torch.int16)):
+                failed.append("bits")
+        except Exception as e:
+            failed.append(repr(e))
+
+    layers = [layer(*a, 61), layer(*b, 62)]
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=l) for l in layers]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed and all(l[0].device_status() == 0 for l in layers)
+
+
 def test_int8_launch_count_follows_the_path():
     large, small = (2, 104, 106, 112, 528), (1, 20, 20, 112, 48)
     plan = nv.Plan(4, point_set("dyadic", 4))
