@@ -228,6 +228,8 @@ size_t nova_conv2d_min_workspace_bytes(const nova_plan* plan, int N, int H, int 
  * one kernel (same bits), which needs V alone; small F(2,3) layers the input transform too.  These paths are taken
  * only with nova_conv2d_workspace_bytes() or more, a smaller workspace
  * (nova_conv2d_fwd_static's for a large problem) gets the chunked three kernels.
+ * y_dev may lie over x_dev or U_dev where the tiles are one chunk (workspace_bytes of nova_conv2d_workspace_bytes() and V and M
+ * of at most 1 GiB): no kernel that reads such a tensor after another CTA may have stored there is used then.
  */
 int nova_conv2d_fwd(const nova_plan* plan, const void* x_dev, const void* U_dev, void* y_dev,
                     int N, int H, int W, int C, int K,

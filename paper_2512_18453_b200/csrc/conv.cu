@@ -137,6 +137,39 @@ bool use_tcgen05(const nova_plan* p, int flags) {
   return (flags & NOVA_GEMM_SIMT) == 0;
 }
 
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t p = reinterpret_cast<uintptr_t>(a), q = reinterpret_cast<uintptr_t>(b);
+  return p < q + nb && q < p + na;
+}
+// Tensors that y lies over.  A kernel that still reads one of them while other CTAs store y is no path for such a call.
+struct Under { bool x, U; };
+Under under_y(const nova_plan* p, const Geom& g, const void* x, const void* U, const void* y, int flags) {
+  const size_t e = elt_bytes(p->mode), pix = (size_t)g.N * g.H * g.W;
+  const size_t ny = (flags & NOVA_POOL2X2 ? pix / 4 : pix) * g.K * e;
+  return {overlap(y, ny, x, pix * g.C * e), overlap(y, ny, U, (size_t)g.n * g.n * g.K * g.C * e)};
+}
+
+// What a call launches: `kernels` per chunk of tiles.
+struct Route {
+  int kernels;
+  bool two;            // product_output.cu after the input transform
+  int few;             // variant of few_tiles.cu (above 10: the input transform in it), or 0
+  Chunking c;
+};
+bool choose_route(const nova_plan* p, const Geom& g, size_t ws_bytes, int flags, Under under, Route* r) {
+  if (!choose_chunking(p, g, ws_bytes, &r->c)) return false;
+  r->two = false;
+  r->few = 0;
+  r->kernels = 1;
+  if (!under.x && !under.U && one_kernel(p, g, flags)) return true;
+  r->two = !under.U && two_kernels(p, g, ws_bytes, flags, &r->c);
+  if (!r->two && !under.U) r->few = few_tiles(p, g, ws_bytes, flags);
+  if (r->few > 10 && under.x) r->few = 0;
+  if (r->few > 10) r->c.chunks = 1;
+  r->kernels = r->few > 10 ? 1 : r->two || r->few ? 2 : 3;
+  return true;
+}
+
 }  // namespace
 }  // namespace nova
 
@@ -180,12 +213,9 @@ extern "C" int nova_conv2d_launch_count(const nova_plan* p, int N, int H, int W,
   if (!p || !shape_ok(N, H, W, C, K)) return NOVA_ERR_INVALID_ARG;
   if (!device_plan(p)) return NOVA_ERR_UNSUPPORTED;
   Geom g = make_geom(p, N, H, W, C, K);
-  Chunking c;
-  if (!choose_chunking(p, g, workspace_bytes, &c)) return NOVA_ERR_WORKSPACE;
-  if (one_kernel(p, g, flags)) return 1;
-  if (two_kernels(p, g, workspace_bytes, flags, &c)) return 2 * c.chunks;
-  const int few = few_tiles(p, g, workspace_bytes, flags);
-  return few > 10 ? 1 : few > 0 ? 2 * c.chunks : 3 * c.chunks;
+  Route r;
+  if (!choose_route(p, g, workspace_bytes, flags, {false, false}, &r)) return NOVA_ERR_WORKSPACE;
+  return r.kernels == 1 ? 1 : r.kernels * r.c.chunks;
 }
 
 namespace {
@@ -206,9 +236,9 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
     if (p->mode != NOVA_FP16_F32ACC || !p->status_dev || (flags & NOVA_TRANSFORM_SIMT)) return NOVA_ERR_UNSUPPORTED;
   }
   Geom g = make_geom(p, N, H, W, C, K);
-  Chunking c;
-  if (!choose_chunking(p, g, ws_bytes, &c)) return NOVA_ERR_WORKSPACE;
-  if (one_kernel(p, g, flags)) {
+  Route route;
+  if (!choose_route(p, g, ws_bytes, flags, under_y(p, g, x, U, y, flags), &route)) return NOVA_ERR_WORKSPACE;
+  if (route.kernels == 1 && !route.few) {
     // steps 2-4 in one kernel, V and M kept on the SM: the workspace is not touched
     if (ev) cudaEventRecord(ev[0], (cudaStream_t)stream);
     const int relu = (flags & NOVA_RELU) ? 1 : 0;
@@ -222,7 +252,7 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
   }
   const bool tc = use_tcgen05(p, flags);
   if (tc && !p->status_dev) return NOVA_ERR_CUDA;
-  const int few = few_tiles(p, g, ws_bytes, flags);
+  const int few = route.few;
   if (few > 10) {
     if (ev) cudaEventRecord(ev[0], (cudaStream_t)stream);
     if (int e = launch_few_tiles_n4(p, g, x, U, y, store_flags(flags), few - 10, stream)) {
@@ -232,7 +262,8 @@ int conv2d_fwd_impl(const nova_plan* p, const void* x, const void* U, void* y, i
     if (ev) cudaEventRecord(ev[1], (cudaStream_t)stream);
     return NOVA_OK;
   }
-  const bool two = two_kernels(p, g, ws_bytes, flags, &c);
+  const bool two = route.two;
+  const Chunking& c = route.c;
   g.ldv = c.ldv;
   char* Vb = static_cast<char*>(ws);
   float* Mb = reinterpret_cast<float*>(Vb + c.v_bytes);
@@ -289,7 +320,10 @@ extern "C" int nova_conv2d_fwd_timed(const nova_plan* p, const void* x, const vo
   if (!kernel_ms) return NOVA_ERR_INVALID_ARG;
   const int launches = nova_conv2d_launch_count(p, N, H, W, C, K, ws_bytes, flags);
   if (launches < 0) return launches;
-  if (launches == 1) {               // the one-kernel path: its time is reported as the product's
+  const Geom g = make_geom(p, N, H, W, C, K);
+  Route route;
+  if (!choose_route(p, g, ws_bytes, flags, under_y(p, g, x, U, y, flags), &route)) return NOVA_ERR_WORKSPACE;
+  if (route.kernels == 1) {          // the one-kernel path: its time is reported as the product's
     cudaEvent_t e2[2];
     cudaEventCreate(&e2[0]);
     cudaEventCreate(&e2[1]);
@@ -301,9 +335,7 @@ extern "C" int nova_conv2d_fwd_timed(const nova_plan* p, const void* x, const vo
     cudaEventDestroy(e2[1]);
     return st1;
   }
-  Chunking two;                      // two kernels per chunk: the second one's time is reported as the product's
-  const Geom g = make_geom(p, N, H, W, C, K);
-  const int chunks = two_kernels(p, g, ws_bytes, flags, &two) ? two.chunks : launches / (few_tiles(p, g, ws_bytes, flags) ? 2 : 3);
+  const int chunks = route.c.chunks;  // two kernels per chunk: the second one's time is reported as the product's
   cudaEvent_t* ev = new cudaEvent_t[4 * chunks];
   for (int i = 0; i < 4 * chunks; ++i) cudaEventCreate(&ev[i]);
   int st = conv2d_fwd_impl(p, x, U, y, N, H, W, C, K, ws, ws_bytes, flags, stream, ev);

@@ -1512,6 +1512,43 @@ def test_host_threads_launch_one_kernel_with_different_shared_memory(a, b):
     assert not failed and all(l[0].device_status() == 0 for l in layers)
 
 
+@pytest.mark.parametrize("m,mode,shape,flag", [
+    # a flag names the three kernels where the one-kernel path sums in another order
+    (2, nv.FP16_F32ACC, (2, 20, 22, 64, 64), 0), (2, nv.FP16_F32ACC, (3, 50, 90, 64, 16), 0), (4, nv.FP16_F32ACC, (2, 30, 26, 64, 64), 0),
+    (2, nv.FP16_F32ACC, (32, 56, 56, 64, 64), 0), (6, nv.FP16_F32ACC, (2, 30, 26, 128, 128), 0), (6, nv.FP16_F32ACC, (2, 40, 44, 8, 8), nv.GEMM_TCGEN05),
+    (4, nv.FP32, (2, 40, 44, 16, 16), nv.GEMM_SIMT), (6, nv.FP32, (2, 40, 44, 24, 16), nv.GEMM_SIMT)])
+def test_output_over_the_input_or_the_filter(m, mode, shape, flag):
+    # a kernel that reads x (or U) and writes y in one pass is not used where y lies over it
+    N, H, W, C, K = shape
+    plan = nv.Plan(m, point_set("std", m), mode)
+    gen = torch.Generator(device="cuda").manual_seed(71)
+    dtype = torch.float32 if mode == nv.FP32 else torch.float16
+    x = torch.randn(N, H, W, C, generator=gen, device="cuda").to(dtype)
+    U = plan.filter_transform((torch.randn(K, 3, 3, C, generator=gen, device="cuda") * (2.0 / (9 * C)) ** 0.5).to(dtype))
+    ws = torch.empty(plan.workspace_bytes(*shape), dtype=torch.uint8, device="cuda")
+    bits = torch.int32 if mode == nv.FP32 else torch.int16
+    for flags in (nv.RELU, nv.RELU | nv.POOL2X2) if mode != nv.FP32 else (nv.RELU,):
+        pool = 2 if flags & nv.POOL2X2 else 1
+        want = plan.conv2d(x, U, flags=flags | flag)
+        for offset in (0, (x.numel() - want.numel()) // 16 * 16):               # the start of x and its end
+            for timed in (False, True):
+                buf = x.clone()
+                y = buf.view(-1)[offset:offset + want.numel()].view(N, H // pool, W // pool, K)
+                if timed:
+                    ms = plan.conv2d_timed(buf, U, y, ws, flags)
+                    assert min(ms[:2]) > 0
+                else:
+                    plan.conv2d(buf, U, y, ws, flags)
+                torch.cuda.synchronize()
+                assert plan.device_status() == 0 and torch.equal(y.view(bits), want.view(bits))
+        if want.numel() <= U.numel():
+            V = U.clone()
+            y = V.view(-1)[:want.numel()].view(want.shape)
+            plan.conv2d(x, V, y, ws, flags)
+            torch.cuda.synchronize()
+            assert plan.device_status() == 0 and torch.equal(y.view(bits), want.view(bits))
+
+
 def test_int8_launch_count_follows_the_path():
     large, small = (2, 104, 106, 112, 528), (1, 20, 20, 112, 48)
     plan = nv.Plan(4, point_set("dyadic", 4))
