@@ -439,6 +439,13 @@ int go_nb(int nb, const nova_plan* plan, const Geom& g, const void* V, const voi
 // at most 4000 tiles and 8 .. 512 channels: n = 4 1.51x (52 layers, none slower), n = 6 1.18x (101, three slower by 1 .. 7 %),
 // n = 8 1.17x (62, none slower).  Some of them (us):
 //   n = 4, input transform included   100 tiles 32 -> 8 9.0 / 4.0, 684 tiles 64 -> 32 8.7 / 4.8, 2040 tiles 48 -> 64 11.5 / 7.2
+//     up to 12 MB of M, which is product_output.cu's line (and none beyond it, should that kernel not be there): 5016 tiles 64 -> 32
+//     15.1 / 10.1, 16 tiles 64 -> 8192 13.2 / 7.3, 182 tiles 64 -> 768 11.0 / 6.9
+//     up to 16 filters in blocks of 16 however many tiles, three kernels / blocks of 32 / blocks of 16: 2808 tiles 24 -> 8 10.7 / 7.2 / 5.6,
+//     7050 tiles 64 -> 16 17.3 / 10.4 / 8.8, 16896 tiles 56 -> 8 32.4 / 26.4 / 21.6
+//     not where ragged rows of x are transformed densely for each of many blocks, more of them than two per SM: 361 tiles 56 -> 512
+//     11.7 / 13.0, 960 tiles 40 -> 192 12.1 / 12.6, 648 tiles 24 -> 256 11.9 / 12.2; the same with symmetric points 11.6 / 11.4, 11.8 / 11.3,
+//     11.7 / 10.8; 1406 tiles 56 -> 128 14.2 / 13.0; 160 tiles 24 -> 1024 12.3 / 11.7
 //   n = 4, more channels              180 tiles 192 -> 32 9.0 / 6.5, 252 tiles 256 -> 16 8.9 / 7.1, 870 tiles 256 -> 72 12.7 / 12.7 (not taken)
 //   n = 6, ks = 1                     36 tiles 64 -> 16 9.1 / 6.6, 1568 tiles 64 -> 64 14.1 / 12.2, 480 tiles 16 -> 512 19.1 / 21.3 (not taken)
 //   n = 6, ks = 2                     60 tiles 128 -> 32 9.4 / 6.8, 513 tiles 128 -> 64 11.8 / 9.3, 828 tiles 104 -> 128 15.4 / 20.8 (not taken)
@@ -448,9 +455,14 @@ int few_tiles_blocks(const nova_plan* plan, const Geom& g) {
   if (plan->mode != NOVA_FP16_F32ACC || plan->n > 8 || !plan->status_dev || plan->sm_count < 64 || g.P > (1 << 20)) return 0;
   const long long sms = plan->sm_count, tb = (g.P + kT - 1) / kT;
   const int ks = (g.C + 63) / 64;
+  const bool ragged = g.C % 16 != 0;                     // rows of channels that are not whole sectors of 32 bytes
   const long long c8 = tb * ((g.K + 7) / 8), c16 = tb * ((g.K + 15) / 16), c32 = tb * ((g.K + 31) / 32);
   if (plan->n == 4) {
-    if (ks == 1) return c16 <= sms ? 11 : 12;
+    if (ks == 1) {
+      if (64e-6 * (double)g.P * g.K >= 12) return 0;
+      if (g.K <= 16 || c16 <= sms) return 11;
+      return ragged && !plan->symmetric && c32 > 2 * sms && g.K > 128 && g.K < 1024 ? 0 : 12;
+    }
     if (ks == 2) return c16 <= sms / 2 ? 11 : c32 <= sms ? 4 : 0;
     if (ks <= 4) return c16 <= sms ? 2 : c32 <= sms / 2 ? 4 : 0;
     return ks <= 6 && c8 <= sms / 2 ? 1 : 0;

@@ -1447,6 +1447,19 @@ def test_few_tiles_kernels_give_the_bits_of_three(m, key, r, shape, launches):
     assert conv.rel_l2(y, y1) < (0.1 if m + r - 1 == 8 else 0.02)
 
 
+@pytest.mark.parametrize("m,key,shape,launches", [
+    # F(2,3), input transform included: up to 12 MB of M, whatever the number of filters (16 tiles 64 -> 8192: 16 tiles, 256 blocks) ...
+    (2, ("std", 2), (1, 306, 306, 16, 8), 1), (2, ("std", 2), (1, 308, 308, 16, 8), 2), (2, ("asym", 2), (1, 8, 8, 64, 8192), 1),
+    # ... but not where x is transformed densely for many blocks that do not all run at once, from rows that are not whole sectors
+    (2, ("asym", 2), (1, 38, 38, 56, 512), 3), (2, ("asym", 2), (1, 62, 62, 40, 192), 3), (2, ("asym", 2), (1, 52, 50, 24, 256), 3),
+    (2, ("std", 2), (1, 38, 38, 56, 512), 1), (2, ("asym", 2), (1, 38, 38, 48, 512), 1), (2, ("asym", 2), (1, 72, 74, 56, 128), 1),
+])
+def test_few_tiles_kernels_run_where_they_are_the_faster_ones(m, key, shape, launches):
+    # the line of the dispatch, by the launches on either side of it; the figures stand at the rule
+    plan = nv.Plan(m, point_set(*key))
+    assert plan.launch_count(*shape, plan.workspace_bytes(*shape), nv.RELU) == launches
+
+
 def test_few_tiles_kernels_follow_each_other_and_other_layers_on_one_workspace():
     # calls in a row without a wait between them, each fed by the one before, the filters made just before: the kernels start
     # before their predecessor has ended
