@@ -448,6 +448,14 @@ int go_nb(int nb, const nova_plan* plan, const Geom& g, const void* V, const voi
 //     11.7 / 10.8; 1406 tiles 56 -> 128 14.2 / 13.0; 160 tiles 24 -> 1024 12.3 / 11.7
 //   n = 4, more channels              180 tiles 192 -> 32 9.0 / 6.5, 252 tiles 256 -> 16 8.9 / 7.1, 870 tiles 256 -> 72 12.7 / 12.7 (not taken)
 //   n = 6, ks = 1                     36 tiles 64 -> 16 9.1 / 6.6, 1568 tiles 64 -> 64 14.1 / 12.2, 480 tiles 16 -> 512 19.1 / 21.3 (not taken)
+//     between one and two blocks of 32 filters per SM, three kernels / blocks of 16 / blocks of 32: 3600 tiles 16 -> 16 18.2 / 11.1 / 15.0, 1404 tiles
+//     32 -> 48 13.7 / 9.9 / 13.8, 1444 tiles 48 -> 64 14.4 / 13.1 / 14.4, 2312 tiles 16 -> 64 16.8 / 14.9 / 14.7, 528 tiles 32 -> 256 14.6 / 13.2 / 12.8,
+//     2256 tiles 64 -> 64 16.4 / 14.3 / 14.2; ragged rows: 1250 tiles 40 -> 64 14.1 / 13.4 / 14.5, 2312 tiles 40 -> 64 19.9 / 18.1 / 17.6,
+//     4416 tiles 56 -> 32 22.0 / 20.6 / 19.7, not taken 1764 tiles 24 -> 64 16.1 / 16.6 / 16.9, 363 tiles 24 -> 256 13.0 / 13.9 / 13.4, 1458 tiles
+//     56 -> 64 14.3 / 16.3 / 15.5
+//   n = 6, ks = 3                     200 tiles 176 -> 88 10.5 / 9.2, 1012 tiles 192 -> 16 13.6 / 11.1, 256 tiles 160 -> 64 9.8 / 9.3; ragged rows:
+//     16 tiles 152 -> 256 9.0 / 8.2, 196 tiles 136 -> 16 9.9 / 9.5, 512 tiles 152 -> 16 11.4 / 10.9, 256 tiles 184 -> 32 9.8 / 10.1 (not taken), 98 tiles 184 -> 96 9.4 / 9.8 (not
+//     taken): the three kernels pay for a third block of 128 tiles from 257 tiles on
 //   n = 6, ks = 2                     60 tiles 128 -> 32 9.4 / 6.8, 513 tiles 128 -> 64 11.8 / 9.3, 828 tiles 104 -> 128 15.4 / 20.8 (not taken)
 //   n = 8                             72 tiles 64 -> 24 9.1 / 6.5, 950 tiles 32 -> 32 14.8 / 10.6, 360 tiles 136 -> 32 14.5 / 15.4 (not taken)
 // With 10 points a CTA's steps are too many (16 tiles 56 -> 80 10.6 / 10.8).
@@ -469,9 +477,15 @@ int few_tiles_blocks(const nova_plan* plan, const Geom& g) {
   }
   if (plan->n == 6) {
     if (ks <= 2 && c8 <= sms / 2) return 1;
-    if (ks == 1) return c16 <= sms ? 2 : c32 <= sms ? 4 : c32 <= 2 * sms ? (g.C > 48 ? 2 : 4) : 0;
-    if (ks == 2) return c16 <= sms ? 2 : c32 <= sms ? 4 : 0;
-    if (ks == 3) return c8 <= sms / 2 ? 1 : c16 <= sms / 2 ? 2 : 0;
+    if (ks <= 2 && (c16 <= sms || c32 <= sms)) return c16 <= sms ? 2 : 4;
+    if (ks == 1 && c32 <= 2 * sms) {
+      // two CTAs of 16 filters on an SM against one of 32
+      const bool halves = c16 <= sms * 8 / 3;
+      if (c16 <= 2 * sms) return 2;
+      if (ragged && g.K > 40) return g.C > 40 ? 0 : halves && g.K <= 128 ? 2 : c32 > sms * 5 / 3 ? 4 : 0;
+      return halves || g.C == 64 ? 2 : 4;
+    }
+    if (ks == 3) return c8 <= (!ragged || tb > 16 ? sms : tb <= 5 || g.C < 144 ? sms / 2 : 16) ? 1 : 0;
     return 0;
   }
   if (ks > 2) return 0;

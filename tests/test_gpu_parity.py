@@ -1453,6 +1453,15 @@ def test_few_tiles_kernels_give_the_bits_of_three(m, key, r, shape, launches):
     # ... but not where x is transformed densely for many blocks that do not all run at once, from rows that are not whole sectors
     (2, ("asym", 2), (1, 38, 38, 56, 512), 3), (2, ("asym", 2), (1, 62, 62, 40, 192), 3), (2, ("asym", 2), (1, 52, 50, 24, 256), 3),
     (2, ("std", 2), (1, 38, 38, 56, 512), 1), (2, ("asym", 2), (1, 38, 38, 48, 512), 1), (2, ("asym", 2), (1, 72, 74, 56, 128), 1),
+    # 6 points, one piece of 64 channels, between one and two blocks of 32 filters per SM: rows of 56 channels, or of 24 and 40 in
+    # the middle of that range, of more than 40 filters
+    (4, ("nova", 4), (1, 152, 152, 56, 64), 3), (4, ("nova", 4), (1, 84, 80, 56, 256), 3), (4, ("asym", 4), (1, 168, 168, 24, 64), 3),
+    (4, ("nova", 4), (3, 43, 43, 24, 256), 3), (4, ("nova", 4), (1, 152, 152, 64, 64), 2), (4, ("asym", 4), (1, 152, 152, 24, 64), 2), (4, ("nova", 4), (1, 264, 264, 56, 32), 2),
+    (4, ("nova", 4), (2, 136, 136, 40, 64), 2), (4, ("asym", 4), (1, 148, 148, 56, 48), 2),
+    # three pieces: rows that are not whole sectors, of more than 80 and up to 256 tiles
+    (4, ("asym", 4), (1, 64, 64, 184, 32), 3), (4, ("std", 4), (2, 28, 28, 152, 128), 3),
+    (4, ("asym", 4), (1, 68, 64, 184, 32), 2), (4, ("asym", 4), (1, 64, 64, 176, 32), 2), (4, ("std", 4), (1, 16, 16, 152, 256), 2),
+    (4, ("std", 4), (2, 40, 40, 176, 88), 2),
 ])
 def test_few_tiles_kernels_run_where_they_are_the_faster_ones(m, key, shape, launches):
     # the line of the dispatch, by the launches on either side of it; the figures stand at the rule
