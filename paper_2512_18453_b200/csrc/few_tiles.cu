@@ -458,6 +458,10 @@ int go_nb(int nb, const nova_plan* plan, const Geom& g, const void* V, const voi
 //     taken): the three kernels pay for a third block of 128 tiles from 257 tiles on
 //   n = 6, ks = 2                     60 tiles 128 -> 32 9.4 / 6.8, 513 tiles 128 -> 64 11.8 / 9.3, 828 tiles 104 -> 128 15.4 / 20.8 (not taken)
 //   n = 8                             72 tiles 64 -> 24 9.1 / 6.5, 950 tiles 32 -> 32 14.8 / 10.6, 360 tiles 136 -> 32 14.5 / 15.4 (not taken)
+//     two pieces of channels: 40 tiles 128 -> 256 10.1 / 8.4, 98 tiles 96 -> 32 9.0 / 8.7, 952 tiles 112 -> 24 17.0 / 14.5; ragged rows from 257 tiles on,
+//     where the three kernels pay for a third block of 128, with many filters and up to 8 tiles: 288 tiles 120 -> 32 11.8 / 11.7, 676 tiles 104 -> 24
+//     15.0 / 13.3, 98 tiles 104 -> 160 11.9 / 10.9, 25 tiles 88 -> 400 11.3 / 10.0, 4 tiles 104 -> 40 9.8 / 8.4; not taken 42 tiles 120 -> 48
+//     9.1 / 10.2, 100 tiles 88 -> 32 9.0 / 9.5, 256 tiles 104 -> 64 10.8 / 11.2
 // With 10 points a CTA's steps are too many (16 tiles 56 -> 80 10.6 / 10.8).
 int few_tiles_blocks(const nova_plan* plan, const Geom& g) {
   if (plan->mode != NOVA_FP16_F32ACC || plan->n > 8 || !plan->status_dev || plan->sm_count < 64 || g.P > (1 << 20)) return 0;
@@ -488,7 +492,7 @@ int few_tiles_blocks(const nova_plan* plan, const Geom& g) {
     if (ks == 3) return c8 <= (!ragged || tb > 16 ? sms : tb <= 5 || g.C < 144 ? sms / 2 : 16) ? 1 : 0;
     return 0;
   }
-  if (ks > 2) return 0;
+  if (ks > 2 || (ks == 2 && ragged && tb <= 16 && g.P > 8 && (g.K < 160 || c8 < 64))) return 0;
   return c8 <= sms ? 1 : c16 <= sms ? 2 : ks == 1 && c32 <= sms ? 4 : 0;
 }
 

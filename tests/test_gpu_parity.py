@@ -1462,6 +1462,10 @@ def test_few_tiles_kernels_give_the_bits_of_three(m, key, r, shape, launches):
     (4, ("asym", 4), (1, 64, 64, 184, 32), 3), (4, ("std", 4), (2, 28, 28, 152, 128), 3),
     (4, ("asym", 4), (1, 68, 64, 184, 32), 2), (4, ("asym", 4), (1, 64, 64, 176, 32), 2), (4, ("std", 4), (1, 16, 16, 152, 256), 2),
     (4, ("std", 4), (2, 40, 40, 176, 88), 2),
+    # 8 points, two pieces: such rows of up to 256 tiles
+    (6, ("half", 6), (1, 96, 96, 104, 64), 3), (6, ("asym", 6), (2, 28, 29, 120, 48), 3), (6, ("nova", 6), (1, 24, 24, 72, 128), 3),
+    (6, ("half", 6), (1, 102, 96, 104, 48), 2), (6, ("asym", 6), (2, 28, 29, 112, 48), 2), (6, ("nova", 6), (1, 24, 24, 56, 128), 2),
+    (6, ("half", 6), (1, 30, 30, 104, 400), 2), (6, ("half", 6), (1, 12, 24, 104, 40), 2), (6, ("half", 6), (1, 18, 18, 104, 40), 3),
 ])
 def test_few_tiles_kernels_run_where_they_are_the_faster_ones(m, key, shape, launches):
     # the line of the dispatch, by the launches on either side of it; the figures stand at the rule
