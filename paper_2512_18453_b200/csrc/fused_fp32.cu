@@ -41,7 +41,8 @@ constexpr int kChunk = 16;               // channels per chunk
 constexpr int kRowBytes = 4 * kChunk;
 constexpr int kRecRing = 8;              // tile records: the producer is at most five blocks ahead of the stores
 
-template <int M, int R>
+// ROWS: the end of a block that exchanges one output row at a time (see kZRows), whatever the tile
+template <int M, int R, bool ROWS>
 struct Fc32 {
   static constexpr int N = M + R - 1, PAD = (R - 1) / 2, NF = N * N;
   static constexpr int NH = (N == 8) ? 1 : 2;                      // warps that share a column nu
@@ -63,7 +64,10 @@ struct Fc32 {
   // Output rows that meet in shared memory at a time.  Row by row, in two buffers in turn, most product warps wait at a barrier
   // per row: a block's end took as long as one of its chunks.  Whole call, row by row / this: F(4,3) 8 x 56 x 56, 64 -> 64 34.6 / 33.9 us,
   // 3 x 46 x 46, 32 -> 32 9.9 / 9.1; F(6,3) 61 x 107, 32 -> 256 28.3 / 26.9.  Two output rows stay with it: 8 x 56 x 56, 64 -> 64, F(2,3) 55.8 / 58.7.
-  static constexpr int kZRows = (M == 2) ? 1 : (N == 8) ? 2 : M;
+  // A kernel compiled with this end is the slower one where a cluster splits the channels, although that path's source is the same: six
+  // points, 1 x 40 x 40, 112 -> 8 9.11 / 9.37, 9 x 24 x 15, 224 -> 8 12.57 / 12.85, 2 x 101 x 32, 224 -> 16 17.9 / 18.3; such calls keep a
+  // kernel with the row-by-row end (eight points gain either way: 2 x 7 x 30, 48 -> 8, asymmetric 24.5 / 21.1).
+  static constexpr int kZRows = (M == 2 || ROWS) ? 1 : (N == 8) ? 2 : M;
   static_assert(M % kZRows == 0, "");
   static constexpr int kOffX = 0;
   static constexpr int kOffV = kOffX + kXBytes;
@@ -175,12 +179,12 @@ __device__ __forceinline__ void put_row(int i, const Dbl2 (&v)[M], float* yt, co
     }
 }
 
-template <int M, int R, bool SYM>
-__global__ void __launch_bounds__(Fc32<M, R>::kThreads, 1)
+template <int M, int R, bool SYM, bool ROWS>
+__global__ void __launch_bounds__(Fc32<M, R, ROWS>::kThreads, 1)
 fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUtensorMap tmX,
                   const __grid_constant__ CUtensorMap tmU, float* __restrict__ y, const __grid_constant__ FcArgs args,
                   int* __restrict__ status) {
-  using Cfg = Fc32<M, R>;
+  using Cfg = Fc32<M, R, ROWS>;
   constexpr int N = Cfg::N, NB = Cfg::NB, ST = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
@@ -451,25 +455,31 @@ fused_fp32_kernel(const __grid_constant__ CoefsD cf, const __grid_constant__ CUt
   }
 }
 
+// Tiles whose split blocks have a kernel of their own (see kZRows).
+template <int M, int R>
+constexpr bool split_by_rows() { return M + R - 1 == 6 && M > 2; }
+
 // setmaxnreg draws on the registers the block was launched with: a build whose register count is not what the split was
 // computed for does without this kernel.
-template <int M, int R, bool SYM>
+template <int M, int R, bool SYM, bool ROWS = false>
 bool built() {
   static const int regs = [] {
     cudaFuncAttributes at;
-    return cudaFuncGetAttributes(&at, fused_fp32_kernel<M, R, SYM>) == cudaSuccess ? at.numRegs : 0;
+    return cudaFuncGetAttributes(&at, fused_fp32_kernel<M, R, SYM, ROWS>) == cudaSuccess ? at.numRegs : 0;
   }();
-  return regs >= Fc32<M, R>::kLaunchRegs;
+  if constexpr (split_by_rows<M, R>() && !ROWS)
+    if (!built<M, R, SYM, true>()) return false;
+  return regs >= Fc32<M, R, ROWS>::kLaunchRegs;
 }
 
-template <int M, int R, bool SYM>
+template <int M, int R, bool SYM, bool ROWS>
 int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void* y, int relu, int nb, int split,
        cudaStream_t stream) {
-  using Cfg = Fc32<M, R>;
+  using Cfg = Fc32<M, R, ROWS>;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return (int)cudaErrorUnknown;
-  auto kernel = fused_fp32_kernel<M, R, SYM>;
-  if (!built<M, R, SYM>()) return (int)cudaErrorInvalidConfiguration;
+  auto kernel = fused_fp32_kernel<M, R, SYM, ROWS>;
+  if (!built<M, R, SYM, ROWS>()) return (int)cudaErrorInvalidConfiguration;
   const int f_run = 8 * nb * Cfg::NH;
   CUtensorMap tmX, tmU;
   cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -565,8 +575,15 @@ int launch_fused_fp32(const nova_plan* plan, const Geom& g, const void* x, const
   cudaStream_t s = (cudaStream_t)stream;
   int nb = 1, split = 1;
   choose_blocks(plan->n, g, plan->sm_count, &nb, &split);
-#define NOVA_FC32(MV, RV)                                                                      \
-  return plan->symmetric ? go<MV, RV, true>(plan, g, x, U, y, relu, nb, split, s) : go<MV, RV, false>(plan, g, x, U, y, relu, nb, split, s)
+#define NOVA_FC32(MV, RV)                                                                                            \
+  do {                                                                                                                 \
+    if constexpr (split_by_rows<MV, RV>())                                                                             \
+      if (split > 1)                                                                                                   \
+        return plan->symmetric ? go<MV, RV, true, true>(plan, g, x, U, y, relu, nb, split, s)                          \
+                               : go<MV, RV, false, true>(plan, g, x, U, y, relu, nb, split, s);                        \
+    return plan->symmetric ? go<MV, RV, true, false>(plan, g, x, U, y, relu, nb, split, s)                             \
+                           : go<MV, RV, false, false>(plan, g, x, U, y, relu, nb, split, s);                           \
+  } while (0)
   if (plan->r == 3) {
     if (plan->m == 2) NOVA_FC32(2, 3);
     if (plan->m == 4) NOVA_FC32(4, 3);
