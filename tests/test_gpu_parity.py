@@ -116,7 +116,11 @@ def test_fp32_mode_matches_direct(kind, m, shape):
     (2, ("std", 2), 3, (1, 5, 7, 8, 520)),       # one block of tiles, ragged last filter block
     (4, ("nova", 4), 3, (1, 14, 14, 256, 24)),   # few blocks, many channels: the channels of a block split over a cluster
     (4, ("asym", 4), 3, (3, 33, 18, 40, 40)),    # 135 tiles, a chunk of 16 channels half outside the tensor
-    (6, ("half", 6), 3, (2, 50, 50, 64, 72)),    # several blocks per CTA
+    (6, ("half", 6), 3, (2, 50, 50, 64, 72)),    # split, blocks of 16 filters, the last one half there
+    (6, ("half", 6), 3, (1, 61, 107, 32, 256)),  # 200 blocks on the SMs, whole channels: two output rows meet at a time, several blocks per CTA
+    (6, ("asym", 6), 3, (1, 61, 107, 16, 264)),  # the same, dense, 225 blocks
+    (4, ("half", 6), 5, (2, 36, 36, 24, 520)),   # 357 blocks
+    (4, ("nova", 4), 3, (8, 36, 36, 16, 72)),    # six points: all four rows at once, 243 blocks
     (6, ("asym", 6), 3, (1, 12, 12, 136, 16)),   # dense transforms, split
     (4, ("half", 6), 5, (2, 23, 19, 24, 64)),
     (2, ("nova", 4), 5, (1, 40, 41, 16, 136))])
@@ -1447,6 +1451,47 @@ def test_few_tiles_kernels_give_the_bits_of_three(m, key, r, shape, launches):
     assert conv.rel_l2(y, y1) < (0.1 if m + r - 1 == 8 else 0.02)
 
 
+def _spread(kind, N, H, W, C, K, r, gen):
+    """Inputs and weights whose products differ by many powers of two, or cancel."""
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    power = lambda lo, hi, *s: torch.exp2(torch.randint(lo, hi + 1, s, generator=gen, device="cuda").float())
+    if kind == "elements":
+        return rand(N, H, W, C) * power(-12, 6, N, H, W, C), rand(K, r, r, C) * power(-12, 2, K, r, r, C) * 0.1
+    if kind == "channels":
+        return rand(N, H, W, C) * power(-12, 7, C), rand(K, r, r, C) * power(-12, 2, C) * 0.1
+    if kind == "subnormal":
+        return rand(N, H, W, C) * 2.0 ** -14, rand(K, r, r, C) * 2.0 ** -13
+    if kind == "neighbours":                                 # a channel and its neighbour cancel but for the last bits
+        x, w = rand(N, H, W, C) * 16, rand(K, r, r, C)
+        x[..., 1::2] = x[..., 0::2]
+        w[..., 1::2] = -w[..., 0::2] * (1 + (power(0, 1, K, r, r, C // 2) - 1) * 2.0 ** -9)
+        return x, w
+    x, w = rand(N, H, W, C) * 2.0 ** -8, rand(K, r, r, C) * 0.25       # large pairs cancel, the small rest is the result
+    x[..., 0::8] = 200 * rand(N, H, W, (C + 7) // 8)
+    x[..., 3::8] = x[..., 0::8]
+    w[..., 3::8] = -w[..., 0::8]
+    return x, w
+
+
+@pytest.mark.parametrize("kind", ["elements", "channels", "subnormal", "neighbours", "pairs"])
+@pytest.mark.parametrize("m,key,r,shape,launches", [
+    (2, ("std", 2), 3, (2, 20, 22, 64, 32), 1), (2, ("asym", 2), 3, (1, 16, 18, 24, 16), 1), (2, ("std", 2), 3, (1, 13, 11, 136, 24), 2),
+    (4, ("nova", 4), 3, (3, 30, 30, 56, 64), 2), (4, ("asym", 4), 3, (1, 13, 11, 104, 24), 2), (2, ("std", 4), 5, (2, 20, 22, 64, 32), 2),
+    (6, ("half", 6), 3, (2, 20, 22, 64, 32), 2), (4, ("nova", 6), 5, (1, 16, 18, 24, 16), 2)])
+def test_few_tiles_sums_are_the_product_kernels_whatever_the_exponents(m, key, r, shape, launches, kind):
+    # nothing documented says that mma.sync and tcgen05.mma add a group of 16 products alike; that the paths give the same bits
+    # (and a part of a batch those of the whole) rests on it
+    N, H, W, C, K = shape
+    x, w = _spread(kind, N, H, W, C, K, r, torch.Generator(device="cuda").manual_seed(5))
+    plan = nv.Plan(m, point_set(*key), r=r)
+    assert plan.launch_count(N, H, W, C, K, plan.workspace_bytes(N, H, W, C, K)) == launches
+    U = plan.filter_transform(w.half())
+    got, want = plan.conv2d(x.half(), U), plan.conv2d(x.half(), U, flags=nv.GEMM_TCGEN05)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0 and torch.isfinite(want.float()).all() and (want != 0).any()
+    assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+
+
 @pytest.mark.parametrize("m,key,shape,launches", [
     # F(2,3), input transform included: up to 12 MB of M, whatever the number of filters (16 tiles 64 -> 8192: 16 tiles, 256 blocks) ...
     (2, ("std", 2), (1, 306, 306, 16, 8), 1), (2, ("std", 2), (1, 308, 308, 16, 8), 2), (2, ("asym", 2), (1, 8, 8, 64, 8192), 1),
@@ -1477,7 +1522,9 @@ def test_few_tiles_kernels_follow_each_other_and_other_layers_on_one_workspace()
     # calls in a row without a wait between them, each fed by the one before, the filters made just before: the kernels start
     # before their predecessor has ended
     gen = torch.Generator(device="cuda").manual_seed(89)
-    chans, plans = (16, 64, 64, 40, 256, 24, 64), [nv.Plan(m, point_set("std", m)) for m in (2, 4, 2, 4, 4, 2)]
+    chans, plans = (16, 64, 64, 40, 256, 24, 64, 136, 24), [nv.Plan(m, point_set("std", m)) for m in (2, 4, 2, 4, 4, 2, 2, 2)]
+    # all three steps in one kernel, product and output after an input transform (4 and 6 points), three kernels
+    assert [p.launch_count(2, 20, 24, a, b, p.workspace_bytes(2, 20, 24, a, b)) for p, a, b in zip(plans, chans, chans[1:])] == [1, 2, 1, 2, 3, 1, 1, 2]
     ws = torch.empty(max(p.workspace_bytes(2, 20, 24, a, b) for p, a, b in zip(plans, chans, chans[1:])), dtype=torch.uint8, device="cuda")
     x = torch.randn(2, 20, 24, 16, generator=gen, device="cuda").half()
     g = [(torch.randn(b, 3, 3, a, generator=gen, device="cuda") * (2.0 / (9 * a)) ** 0.5).half() for a, b in zip(chans, chans[1:])]
