@@ -37,6 +37,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "nova_internal.h"
 #include "sm100.cuh"
 #include "tma_host.h"
@@ -242,9 +244,10 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     const size_t f_stride = (size_t)pc_pad * ldv;
     float qs = 1.f, amax = 0.f;
     // With the data's own scale no code passes 127, and adding 1.5 * 2^23 rounds a value to nearest even into the low bits: two
-    // instructions of the FMA pipe where the conversion, which this pass was bound by, takes the quarter-rate one (61 % busy).
-    // Whole call, conversion / addition: F(4,3) 32 x 56 x 56, 256 -> 256 120.0 / 119.0 us, 128 -> 64 48.8 / 48.2, 7 x 56 x 77, 64 -> 368 46.1 / 45.5.
-    // A caller's scale may send values out of range, a scale below 2^-128 has no reciprocal, and NaN becomes 0: those convert.
+    // instructions of the FMA pipe where the conversion, which this pass was bound by, takes the quarter-rate one (62 % busy, 14 % now).
+    // Whole call, conversion / addition: F(4,3) 32 x 56 x 56, 256 -> 256 119.8 / 116.1 us, 128 -> 64 48.7 / 46.7, 7 x 56 x 77, 64 -> 368 46.0 / 45.0.
+    // A caller's scale may send values out of range, a scale below 2^-128 has no reciprocal, and NaN becomes 0: those convert.  A whole
+    // warp takes one of the two loops: decided value by value, both were executed, the conversion still 63 % of its pipe.
     bool in_range = !(qgiven > 0.f);
     if constexpr (QMODE == 2) {
       qs = qgiven;
@@ -291,30 +294,36 @@ input_transform_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
           // group of four channels is inside or outside the tensor as a whole).
           const int li = lane & 3;
           int8_t* d4 = dst8 - li + (size_t)li * f_stride;
+          float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int cc = 0; cc < kMaxCols; cc += 4)
-            if (col0 + cc < Cfg::NF) {
-              uint32_t q[4];
-              float v[4];
+            if (col0 + cc < Cfg::NF)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) v[j] = __fmul_rn(__uint_as_float(r[cc + j]), qs);
-              const float any = (v[0] + v[1]) + (v[2] + v[3]);          // NaN where one of them is
-              if (in_range && any == any) {
+              for (int j = 0; j < 4; ++j) sum[j] += __uint_as_float(r[cc + j]);
+          const float any = (sum[0] + sum[1]) + (sum[2] + sum[3]);      // finite only where all of them are
+          auto quantise = [&](auto add) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) q[j] = __float_as_uint(__fadd_rn(v[j], 12582912.f));
-              } else {
+            for (int cc = 0; cc < kMaxCols; cc += 4)
+              if (col0 + cc < Cfg::NF) {
+                uint32_t q[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) asm("cvt.rni.sat.s8.f32 %0, %1;" : "=r"(q[j]) : "f"(v[j]));
+                for (int j = 0; j < 4; ++j) {
+                  const float v = __fmul_rn(__uint_as_float(r[cc + j]), qs);
+                  if constexpr (decltype(add)::value) q[j] = __float_as_uint(__fadd_rn(v, 12582912.f));
+                  else asm("cvt.rni.sat.s8.f32 %0, %1;" : "=r"(q[j]) : "f"(v));
+                }
+                // the low bytes of the four codes, packed with three byte permutations
+                const uint32_t w = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+                const uint32_t p1 = __shfl_xor_sync(0xffffffffu, w, 1);
+                const uint32_t t = __byte_perm(w, p1, (li & 1) ? 0x3715 : 0x6240);
+                const uint32_t p2 = __shfl_xor_sync(0xffffffffu, t, 2);
+                const uint32_t o = __byte_perm(t, p2, (li & 2) ? 0x3276 : 0x5410);
+                if (c < C) *reinterpret_cast<uint32_t*>(d4) = o;
+                d4 += 4 * f_stride;
               }
-              // the low bytes of the four codes, packed with three byte permutations
-              const uint32_t w = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
-              const uint32_t p1 = __shfl_xor_sync(0xffffffffu, w, 1);
-              const uint32_t t = __byte_perm(w, p1, (li & 1) ? 0x3715 : 0x6240);
-              const uint32_t p2 = __shfl_xor_sync(0xffffffffu, t, 2);
-              const uint32_t o = __byte_perm(t, p2, (li & 2) ? 0x3276 : 0x5410);
-              if (c < C) *reinterpret_cast<uint32_t*>(d4) = o;
-              d4 += 4 * f_stride;
-            }
+          };
+          if (__all_sync(0xffffffffu, in_range && any - any == 0.f)) quantise(std::true_type{});
+          else quantise(std::false_type{});
           dst8 += (size_t)((Cfg::NF - col0 < kMaxCols) ? (Cfg::NF - col0) : kMaxCols) * f_stride;
         } else if (c < C) {
 #pragma unroll
