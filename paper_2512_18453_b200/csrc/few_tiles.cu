@@ -4,12 +4,15 @@
 // A CTA owns 16 tiles x KB filters and ALL frequencies of them: warp (xi, h) the row xi of frequencies for its share of the
 // filters.  No CTA waits for another one, and M goes no further than registers and shared memory.
 //
-// What bounds it: the register-level tensor-core instruction (mma.sync m16n8k16: some 30 cycles of a scheduler each, 270
-// multiply-adds per clock and SM against 8192 of tcgen05), and U, which every block of 16 tiles fetches again.  So it is for
-// layers whose work per CTA is a few dozen of them; which ones, and figures: see few_tiles_blocks.
+// What bounds it: latency.  A warp's step (64 channels of one frequency: ldmatrix, 4 to 16 mma.sync, the copies of a later
+// step) is a chain that one or two warps per scheduler do not hide: F(4,3), 8 x 56 x 56, 64 -> 64, 12.0 us by itself with 45 % of the
+// issue slots and 12 % of the tensor pipe used; a contraction of nothing but such steps makes some 270 multiply-adds per clock
+// and SM, where tcgen05 makes 4096.  And U, which every block of 16 tiles fetches again.  So it is for layers whose work per
+// CTA is a few dozen of these steps; which ones, and figures: see few_tiles_blocks.
 //
-// V and U are contracted in the same groups of 16 channels as by tcgen05.mma, and the sums of both instructions agree bit
-// for bit; the transforms' arithmetic and its order are the three-kernel path's: the results are the same bits.
+// V and U are contracted in the same groups of 16 channels as by tcgen05.mma.  Nothing documented says that both instructions
+// add such a group alike; on every input tried they do, to the bit (unit normals, values spread over 18 powers of two,
+// subnormals, cancelling channels: the tests).  The transforms' arithmetic and its order are the three-kernel path's.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -285,6 +288,7 @@ struct N4Cfg : FtCfg<2, 3, 2, NB> {
   static_assert(Base::kZBytes <= kOffRec, "the rows of sums fit over the operands");
 };
 
+// 128 registers, so that two CTAs share an SM, cost the kernel of 32 filters a block 76 bytes of spills (120 with dense transforms).
 template <bool SYM, int NB>
 __global__ void __launch_bounds__(256, 2)
 few_tiles_n4_kernel(const __grid_constant__ Coefs cf, const __half* x, const __half* U, __half* y, const __grid_constant__ FtArgs a) {
@@ -396,7 +400,8 @@ FtArgs make_args(const Geom& g, long long p0, int pc, int pc_pad, int relu, int 
 
 constexpr int kOwnSm = 120 * 1024;
 // Shared memory that keeps two CTAs off one SM while another SM has none.  Without it CTAs that become resident while the
-// input transform still runs share SMs: F(4,3), 2 x 26 x 20, 344 -> 104, 65 CTAs 27.7 / 13.4 us; 4 x 97 x 37, 184 -> 16 21.1 / 12.9.
+// input transform still runs share SMs: F(4,3), 4 x 97 x 37, 184 -> 16 21.1 / 12.9 us, 8 x 30 x 26, 176 -> 16 15.7 / 10.0, 8 x 28 x 28, 64 -> 64
+// 7.7 / 7.0; F(6,3) 2 x 30 x 30, 64 -> 64 and F(2,3) 2 x 24 x 24, 128 -> 136 6.7 and 6.8 either way.
 int own_sm(int bytes, int grid, int sms) { return bytes < kOwnSm && grid <= sms ? kOwnSm : bytes; }
 
 template <int M, int R, bool SYM, int NB>
@@ -435,9 +440,9 @@ int go_nb(int nb, const nova_plan* plan, const Geom& g, const void* V, const voi
 
 // The block of filters, in eights (1, 2 or 4), where these kernels are the faster ones; plus 10 where the input transform is in
 // them; 0 elsewhere.  The line lies at the number of CTAs and ks = 64-channel pieces, which are steps of each warp.
-// Whole call, kernels without a merged product / this rule, geometric mean over layers of 1 .. 32 images of 7 .. 112 pixels with
-// at most 4000 tiles and 8 .. 512 channels: n = 4 1.51x (52 layers, none slower), n = 6 1.18x (101, three slower by 1 .. 7 %),
-// n = 8 1.17x (62, none slower).  Some of them (us):
+// Whole call, kernels without a merged product / this rule, geometric mean over the layers that the rule takes of 220 random ones
+// each, 1 .. 32 images of 7 .. 112 pixels with 16 .. 512 channels: n = 4 1.56x (147 layers, none slower), n = 6 1.32x (155, none
+// slower), n = 8 1.28x (128, two slower: 100 tiles 80 -> 64 10.0 / 10.2, 50 tiles 120 -> 256 9.9 / 10.4).  Some of them (us):
 //   n = 4, input transform included   100 tiles 32 -> 8 9.0 / 4.0, 684 tiles 64 -> 32 8.7 / 4.8, 2040 tiles 48 -> 64 11.5 / 7.2
 //     up to 12 MB of M, which is product_output.cu's line (and none beyond it, should that kernel not be there): 5016 tiles 64 -> 32
 //     15.1 / 10.1, 16 tiles 64 -> 8192 13.2 / 7.3, 182 tiles 64 -> 768 11.0 / 6.9

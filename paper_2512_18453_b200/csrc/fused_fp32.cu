@@ -13,8 +13,8 @@
 //                    8 tiles x 8 * nb filters x n rows xi live in its registers while the loop over the
 //                    channels runs (mma.sync m8n8k4 f64).  A thread's operands of a row are 16 CONSECUTIVE
 //                    bytes of channels, which only permutes the order of the contraction.  After the last
-//                    chunk: A^T along xi in registers, the n columns meet in shared memory one output row
-//                    at a time, A^T along nu, y.
+//                    chunk: A^T along xi in registers, the n columns meet in shared memory (kZRows output
+//                    rows at a time), A^T along nu, y.
 //   transform warps  V of the next chunk from the patches of x; a thread owns one (tile, channel), reads
 //                    its patch once and produces V row pair by row pair.  With eight warps the row pairs of
 //                    a patch are shared out to two threads.
@@ -527,9 +527,11 @@ int go(const nova_plan* plan, const Geom& g, const void* x, const void* U, void*
 
 // Filters per block and channel split.  Wide blocks transform x less often, narrow ones and clusters reach
 // more SMs; the estimate is rounds of blocks x (chunks x time per chunk + time for the end of a block), in
-// units of 10 ns fitted to B200 timings of 12 layers.  Clusters of 4: 33 fit the chip at once; of 8, fewer than 16
+// units of 10 ns fitted to B200 timings of 12 layers, with the end of a block by single rows.  With the present one the
+// choice is still within 2 % of the best of all in 90 of 94 random layers, 4 % in 92 (the others: F(2,3) 2 x 12 x 28, 184 -> 248 34.7 / 31.9
+// us, F(6,3), asymmetric, 5 x 15 x 28, 24 -> 80 22.0 / 17.5).  Clusters of 4: 33 fit the chip at once; of 8, fewer than 16
 // do, and they lost on every layer tried (14 x 14, 256 -> 256, F(4,3): 13.5 us with 4, 27.7 us with 8).
-// Measured against the three kernels before, whole call: F(4,3) 8 images 56 x 56, 64 -> 64: 82.5 -> 34.2 us;
+// Measured against the three kernels before, whole call: F(4,3) 8 images 56 x 56, 64 -> 64: 82.5 -> 33.9 us;
 // F(2,3) 16 x 16, 8 -> 8: 10.6 -> 3.4; F(6,3) 112 x 112, 64 -> 64: 49.3 -> 24.6; F(4,3) 14 x 14, 512 -> 512:
 // 113 -> 29.5; F(6,3), asymmetric set, 2 x 28 x 28, 128 -> 128: 33.6 -> 31.8.
 void choose_blocks(int n, const Geom& g, int sms, int* nb_out, int* split_out) {

@@ -71,8 +71,8 @@ struct PoCfg {
   static_assert(total(kMaxF, 2) <= kMaxTotal && total(kMaxF, 4) <= kMaxTotal && total(16, 2) <= kMaxTotal && total(16, 4) <= kMaxTotal &&
                 total(32, 2) <= kMaxTotal && total(32, 4) <= kMaxTotal && stages(kMaxF, 2) >= 2, "shared memory of one CTA");
   // Exchange buffers: four for few channels, where the ring of operands can spare a stage.  With two, a row group waits for the
-  // buffer that it filled a slice ago to be read in all CTAs.  Whole call, two / four: F(2,3) 32 x 56 x 56, 128 -> 128 75.6 / 70.7 us,
-  // 32 x 112 x 112, 64 -> 64 136 / 133; F(4,3) 32 x 112 x 112, 64 -> 128 152.8 / 147.7, 8 x 112 x 112, 64 -> 256 75.3 / 70.9.  With more channels
+  // buffer that it filled a slice ago to be read in all CTAs.  Whole call, two / four: F(2,3) 32 x 56 x 56, 128 -> 128 75.1 / 69.8 us,
+  // 32 x 112 x 112, 64 -> 64 135.7 / 131.9; F(4,3) 32 x 112 x 112, 64 -> 128 152.7 / 148.0, 64 -> 64 93.3 / 92.3, 8 x 112 x 112, 64 -> 256 73.6 / 69.7.  With more channels
   // the stage is worth more: F(2,3) 8 x 56 x 56, 256 -> 64 29.4 / 30.2, F(4,3) 32 x 112 x 112, 128 -> 128 202 / 235, F(2,5) 8 x 56 x 56, 128 -> 256
   // 66.1 / 69.9; with 8 points 32 x 56 x 56, 64 -> 128, F(4,5) 62.4 / 64.9.
   static constexpr int bufs(int F, int num_ks) { return N <= 6 && num_ks <= (N == 4 ? 2 : 1) && stages(F, 4) >= 2 ? 4 : 2; }
